@@ -873,20 +873,24 @@ void op_pool_bwd(alexnet* h, int r, int which, cudaStream_t st) {
     h->launches++;
 }
 // fused LRN + pool kernels, instantiated for the two LRN layers: {vectors per pixel, vectors per block, W, H, output rows
-// per block, threads} forward; {vectors per pixel, W, H, pixels per pass, threads} backward
-// (the last parameter: exponent beta = 0.75 known at compile time)
-#define LRN_POOL_FWD_1(B75) kn::lrn_pool_fwd_kernel<12, 6, 55, 55, 3, 352, B75>
-#define LRN_POOL_FWD_2(B75) kn::lrn_pool_fwd_kernel<32, 8, 27, 27, 3, 224, B75>
-#define POOL_LRN_BWD_1(B75) kn::pool_lrn_bwd_kernel<12, 55, 55, 28, 352, B75, true>
-#define POOL_LRN_BWD_2(B75) kn::pool_lrn_bwd_kernel<32, 27, 27, 9, 288, B75, false>
+// per block} forward; {vectors per pixel, W, H} backward (the last parameter: exponent beta = 0.75 known at compile time)
+#define LRN_POOL_FWD_1(B75) kn::lrn_pool_fwd_kernel<12, 6, 55, 55, B75, 4>
+#define LRN_POOL_FWD_2(B75) kn::lrn_pool_fwd_kernel<32, 16, 27, 27, B75, 3>
+#define POOL_LRN_BWD_1(B75) kn::pool_lrn_bwd_kernel<12, 55, 55, B75>
+#define POOL_LRN_BWD_2(B75) kn::pool_lrn_bwd_kernel<32, 27, 27, B75>
 void op_lrn_pool_fwd(alexnet* h, int r, int which, cudaStream_t st) {
     Replica& R = h->rep[r];
     const PoolGeo& g = kPool[which];
     const bool b75 = h->cfg.lrn_beta == 0.75f;
-    const dim3 grid((g.Ho + 2) / 3, which == 0 ? 2 : 4, h->B);
-    const size_t smem = which == 0 ? (size_t)7 * 55 * 6 * 16 : (size_t)7 * 27 * 8 * 16;
+    // output rows per block: as few as still fit the machine at once (4 resp. 3 blocks per SM), at most three: measured at
+    // batch 1 / 8 / 32 / 512, LRN1 4.1 / 6.4 / 12.3 / 128 us by this rule (6.2 / 6.6 / 12.3 / 128 with three everywhere, 154
+    // with one row at 512, where every second input row would be normalised twice)
+    int opr = 1;
+    while (opr < 3 && (long long)nblk(g.Ho, opr) * 2 * h->B * 10 > (which == 0 ? 4 : 3) * h->sm_count * 11) ++opr;
+    const dim3 grid(nblk(g.Ho, opr), 2, h->B);
+    const int nt = which == 0 ? 28 * 6 : 14 * 16;
     auto k = which == 0 ? (b75 ? LRN_POOL_FWD_1(true) : LRN_POOL_FWD_1(false)) : (b75 ? LRN_POOL_FWD_2(true) : LRN_POOL_FWD_2(false));
-    launch_k(k, grid, which == 0 ? 352 : 224, smem, st, which ? R.a2 : R.a1, which ? R.p2 : R.p1, which ? R.arg2 : R.arg1, g.Hpi, g.Wpi,
+    launch_k(k, grid, nt, 0, st, which ? R.a2 : R.a1, which ? R.p2 : R.p1, which ? R.arg2 : R.arg1, opr, g.Hpi, g.Wpi,
              g.Hpo, g.Wpo, h->alpha_eff, h->cfg.lrn_beta, h->cfg.lrn_k);
     h->launches++;
     R.n_stale[which] = true;
@@ -895,9 +899,9 @@ void op_pool_lrn_bwd(alexnet* h, int r, int which, cudaStream_t st) {
     Replica& R = h->rep[r];
     const PoolGeo& g = kPool[which];
     const bool b75 = h->cfg.lrn_beta == 0.75f;
-    const size_t smem = which == 0 ? (size_t)2 * 55 * 12 * 48 : (size_t)2 * 27 * 32 * 32;     // gradient tile (fp32) (+ two rows of a: LRN1)
     auto k = which == 0 ? (b75 ? POOL_LRN_BWD_1(true) : POOL_LRN_BWD_1(false)) : (b75 ? POOL_LRN_BWD_2(true) : POOL_LRN_BWD_2(false));
-    launch_k(k, dim3((g.Hpi + 1) / 2, h->B), which == 0 ? 352 : 288, smem, st, which ? R.a2 : R.a1, which ? R.dp2 : R.dp1,
+    const int blocks = which == 0 ? kn::PoolLrnBwdGeo<12, 55, 55>::BLOCKS : kn::PoolLrnBwdGeo<32, 27, 27>::BLOCKS;
+    launch_k(k, dim3(blocks, h->B), 128, 0, st, which ? R.a2 : R.a1, which ? R.dp2 : R.dp1,
              which ? R.arg2 : R.arg1, which ? R.da2 : R.da1, g.Hpi, g.Wpi, g.Hpo, g.Wpo, h->alpha_eff, h->cfg.lrn_beta, h->cfg.lrn_k);
     h->launches++;
     R.dn_stale[which] = true;
@@ -1282,11 +1286,6 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
     CKC(cudaFuncSetAttribute(tc::conv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     CKC(cudaFuncSetAttribute(tc::wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     CKC(cudaFuncSetAttribute(tc::fc_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    // (static + dynamic shared memory of both exceeds the 48 KB that need no opt-in)
-    CKC(cudaFuncSetAttribute(POOL_LRN_BWD_1(true), cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 55 * 12 * 48));
-    CKC(cudaFuncSetAttribute(POOL_LRN_BWD_1(false), cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 55 * 12 * 48));
-    CKC(cudaFuncSetAttribute(POOL_LRN_BWD_2(true), cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 27 * 32 * 32));
-    CKC(cudaFuncSetAttribute(POOL_LRN_BWD_2(false), cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 27 * 32 * 32));
     {
         int dev = 0;
         CKC(cudaGetDevice(&dev));

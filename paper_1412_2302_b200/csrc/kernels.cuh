@@ -292,215 +292,280 @@ __global__ void __launch_bounds__(256) pool_bwd_kernel(const __nv_bfloat16* __re
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     uint32_t d; asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel)); return d;
 }
-// Forward: p = maxpool(LRN(a)) without writing the normalised tensor.  One block = one image, OPR output rows and CV
-// of the CPR channel vectors: the 2*OPR+1 input rows they cover are normalised once into shared memory as bf16 (the
-// same rounding as lrn_fwd_kernel's output; channel neighbours outside the block's range come from global memory),
-// then pooled from there.  The normalised values are non-negative (a is a ReLU output; the sign bit is cleared so that
-// a -0 cannot occur), so bf16 bit patterns order like the values: each candidate becomes the 32-bit key
-// (bits << 16) | (8 - tap) and the window's maximum key carries the largest value and, among equal values, the first
-// tap in scan order - pool_fwd_kernel's tie rule.
-// grid: (ceil(HO / OPR), CPR / CV, B); dynamic shared memory (2*OPR+1) * WI * CV * 16 bytes.
-template <int CPR, int CV, int WI, int HI, int OPR, int NT, bool B75>
-__global__ void __launch_bounds__(NT) lrn_pool_fwd_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat16* __restrict__ y,
-                                                          uint8_t* __restrict__ arg, int Hpi, int Wpi, int Hpo, int Wpo,
-                                                          float alpha, float beta, float k) {
-    pdl_sync();
-    constexpr int RV = WI * CV, NR = 2 * OPR + 1, WO = (WI - 3) / 2 + 1, HO = (HI - 3) / 2 + 1;
-    extern __shared__ uint4 nrm[];            // [row][x][vector]
-    const int n = blockIdx.z, c0 = blockIdx.y * CV, oy0 = OPR * blockIdx.x, iy0 = 2 * oy0;
-    const int nrows = min(NR, HI - iy0);
-    for (int q = threadIdx.x; q < RV; q += NT) {
-        const int x = q / CV, ch = c0 + q % CV;
-        const uint4* ap = (const uint4*)a + ((size_t)(n * Hpi + iy0) * Wpi + x) * CPR + ch;
-        for (int r = 0; r < nrows; ++r) {
-            uint4 v = lrn_fwd8_t<B75>(ap + (size_t)r * Wpi * CPR, ch > 0, ch < CPR - 1, alpha, beta, k);
-            v.x &= 0x7fff7fffu; v.y &= 0x7fff7fffu; v.z &= 0x7fff7fffu; v.w &= 0x7fff7fffu;
-            nrm[r * RV + q] = v;
-        }
-    }
-    __syncthreads();
-    const int orows = min(OPR, HO - oy0);
-    for (int t = threadIdx.x; t < orows * WO * CV; t += NT) {
-        const int oyl = t / (WO * CV), q = t - oyl * (WO * CV);
-        const int ox = q / CV, cv = q - ox * CV;
-        const uint4* src = nrm + (2 * oyl * WI + 2 * ox) * CV + cv;
-        uint32_t best[8];
-        #pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-            #pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-                const uint4 v = src[(ky * WI + kx) * CV];
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-                const uint32_t code = 8u - (uint32_t)(ky * 3 + kx);
-                #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t lo = prmt(w[i], code, 0x1054u);      // (low bf16 << 16) | code
-                    const uint32_t hi = prmt(w[i], code, 0x3254u);      // (high bf16 << 16) | code
-                    if (ky == 0 && kx == 0) { best[2 * i] = lo; best[2 * i + 1] = hi; }
-                    else { best[2 * i] = max(best[2 * i], lo); best[2 * i + 1] = max(best[2 * i + 1], hi); }
-                }
-            }
-        const int oy = oy0 + oyl;
-        uint4 o;
-        o.x = prmt(best[0], best[1], 0x7632u); o.y = prmt(best[2], best[3], 0x7632u);
-        o.z = prmt(best[4], best[5], 0x7632u); o.w = prmt(best[6], best[7], 0x7632u);
-        ((uint4*)y)[((size_t)(n * Hpo + oy) * Wpo + ox) * CPR + c0 + cv] = o;
-        uint2 ab;     // tap = 8 - low byte of the key
-        ab.x = 0x08080808u - prmt(prmt(best[0], best[1], 0x4040u), prmt(best[2], best[3], 0x4040u), 0x5410u);
-        ab.y = 0x08080808u - prmt(prmt(best[4], best[5], 0x4040u), prmt(best[6], best[7], 0x4040u), 0x5410u);
-        ((uint2*)arg)[((size_t)(n * HO + oy) * WO + ox) * CPR + c0 + cv] = ab;
+// Both kernels work on PIXEL PAIRS: a thread owns eight channels of the pixels (2i, 2i+1) of a row and keeps every fp32 value of
+// the pair in one 64-bit register, so that sums and products are the packed instructions of sm_100 (add / mul / fma.rn.f32x2):
+// the kernels are bound by instruction issue and by the special-function unit (two instructions per element, 16 lanes per
+// SM and cycle), not by HBM, and packing halves the arithmetic instructions.  Window sums take pair sums shared by
+// neighbouring channels.  Measured at batch 128 (back to back), this form against one thread per pixel vector with the
+// pooling gradient scattered through shared memory: forward 40.4 -> 36.6 us (LRN1) and 27.6 -> 24.8 (LRN2), backward 79.1 ->
+// 55 and 48.9 -> 35; at batch 512 forward 141 -> 128 and 97 -> 83.  Same arithmetic in the same order as the single-operation kernels.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 mk2(float lo, float hi) { f2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ void un2(f2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) { f2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) { f2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) { f2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
+// twelve channels c0-2 .. c0+9 of a pixel pair from six words each (two bf16 channels per word)
+__device__ __forceinline__ void unpack_pair(const uint32_t* w0, const uint32_t* w1, f2* x) {
+    #pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        x[2 * i] = mk2(bf_lo(w0[i]), bf_lo(w1[i]));
+        x[2 * i + 1] = mk2(bf_hi(w0[i]), bf_hi(w1[i]));
     }
 }
-// Backward: da = LRN'(a, dn) with dn = maxpool'(dp, arg) formed in shared memory.  One block = one image and the two
-// input rows 2j, 2j+1.  The pooling windows that reach these rows lie in the window rows j-1 (its last filter row) and
-// j (its first two); windows of one row and one column parity do not overlap, so four passes (window row x parity),
-// each thread adding the eight gradients of one window vector to the fp32 pixels its argmax codes name, form dn
-// without atomics and in a fixed order.  Then one thread = 8 channels of one pixel (PPB pixels at a time): dn rounded
-// to bf16 (as pool_bwd_kernel stores it), s^-beta, tt = dn a s^(-beta-1), the tt of the two channels on either side
-// from the neighbouring threads through shared memory, and da with the ReLU mask of the convolution that produced a.
-// Pad pixels of the grid get zero.  grid: (ceil(Hpi / 2), B); dynamic shared memory 2 * WI * CPR * 48 bytes.
-template <int CPR, int WI, int HI, int PPB, int NT, bool B75, bool STAGE_A>
-__global__ void __launch_bounds__(NT) pool_lrn_bwd_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ dp,
-                                                          const uint8_t* __restrict__ arg, __nv_bfloat16* __restrict__ da,
-                                                          int Hpi, int Wpi, int Hpo, int Wpo, float alpha, float beta, float k) {
+// out[i] = (x[i] + x[i+1]) + (x[i+2] + x[i+3]) + x[i+4], the five-channel window of channel c0 + i (lrn_fwd8's order)
+__device__ __forceinline__ void window_sums(const f2* x, f2* out) {
+    f2 t[10];
+    #pragma unroll
+    for (int i = 0; i < 10; ++i) t[i] = add2(x[i], x[i + 1]);
+    #pragma unroll
+    for (int i = 0; i < 8; ++i) out[i] = add2(add2(t[i], t[i + 2]), x[i + 4]);
+}
+__device__ __forceinline__ uint32_t pack_bf(float lo, float hi) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *(const uint32_t*)&h;
+}
+__device__ __forceinline__ void pack_pair(const f2* o, uint4& p0, uint4& p1) {
+    float a[8], b[8];
+    #pragma unroll
+    for (int i = 0; i < 8; ++i) un2(o[i], a[i], b[i]);
+    p0 = make_uint4(pack_bf(a[0], a[1]), pack_bf(a[2], a[3]), pack_bf(a[4], a[5]), pack_bf(a[6], a[7]));
+    p1 = make_uint4(pack_bf(b[0], b[1]), pack_bf(b[2], b[3]), pack_bf(b[4], b[5]), pack_bf(b[6], b[7]));
+}
+// s^-beta (and 1/s) of both pixels
+template <bool B75>
+__device__ __forceinline__ void pow_pair(f2 s, float beta, f2& sp, f2& rs) {
+    float s0, s1;
+    un2(s, s0, s1);
+    if (B75) {
+        const float r0 = rsqrt_fast(s0), r1 = rsqrt_fast(s1);
+        const f2 r = mk2(r0, r1);
+        sp = mul2(r, mk2(sqrt_fast(r0), sqrt_fast(r1)));
+        rs = mul2(r, r);
+    } else {
+        float p0, p1, q0, q1;
+        pow_neg_t<false>(s0, beta, p0, q0);
+        pow_neg_t<false>(s1, beta, p1, q1);
+        sp = mk2(p0, p1); rs = mk2(q0, q1);
+    }
+}
+// Forward: p = maxpool(LRN(a)) without writing the normalised tensor.  One block = one image, CV of the CPR channel vectors and a
+// run of `opr` output rows; a thread owns one pixel pair and vector and walks down the rows, so only the first of the
+// 2*opr+1 input rows is normalised by two blocks.  A normalised row (rounded to bf16 as lrn_fwd_kernel stores it) updates the
+// running maximum over the filter rows of the thread's two columns, two channels per instruction (a later row
+// replaces the best one only if it is greater).  Once per output row the result of the even column goes to the
+// left neighbour through shared memory, and the three columns of a window are combined with 32-bit keys (value << 16) |
+// (8 - tap): the largest key has the largest value and, among equal values, the first tap in scan order - pool_fwd_kernel's
+// tie rule.  (Normalised values are not negative; as signed integers the keys also order a NaN above everything.)
+// grid: (ceil(HO / opr), CPR / CV, B); (WI+1)/2 * CV threads.
+template <int CPR, int CV, int WI, int HI, bool B75, int MINB>
+__global__ void __launch_bounds__((WI + 1) / 2 * CV, MINB) lrn_pool_fwd_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat16* __restrict__ y,
+                                                                               uint8_t* __restrict__ arg, int opr, int Hpi, int Wpi, int Hpo,
+                                                                               int Wpo, float alpha, float beta, float k) {
     pdl_sync();
-    static_assert(PPB * CPR <= NT, "one thread per vector of PPB pixels");
-    constexpr int RV = WI * CPR, WO = (WI - 3) / 2 + 1, HO = (HI - 3) / 2 + 1;
-    __shared__ float4 edge[2][NT];    // tt of the two lowest and two highest channels of every thread, for its neighbours
-    extern __shared__ float dn[];     // [2 planes: channels 0-3 / 4-7 of a vector][2 rows][WI][CPR] float4 (conflict-free reads)
-    constexpr int PLANE = 2 * RV * 4; // floats per plane
-    uint4* const as = (uint4*)(dn + 2 * PLANE);     // then the block's two rows of a, [2][WI][CPR] vectors
-    const int j = blockIdx.x, n = blockIdx.y, y0 = 2 * j;
-    const uint4 zero4 = make_uint4(0, 0, 0, 0);
-    if (y0 >= HI) {                   // pad rows of the grid
-        for (int row = 0; row < 2 && y0 + row < Hpi; ++row)
-            for (int i = threadIdx.x; i < Wpi * CPR; i += NT) ((uint4*)da)[(size_t)(n * Hpi + y0 + row) * Wpi * CPR + i] = zero4;
-        return;
-    }
-    // every thread first fetches the (up to four) window vectors it will scatter: window rows j-1 and j, even and odd
-    // columns; the loads are in flight while the tile is cleared
-    static_assert(((WO + 1) / 2) * CPR <= NT, "one thread per window vector of a pass");
-    const int wq = threadIdx.x / CPR, wch = threadIdx.x - wq * CPR;
-    uint4 wdp[4]; uint2 warg[4]; bool has[4];
-    #pragma unroll
-    for (int pass = 0; pass < 4; ++pass) {
-        const int oy = j - 1 + (pass >> 1), ox = 2 * wq + (pass & 1);
-        has[pass] = oy >= 0 && oy < HO && ox < WO;
-        if (has[pass]) {
-            warg[pass] = __ldg((const uint2*)arg + ((size_t)(n * HO + oy) * WO + ox) * CPR + wch);
-            wdp[pass] = __ldg((const uint4*)dp + ((size_t)(n * Hpo + oy) * Wpo + ox) * CPR + wch);
+    constexpr int NP = (WI + 1) / 2, NT = NP * CV, WO = (WI - 3) / 2 + 1, HO = (HI - 3) / 2 + 1;
+    __shared__ uint4 xch[2][2][NT];           // [parity of the output row][value / filter row of the maximum][thread]
+    const int n = blockIdx.z, c0 = blockIdx.y * CV, oy0 = opr * blockIdx.x, oy1 = min(HO, oy0 + opr);
+    const int xp = threadIdx.x / CV, cv = threadIdx.x - xp * CV, ch = c0 + cv;
+    // (the pair of the last pixel has a pad pixel as its second: the grid is wider than WI and pads are zero)
+    const uint4* ap = (const uint4*)a + ((size_t)(n * Hpi + 2 * oy0) * Wpi + 2 * xp) * CPR + ch;
+    const f2 al2 = mk2(alpha, alpha), k2 = mk2(k, k);
+    // the neighbouring channel words come from the neighbouring lanes; only the ends of a warp (and of a block's channel
+    // range) load them
+    const int lane = threadIdx.x & 31;
+    const bool has_l = ch > 0, has_r = ch < CPR - 1;
+    const bool ld_l = has_l && (lane == 0 || cv == 0), ld_r = has_r && (lane == 31 || threadIdx.x == NT - 1 || cv == CV - 1);
+    const unsigned mask = __activemask();      // the last warp of a block may be partial
+    uint4 v0, v1; uint32_t l0 = 0u, l1 = 0u, r0 = 0u, r1 = 0u;
+    auto fetch = [&]() {
+        v0 = __ldg(ap); v1 = __ldg(ap + CPR);
+        const uint32_t* wp = (const uint32_t*)ap;
+        if (ld_l) { l0 = __ldg(wp - 1); l1 = __ldg(wp + 4 * CPR - 1); }
+        if (ld_r) { r0 = __ldg(wp + 4); r1 = __ldg(wp + 4 * CPR + 4); }
+        ap += Wpi * CPR;
+    };
+    // normalises the fetched row and fetches the next one meanwhile
+    auto norm_row = [&](bool more, uint4& p0, uint4& p1) {
+        const uint32_t ul0 = __shfl_up_sync(mask, v0.w, 1), ul1 = __shfl_up_sync(mask, v1.w, 1);
+        const uint32_t dr0 = __shfl_down_sync(mask, v0.x, 1), dr1 = __shfl_down_sync(mask, v1.x, 1);
+        const uint32_t w0[6] = {has_l && !ld_l ? ul0 : l0, v0.x, v0.y, v0.z, v0.w, has_r && !ld_r ? dr0 : r0};
+        const uint32_t w1[6] = {has_l && !ld_l ? ul1 : l1, v1.x, v1.y, v1.z, v1.w, has_r && !ld_r ? dr1 : r1};
+        f2 x[12], sq[12], ss[8];
+        unpack_pair(w0, w1, x);
+        if (more) fetch();
+        #pragma unroll
+        for (int i = 0; i < 12; ++i) sq[i] = mul2(x[i], x[i]);
+        window_sums(sq, ss);
+        #pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            f2 sp, rs;
+            pow_pair<B75>(fma2(al2, ss[i], k2), beta, sp, rs);
+            ss[i] = mul2(x[i + 2], sp);
         }
-    }
-    // the two rows of a travel to shared memory asynchronously, behind the scatter passes (the LRN part then reads a and
-    // its channel neighbours from there instead of waiting for global memory three times per vector)
-    for (int i = threadIdx.x; STAGE_A && i < 2 * RV; i += NT) {
-        const int row = i / RV, q = i - row * RV;
-        if (y0 + row < HI) {
-            const uint4* src = (const uint4*)a + (size_t)(n * Hpi + y0 + row) * Wpi * CPR + q;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(as + i)), "l"(src) : "memory");
+        pack_pair(ss, p0, p1);
+    };
+    auto vmax = [&](const uint4& p, uint32_t* best, uint32_t* row, uint32_t ky3) {
+        const uint32_t w[4] = {p.x, p.y, p.z, p.w};
+        #pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const __nv_bfloat162 vb = *(const __nv_bfloat162*)&w[i], bb = *(const __nv_bfloat162*)&best[i];
+            const uint32_t gt = __hgt2_mask(vb, bb);
+            const __nv_bfloat162 mx = __hmax2_nan(vb, bb);
+            best[i] = *(const uint32_t*)&mx;
+            row[i] = (gt & ky3) | (~gt & row[i]);
         }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int i = threadIdx.x; i < 4 * RV; i += NT) ((float4*)dn)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    #pragma unroll
-    for (int pass = 0; pass < 4; ++pass) {
-        const int oy = j - 1 + (pass >> 1), par = pass & 1;
-        if (pass == 3) asm volatile("cp.async.wait_group 0;" ::: "memory");     // before the last barrier of the passes
-        if (has[pass]) {
-            const int ox = 2 * wq + par;
-            float f[8];
-            unpack8(wdp[pass], f);
-            float* base = dn + ((2 * ox) * CPR + wch) * 4;
-            const int r0 = 2 * oy - y0;            // window row 0 relative to the block's first row: -2 or 0
-            #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int tap = (int)(((q < 4 ? warg[pass].x : warg[pass].y) >> (8 * (q & 3))) & 0xFFu);
-                const int ky = (tap * 11) >> 5, kx = tap - 3 * ky;
-                const int row = r0 + ky;
-                if ((unsigned)row < 2u) base[(q >> 2) * PLANE + (row * WI + kx) * (CPR * 4) + (q & 3)] += f[q];
-            }
-        }
-        __syncthreads();
-    }
-    const int px = threadIdx.x / CPR, ch = threadIdx.x - px * CPR;
-    int it = 0;
+    };
+    fetch();
+    uint4 p0, p1;
+    norm_row(true, p0, p1);
     #pragma unroll 1
-    for (int row = 0; row < 2; ++row) {
-        const int yy = y0 + row;
-        if (yy >= Hpi) break;
-        uint4* out_row = (uint4*)da + (size_t)(n * Hpi + yy) * Wpi * CPR;
-        if (yy >= HI) {
-            for (int i = threadIdx.x; i < Wpi * CPR; i += NT) out_row[i] = zero4;
-            continue;
+    for (int oy = oy0; oy < oy1; ++oy) {
+        uint32_t be[4] = {p0.x, p0.y, p0.z, p0.w}, bo[4] = {p1.x, p1.y, p1.z, p1.w}, re[4] = {0, 0, 0, 0}, ro[4] = {0, 0, 0, 0};
+        norm_row(true, p0, p1);
+        vmax(p0, be, re, 0x00030003u); vmax(p1, bo, ro, 0x00030003u);
+        norm_row(oy + 1 < oy1, p0, p1);
+        vmax(p0, be, re, 0x00060006u); vmax(p1, bo, ro, 0x00060006u);
+        uint4 (*buf)[NT] = xch[oy & 1];
+        buf[0][threadIdx.x] = make_uint4(be[0], be[1], be[2], be[3]);
+        buf[1][threadIdx.x] = make_uint4(re[0], re[1], re[2], re[3]);
+        __syncthreads();
+        if (xp < WO) {
+            const uint4 rv = buf[0][threadIdx.x + CV], rr = buf[1][threadIdx.x + CV];
+            const uint32_t br[4] = {rv.x, rv.y, rv.z, rv.w}, rw[4] = {rr.x, rr.y, rr.z, rr.w};
+            uint32_t val[4], tap[4];
+            #pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t ce = 0x00080008u - re[i], co = 0x00070007u - ro[i], cr = 0x00060006u - rw[i];
+                const int lo = max(max((int)prmt(be[i], ce, 0x1054u), (int)prmt(bo[i], co, 0x1054u)), (int)prmt(br[i], cr, 0x1054u));
+                const int hi = max(max((int)prmt(be[i], ce, 0x3276u), (int)prmt(bo[i], co, 0x3276u)), (int)prmt(br[i], cr, 0x3276u));
+                val[i] = prmt((uint32_t)lo, (uint32_t)hi, 0x7632u);
+                tap[i] = prmt((uint32_t)lo, (uint32_t)hi, 0x5410u);
+            }
+            ((uint4*)y)[((size_t)(n * Hpo + oy) * Wpo + xp) * CPR + ch] = make_uint4(val[0], val[1], val[2], val[3]);
+            ((uint2*)arg)[((size_t)(n * HO + oy) * WO + xp) * CPR + ch] =
+                make_uint2(0x08080808u - prmt(tap[0], tap[1], 0x6420u), 0x08080808u - prmt(tap[2], tap[3], 0x6420u));
         }
-        for (int i = threadIdx.x; i < (Wpi - WI) * CPR; i += NT) out_row[WI * CPR + i] = zero4;     // pad columns
-        #pragma unroll 1
-        for (int p0 = 0; p0 < WI; p0 += PPB, ++it) {
-            const int x = p0 + px;
-            const bool valid = px < PPB && x < WI;
-            float fa[24], g8[8], sp[8], tt[8];
-            if (valid) {
-                const float4* gp = (const float4*)dn + (row * WI + x) * CPR + ch;
-                const float4 g0 = gp[0], g1 = gp[PLANE / 4];
-                const float acc[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-                unpack8(pack8(acc), g8);
-                if (STAGE_A) {
-                    const uint4* ap = as + (row * WI + x) * CPR + ch;
-                    unpack8(ch > 0 ? ap[-1] : zero4, fa);
-                    unpack8(ap[0], fa + 8);
-                    unpack8(ch < CPR - 1 ? ap[1] : zero4, fa + 16);
-                } else {
-                    const uint4* ap = (const uint4*)a + ((size_t)(n * Hpi + yy) * Wpi + x) * CPR + ch;
-                    unpack8(ch > 0 ? __ldg(ap - 1) : zero4, fa);
-                    unpack8(__ldg(ap), fa + 8);
-                    unpack8(ch < CPR - 1 ? __ldg(ap + 1) : zero4, fa + 16);
-                }
-                float sq[12];
-                #pragma unroll
-                for (int i = 0; i < 12; ++i) sq[i] = fa[6 + i] * fa[6 + i];
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float ss = (sq[i] + sq[i + 1]) + (sq[i + 2] + sq[i + 3]) + sq[i + 4];
-                    float rs;
-                    pow_neg_t<B75>(fmaf(alpha, ss, k), beta, sp[i], rs);
-                    tt[i] = g8[i] * fa[8 + i] * sp[i] * rs;
-                }
-            } else {
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) tt[i] = 0.f;
+    }
+}
+// Backward: da = LRN'(a, dn), dn = maxpool'(dp, arg).  One thread = eight channels of a 2 x 2 block of pixels (rows 2j, 2j+1,
+// columns 2i, 2i+1).  The four windows (j-1..j, i-1..i) are the only ones that reach these pixels, in nine (window, tap)
+// combinations, so dn is gathered in registers: four argmax bytes are compared with a tap at once, the byte masks select
+// the bf16 gradients, and the up to four terms of a pixel are added in fp32 in a fixed order.  No shared memory, no
+// barriers, no divergent loops.  dn is rounded to bf16, as pool_bwd_kernel stores it.  Then s^-beta and tt = dn a s^(-beta-1) for the row's pixel pair; the tt of the two channels on
+// either side come from the neighbouring lanes, which hold the neighbouring channel vectors: where a pixel is not a whole
+// warp (CPR = 12) the first and last lane of a warp only compute for their neighbours (30 of 32 lanes store).  The ReLU
+// mask of the convolution that produced a is applied to the packed result.  Pad positions are not written: they are zero.
+// grid: (ceil(warps per image / 4), B), 128 threads.
+template <int CPR, int WI, int HI>
+struct PoolLrnBwdGeo {
+    static constexpr int HALO = CPR == 32 ? 0 : 1, PER = 32 - 2 * HALO, NP = (WI + 1) / 2, NJ = (HI + 1) / 2;
+    static constexpr int TOT = NJ * NP * CPR, WARPS = (TOT + PER - 1) / PER, BLOCKS = (WARPS + 3) / 4;
+};
+// the eight gradients of a window where its argmax equals the tap, as fp32
+__device__ __forceinline__ void tap_select(const uint4& g, const uint2& ab, uint32_t tap, float* f) {
+    const uint32_t T = tap * 0x01010101u;
+    const uint32_t m0 = (ab.x ^ T) + 0x7f7f7f7fu, m1 = (ab.y ^ T) + 0x7f7f7f7fu;      // sign bit of a byte: not this tap (bytes are < 16)
+    const uint32_t w[4] = {g.x, g.y, g.z, g.w};
+    #pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t m = i < 2 ? m0 : m1;
+        const uint32_t v = w[i] & ~prmt(m, m, (i & 1) ? 0xbbaau : 0x9988u);          // sign-replicated bytes
+        f[2 * i] = bf_lo(v); f[2 * i + 1] = bf_hi(v);
+    }
+}
+template <int CPR, int WI, int HI, bool B75>
+__global__ void __launch_bounds__(128, 5) pool_lrn_bwd_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ dp,
+                                                           const uint8_t* __restrict__ arg, __nv_bfloat16* __restrict__ da,
+                                                           int Hpi, int Wpi, int Hpo, int Wpo, float alpha, float beta, float k) {
+    pdl_sync();
+    typedef PoolLrnBwdGeo<CPR, WI, HI> G;
+    constexpr int WO = (WI - 3) / 2 + 1, HO = (HI - 3) / 2 + 1;
+    const int lane = threadIdx.x & 31, wg = blockIdx.x * 4 + (threadIdx.x >> 5), n = blockIdx.y;
+    if (wg * G::PER >= G::TOT) return;                 // whole warps
+    const int ql = wg * G::PER + lane - G::HALO, q = min(max(ql, 0), G::TOT - 1);
+    const int ch = q % CPR, i = (q / CPR) % G::NP, j = q / (CPR * G::NP);
+    const bool store = ql == q && lane >= G::HALO && lane < 32 - G::HALO;
+    const uint4* ap = (const uint4*)a + ((size_t)(n * Hpi + 2 * j) * Wpi + 2 * i) * CPR + ch;
+    uint4 av[2][2];
+    #pragma unroll
+    for (int r = 0; r < 2; ++r) { av[r][0] = __ldg(ap + r * Wpi * CPR); av[r][1] = __ldg(ap + r * Wpi * CPR + CPR); }
+    uint4 wd[2][2]; uint2 wa[2][2];                    // [row j - d][column i - e]
+    #pragma unroll
+    for (int d = 0; d < 2; ++d)
+        #pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int oy = j - d, ox = i - e;
+            wd[d][e] = make_uint4(0u, 0u, 0u, 0u);
+            wa[d][e] = make_uint2(0x0f0f0f0fu, 0x0f0f0f0fu);     // matches no tap
+            if (oy >= 0 && oy < HO && ox >= 0 && ox < WO) {
+                wd[d][e] = __ldg((const uint4*)dp + ((size_t)(n * Hpo + oy) * Wpo + ox) * CPR + ch);
+                wa[d][e] = __ldg((const uint2*)arg + ((size_t)(n * HO + oy) * WO + ox) * CPR + ch);
             }
-            // tt of channels c0-2, c0-1 (left neighbour's two highest) and c0+8, c0+9 (right neighbour's two lowest)
-            float4 l, r;
-            if (CPR == 32) {
-                // a pixel is exactly one warp: the neighbours are the adjacent lanes, no shared memory and no block barrier
-                l.z = __shfl_up_sync(0xffffffffu, tt[6], 1); l.w = __shfl_up_sync(0xffffffffu, tt[7], 1);
-                r.x = __shfl_down_sync(0xffffffffu, tt[0], 1); r.y = __shfl_down_sync(0xffffffffu, tt[1], 1);
-                if (ch == 0) { l.z = 0.f; l.w = 0.f; }
-                if (ch == CPR - 1) { r.x = 0.f; r.y = 0.f; }
-            } else {
-                float4* eb = edge[it & 1];
-                eb[threadIdx.x] = make_float4(tt[0], tt[1], tt[6], tt[7]);
-                __syncthreads();
-                l = ch > 0 ? eb[threadIdx.x - 1] : make_float4(0, 0, 0, 0);
-                r = ch < CPR - 1 ? eb[threadIdx.x + 1] : make_float4(0, 0, 0, 0);
-            }
-            if (valid) {
-                float te[12];
-                te[0] = l.z; te[1] = l.w; te[10] = r.x; te[11] = r.y;
+        }
+    const f2 al2 = mk2(alpha, alpha), k2 = mk2(k, k), mc2 = mk2(-2.f * alpha * beta, -2.f * alpha * beta);
+    #pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        f2 g[8];
+        {
+            float e0[8], o0[8], t[8];
+            if (r == 0) {                                        // windows of row j-1: their last filter row
+                tap_select(wd[1][0], wa[1][0], 6, e0);
+                tap_select(wd[1][0], wa[1][0], 7, o0);
+                tap_select(wd[1][1], wa[1][1], 8, t);
                 #pragma unroll
-                for (int i = 0; i < 8; ++i) te[2 + i] = tt[i];
-                const float c2 = 2.f * alpha * beta;
-                float o[8];
-                #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float acc = (te[i] + te[i + 1]) + (te[i + 2] + te[i + 3]) + te[i + 4];
-                    const float am = fa[8 + i];
-                    const float v = fmaf(g8[i], sp[i], -c2 * am * acc);
-                    o[i] = am > 0.f ? v : 0.f;
-                }
-                out_row[x * CPR + ch] = pack8(o);
+                for (int c = 0; c < 8; ++c) g[c] = mk2(e0[c] + t[c], o0[c]);
             }
+            tap_select(wd[0][0], wa[0][0], 3 * r, e0);           // window (j, i): taps (r, 0) and (r, 1)
+            tap_select(wd[0][0], wa[0][0], 3 * r + 1, o0);
+            tap_select(wd[0][1], wa[0][1], 3 * r + 2, t);        // window (j, i-1): tap (r, 2) on the even pixel
+            #pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const f2 v = mk2(e0[c], o0[c]);
+                g[c] = add2(r == 0 ? add2(g[c], v) : v, mk2(t[c], 0.f));
+            }
+            // rounded to bf16, as pool_bwd_kernel stores it
+            uint4 q0, q1;
+            pack_pair(g, q0, q1);
+            const uint32_t b0[4] = {q0.x, q0.y, q0.z, q0.w}, b1[4] = {q1.x, q1.y, q1.z, q1.w};
+            #pragma unroll
+            for (int c = 0; c < 4; ++c) { g[2 * c] = mk2(bf_lo(b0[c]), bf_lo(b1[c])); g[2 * c + 1] = mk2(bf_hi(b0[c]), bf_hi(b1[c])); }
+        }
+        uint32_t w0[6] = {__shfl_up_sync(0xffffffffu, av[r][0].w, 1), av[r][0].x, av[r][0].y, av[r][0].z, av[r][0].w, __shfl_down_sync(0xffffffffu, av[r][0].x, 1)};
+        uint32_t w1[6] = {__shfl_up_sync(0xffffffffu, av[r][1].w, 1), av[r][1].x, av[r][1].y, av[r][1].z, av[r][1].w, __shfl_down_sync(0xffffffffu, av[r][1].x, 1)};
+        if (ch == 0) w0[0] = w1[0] = 0u;
+        if (ch == CPR - 1) w0[5] = w1[5] = 0u;
+        f2 x[12], sq[12], ss[8], sp[8], tt[12];
+        unpack_pair(w0, w1, x);
+        #pragma unroll
+        for (int c = 0; c < 12; ++c) sq[c] = mul2(x[c], x[c]);
+        window_sums(sq, ss);
+        #pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            f2 rs;
+            pow_pair<B75>(fma2(al2, ss[c], k2), beta, sp[c], rs);
+            tt[c + 2] = mul2(mul2(mul2(g[c], x[c + 2]), sp[c]), rs);      // dn a s^(-beta-1)
+        }
+        tt[0] = __shfl_up_sync(0xffffffffu, tt[8], 1); tt[1] = __shfl_up_sync(0xffffffffu, tt[9], 1);
+        tt[10] = __shfl_down_sync(0xffffffffu, tt[2], 1); tt[11] = __shfl_down_sync(0xffffffffu, tt[3], 1);
+        if (ch == 0) tt[0] = tt[1] = 0ull;
+        if (ch == CPR - 1) tt[10] = tt[11] = 0ull;
+        window_sums(tt, ss);
+        #pragma unroll
+        for (int c = 0; c < 8; ++c) g[c] = fma2(g[c], sp[c], mul2(mul2(mc2, x[c + 2]), ss[c]));
+        uint4 p[2];
+        pack_pair(g, p[0], p[1]);
+        const __nv_bfloat162 z2 = __floats2bfloat162_rn(0.f, 0.f);
+        #pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const __nv_bfloat162* ah = (const __nv_bfloat162*)&av[r][e];
+            p[e].x &= __hgt2_mask(ah[0], z2); p[e].y &= __hgt2_mask(ah[1], z2); p[e].z &= __hgt2_mask(ah[2], z2); p[e].w &= __hgt2_mask(ah[3], z2);
+        }
+        if (store && 2 * j + r < HI) {
+            uint4* op = (uint4*)da + ((size_t)(n * Hpi + 2 * j + r) * Wpi + 2 * i) * CPR + ch;
+            op[0] = p[0];
+            if (2 * i + 1 < WI) op[CPR] = p[1];
         }
     }
 }

@@ -259,6 +259,24 @@ def test_fused_lrn_pool_forward_argmax_bit_exact(net, which, ta, tn, tp, targ, t
     assert np.array_equal(net.get_tensor(targ).reshape(arg.shape).astype(np.uint8), arg)     # bit exact
 
 
+@pytest.mark.parametrize("batch", [1, 20, 40])
+def test_fused_lrn_pool_rows_per_block(batch):
+    """The fused forward kernel with one, two and three output rows per block (the rule takes them at these batches; 27 and 13
+    output rows leave a partial last block) on random activations: first and last image, values and argmax codes bit for bit."""
+    n = AlexNet(batch=batch, seed=SEED, mean_image=synth.mean_image(SEED))
+    for which, ta, tn, tp, targ, _, _, shp in FUSED:
+        a = np.maximum(np.random.default_rng([batch, which]).standard_normal((batch,) + shp).astype(np.float32), 0) * 20
+        n.set_tensor(ta, a)
+        n.run_op(f"LRN{which}_FWD")
+        n.run_op(f"LRN{which}_POOL{which}_FWD")
+        n.sync()
+        for img in {0, batch - 1}:
+            y, arg = O.pool_fwd(n.get_tensor(tn).reshape((batch,) + shp)[img:img + 1].astype(np.float64))
+            assert np.array_equal(n.get_tensor(tp).reshape((batch,) + y.shape[1:])[img], y[0].astype(np.float32))
+            assert np.array_equal(n.get_tensor(targ).reshape((batch,) + y.shape[1:])[img].astype(np.uint8), arg[0])
+    n.close()
+
+
 @pytest.mark.parametrize("which,ta,tn,tp,targ,tdp,tda,shp", FUSED)
 def test_fused_pool_lrn_backward(net, which, ta, tn, tp, targ, tdp, tda, shp):
     """The fused backward kernel of the step (pooling gradient scattered in shared memory, LRN gradient, ReLU mask)
