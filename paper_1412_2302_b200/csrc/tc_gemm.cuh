@@ -9,7 +9,7 @@
 // 2..5 = epilogue (each reads the 32 TMEM lanes of its quadrant and stores its
 // rows through a swizzled shared-memory tile and TMA).  The producer and issuer
 // loops carry no division or modulo: stage, phase, tap and chunk counters
-// advance incrementally.  This file holds three kernels: gemm_kernel (FC
+// advance incrementally.  The main kernels of this file: gemm_kernel (FC
 // backward), conv_kernel (convolution forward / backward-data, FC forward) and
 // wgrad_kernel (convolution weight gradients).
 // Three operand arrangements:
@@ -21,7 +21,7 @@
 // every A tile is a plain 2-D TMA box; out-of-range rows are zero-filled by TMA.
 // Every wait is bounded: on expiry the CTA raises *status and drains.
 // conv_kernel also runs as CTA pairs (clusters of two, tcgen05.mma.cta_group::2: one instruction of the leader covers 128
-// rows of each CTA), and gemm_kernel can apply the momentum update to the FC weights in its weight-gradient epilogue.
+// rows of each CTA); fc_update_kernel forms the FC weight gradients and applies the momentum update to the weights in place.
 // All kernels are launched with programmatic stream serialization: they let the next launch of the stream start early
 // (griddepcontrol.launch_dependents first thing) and wait for their predecessors (griddepcontrol.wait) after their
 // barriers, tensor memory and descriptors are set up and before they touch global memory.
@@ -55,12 +55,6 @@ constexpr long long kWaitBudgetCycles = 400000000LL;  // ~0.2 s at 2 GHz
 struct GemmParams {
     CUtensorMap tmA, tmB, tmOut;   // tmOut: output as {columns, rows, splits}, box {128 bytes, 32, 1}, when tma_store
     int tma_store;
-    // MODE_MNMN with fuse_update: the tile is an FC weight gradient and the epilogue applies the momentum update to the
-    // weights in place instead of storing the gradient: tmW / tmV = fp32 weights and momentum ({32, 32, 1} boxes, 128-byte
-    // swizzle), tmS = bf16 copy of the weights ({32, 32, 1} boxes, no swizzle); upd_d = lr * weight decay
-    CUtensorMap tmW, tmV, tmS;
-    int fuse_update;
-    float upd_lr, upd_mu, upd_d;
     int mode, epi;
     int m_tiles, n_tiles, groups, taps_grid, splits;  // tile decomposition (m fastest)
     int tiles_total;
@@ -247,6 +241,9 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, uint32_t src
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
                  ::"l"(tm), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
 }
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(tm), "r"(src), "r"(x), "r"(y) : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
@@ -427,11 +424,8 @@ constexpr int kABytes = 128 * 128;  // 128 rows x 64 bf16, or 2 boxes of 64 x 64
 __host__ __device__ inline int b_stage_bytes(int mode, int BN) {
     return mode == MODE_KK ? BN * 128 : ((BN + 63) / 64) * 8192;
 }
-// per epilogue warp of a fused-update kernel: kUpdBufs {w tile, v tile} pairs of 4 KB each and two 2 KB bf16 tiles
-constexpr int kUpdBufs = 5;
-constexpr uint32_t kUpdWarpBytes = kUpdBufs * 8192 + 2 * 2048;
-inline size_t smem_bytes(int mode, int BN, int stages, bool fuse_update = false) {
-    return 1024 + (size_t)stages * (kABytes + b_stage_bytes(mode, BN)) + (fuse_update ? 4 * kUpdWarpBytes : 4 * kEpiStageBytes) + 512;
+inline size_t smem_bytes(int mode, int BN, int stages) {
+    return 1024 + (size_t)stages * (kABytes + b_stage_bytes(mode, BN)) + 4 * kEpiStageBytes + 512;
 }
 
 // position of a CTA in the tile list; tiles are numbered with m fastest, then
@@ -471,8 +465,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     // epilogue staging (4 warps x kEpiStageBytes), then barriers: full[8] @0, empty[8] @64, acc_full[2] @128,
     // acc_empty[2] @144, tmem slot @160, abort flag @168
     const uint32_t epi_stage0 = base + stages * stage_bytes;
-    const uint32_t upd0 = epi_stage0 + (p.fuse_update ? 0u : 4u * kEpiStageBytes);   // fused update: per-warp tiles instead of the staging
-    const uint32_t bar_base = upd0 + (p.fuse_update ? 4u * kUpdWarpBytes : 0u);  // ... + per-warp load barriers [4][kUpdBufs] @176
+    const uint32_t bar_base = epi_stage0 + 4u * kEpiStageBytes;
     uint8_t* gen = smem_raw + (bar_base - raw);
     volatile int* abort_flag = (volatile int*)(gen + 168);
     volatile uint32_t* tmem_slot = (volatile uint32_t*)(gen + 160);
@@ -487,7 +480,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         *abort_flag = 0;
         for (int s = 0; s < stages; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(accf0 + 8u * s, 1); mbar_init(acce0 + 8u * s, 128); }
-        for (int s = 0; s < 4 * kUpdBufs; ++s) mbar_init(bar_base + 176u + 8u * s, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&p.tmA);
         tma_prefetch_desc(&p.tmB);
@@ -591,80 +583,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
         TileCursor tc; tc.init(p);
         int ab = 0; uint32_t aph = 0;
         bool ok = true;
-        if (p.fuse_update) {
-            // FC weight gradient consumed in place: for every 32 x 32 slab of the tile this warp loads the weights and the
-            // momentum by TMA (kUpdBufs - 2 = three slabs ahead of the arithmetic), applies v <- mu v - d w - lr g, w <- w + v to the
-            // accumulator values and stores w, v and the bf16 copy of w by TMA.  A buffer (of kUpdBufs = 5) is reloaded
-            // only after the stores issued from it two slabs earlier have finished reading (wait_group.read 1).
-            const uint32_t ureg = upd0 + (uint32_t)quad * kUpdWarpBytes, ub0 = bar_base + 176u + (uint32_t)quad * (8u * kUpdBufs);
-            TileCursor tp = tc;                      // prefetch cursor
-            int tile = blockIdx.x, c = 0, q = 0;     // tile, column and count of the slab being processed
-            int ptile = blockIdx.x, pc = 0, pq = 0;  // the same for the slab whose loads are issued next
-            auto issue_loads = [&]() {
-                const uint32_t bar = ub0 + 8u * (uint32_t)(pq % kUpdBufs), dst = ureg + (uint32_t)(pq % kUpdBufs) * 8192u;
-                const int x = tp.n_tile * p.BN + pc, y = tp.m_tile * 128 + quad * 32;
-                mbar_expect_tx(bar, 8192u);
-                tma_load_3d(dst, &p.tmW, x, y, 0, bar);
-                tma_load_3d(dst + 4096u, &p.tmV, x, y, 0, bar);
-                ++pq; pc += 32;
-                if (pc == p.BN) { pc = 0; ptile += gridDim.x; tp.next(p); }
-            };
-            if (lane == 0) {
-                #pragma unroll 1
-                for (int i = 0; i < kUpdBufs - 2 && ptile < p.tiles_total; ++i) issue_loads();
-            }
-            __syncwarp();
-            while (tile < p.tiles_total) {
-                if (lane == 0) { bulk_wait_read_1(); if (ptile < p.tiles_total) issue_loads(); }
-                __syncwarp();
-                if (c == 0) {
-                    if (!(ok = mbar_wait(accf0 + 8u * ab, aph, abort_flag))) break;
-                    tc_fence_after();
-                }
-                uint32_t g[32];
-                tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * p.BN + c), g);
-                tmem_ld_wait();
-                if (!(ok = mbar_wait(ub0 + 8u * (uint32_t)(q % kUpdBufs), (uint32_t)((q / kUpdBufs) & 1), abort_flag))) break;
-                const uint32_t buf = ureg + (uint32_t)(q % kUpdBufs) * 8192u, rowp = buf + (uint32_t)lane * 128u;
-                const uint32_t sbuf = ureg + (uint32_t)kUpdBufs * 8192u + (uint32_t)(q & 1) * 2048u;
-                uint32_t sh[16];
-                #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t ch = (uint32_t)((j ^ (lane & 7)) << 4);
-                    float4 w4, v4;
-                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(w4.x), "=f"(w4.y), "=f"(w4.z), "=f"(w4.w) : "r"(rowp + ch));
-                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v4.x), "=f"(v4.y), "=f"(v4.z), "=f"(v4.w) : "r"(rowp + 4096u + ch));
-                    kn::sgd_step(w4.x, v4.x, __uint_as_float(g[4 * j]), p.upd_d, p.upd_lr, p.upd_mu);
-                    kn::sgd_step(w4.y, v4.y, __uint_as_float(g[4 * j + 1]), p.upd_d, p.upd_lr, p.upd_mu);
-                    kn::sgd_step(w4.z, v4.z, __uint_as_float(g[4 * j + 2]), p.upd_d, p.upd_lr, p.upd_mu);
-                    kn::sgd_step(w4.w, v4.w, __uint_as_float(g[4 * j + 3]), p.upd_d, p.upd_lr, p.upd_mu);
-                    st_shared_v4(rowp + ch, __float_as_uint(w4.x), __float_as_uint(w4.y), __float_as_uint(w4.z), __float_as_uint(w4.w));
-                    st_shared_v4(rowp + 4096u + ch, __float_as_uint(v4.x), __float_as_uint(v4.y), __float_as_uint(v4.z), __float_as_uint(v4.w));
-                    __nv_bfloat162 lo = __floats2bfloat162_rn(w4.x, w4.y), hi = __floats2bfloat162_rn(w4.z, w4.w);
-                    sh[2 * j] = *(uint32_t*)&lo; sh[2 * j + 1] = *(uint32_t*)&hi;
-                }
-                #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    st_shared_v4(sbuf + (uint32_t)lane * 64u + 16u * j, sh[4 * j], sh[4 * j + 1], sh[4 * j + 2], sh[4 * j + 3]);
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    const int x = tc.n_tile * p.BN + c, y = tc.m_tile * 128 + quad * 32;
-                    tma_store_3d(&p.tmW, buf, x, y, 0);
-                    tma_store_3d(&p.tmV, buf + 4096u, x, y, 0);
-                    tma_store_3d(&p.tmS, sbuf, x, y, 0);
-                    bulk_commit();
-                }
-                ++q; c += 32;
-                if (c == p.BN) {
-                    tc_fence_before();
-                    mbar_arrive(acce0 + 8u * ab);
-                    if (++ab == 2) { ab = 0; aph ^= 1u; }
-                    c = 0; tile += gridDim.x; tc.next(p);
-                }
-            }
-            if (lane == 0) bulk_wait_all();
-        } else
         for (int tile = blockIdx.x; tile < p.tiles_total && ok; tile += gridDim.x, tc.next(p)) {
             const int m0 = tc.m_tile * 128, n0 = tc.n_tile * p.BN, g = tc.g;
             const int s_begin = tc.z * per;
@@ -708,7 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             mbar_arrive(acce0 + 8u * ab);
             if (++ab == 2) { ab = 0; aph ^= 1u; }
         }
-        if (!p.fuse_update && p.tma_store && lane == 0) bulk_wait_all();
+        if (p.tma_store && lane == 0) bulk_wait_all();
     }
     tc_fence_before();
     __syncthreads();
@@ -747,6 +665,8 @@ struct ConvParams {
     int tma_store;
     int m_tiles, n_tiles, groups, splits;   // tile decomposition (m fastest, then n, group, k split)
     int tiles_total;
+    int rot_mod;        // tile t starts its reduction at (filter row, chunk) step (t % rot_mod) % steps of its range: neighbouring tiles
+                        // start at different steps, whatever CTA works on them
     int b_res;          // 1: all kh*kw weight tiles of the layer fit in one group slot and stay there for the whole CTA (one
                         // n tile, one group, one chunk, no split: conv1), loaded once instead of once per tile
     int cg;             // 1, or 2: CTA pairs (clusters of two) work on tiles of 2 x MH halves with cta_group::2 instructions
@@ -908,10 +828,10 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 const int m0 = tc.m_tile * tile_rows + row0;
                 const int a_begin = tc.z * per;
                 const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
-                // the reduction order is free: every CTA starts at a different (filter row, chunk) so that the SMs do not
-                // all ask L2 for the same weight tile at the same moment
+                // the reduction order is free: neighbouring tiles start at different (filter row, chunk) steps so that the SMs
+                // do not all ask L2 for the same weight tile at the same moment
                 const int a_end = a_begin + nsteps;
-                int a = a_begin + (int)((unsigned)vb % (unsigned)nsteps);
+                int a = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);
                 int ky = a / p.chunks, ch = a - ky * p.chunks;
                 const int ky0 = a_begin / p.chunks, ch0 = a_begin - ky0 * p.chunks;
                 const int xa = p.a_x0 + tc.g * p.a_gx;
@@ -951,10 +871,10 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 const int n0 = tc.n_tile * BN + rank * (BN / CG);       // this CTA's rows of the weight tile
                 const int a_begin = tc.z * per;
                 const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
-                // the reduction order is free: every CTA starts at a different (filter row, chunk) so that the SMs do not
-                // all ask L2 for the same weight tile at the same moment
+                // the reduction order is free: neighbouring tiles start at different (filter row, chunk) steps so that the SMs
+                // do not all ask L2 for the same weight tile at the same moment
                 const int a_end = a_begin + nsteps;
-                int a = a_begin + (int)((unsigned)vb % (unsigned)nsteps);
+                int a = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);
                 int ky = a / p.chunks, ch = a - ky * p.chunks;
                 const int ky0 = a_begin / p.chunks, ch0 = a_begin - ky0 * p.chunks;
                 const int yb = tc.g * p.b_g_rows + n0;
@@ -999,7 +919,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             for (int tile = vb; tile < p.tiles_total && ok; tile += vgrid) {
                 const int a_begin = z * per;
                 const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
-                int ares = a_begin + (int)((unsigned)vb % (unsigned)nsteps);      // resident filter: the producer's rotation of the filter rows
+                int ares = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);      // resident filter: the producer's rotation of the filter rows
                 TL(const long long cc0 = clock64();)
                 ok = mbar_wait_warp(acce0 + 8u * ab, aph ^ 1u, abort_flag);
                 TL(wC += clock64() - cc0;)
@@ -1619,7 +1539,9 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
             for (int i = 0; i < nsteps; ++i) {
                 if (!(ok = mbar_wait_warp(full0 + 8u * st, ph, abort_flag))) break;
                 tc_fence_after();
-                const uint32_t sa = base + st * stage_bytes;
+                // (masked: in a cluster launch the address of a CTA's shared memory carries its rank above these bits, which
+                // would reach into the descriptor's leading-dimension field)
+                const uint32_t sa = (base + st * stage_bytes) & 0x3FFFFu;
                 const uint64_t ad = adesc0 + (uint64_t)(sa >> 4);
                 const uint64_t bd = bdesc0 + (uint64_t)((sa + kWgABytes + (uint32_t)kx0 * 128u) >> 4);
                 #pragma unroll
@@ -1698,6 +1620,201 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, ncols);
+    }
+}
+
+// ===========================================================================
+// FC weight gradient + momentum update in one pass (HBM-bound: 18 bytes per parameter, 22 with the gradient stored).
+//
+//   dW[n][k] = sum_b dy[b][n] * x[b][k];  v <- mu v - d w - lr dW;  w <- w + v;  bf16 copy of w
+//
+// The GEMM runs transposed: the 128 rows of a tile (TMEM lanes) are consecutive k, its columns are rows n of the weight
+// matrix.  An epilogue warp then holds, per accumulator column, 32 consecutive weights of one row: w and v come from a ring of
+// TMA boxes (128 k x 16 rows, read without bank conflicts), the new values leave as full 128-byte lines.
+// What bounds it on few SMs: an SM moves about 93 GB/s to and from HBM (46 each way, measured with a copy on 8-64 SMs; 62 GB/s of
+// stores alone), and this kernel about 80 with its operand tiles included.  So 64 SMs reach 4.7 TB/s of algorithmic bytes
+// (fc6 at batch 128: 161 us; 80 SMs 134 us, all 148 no faster than 136 us), and the grid is kept well below the machine: the
+// other SMs run the tensor-bound data gradients of conv5..conv3 meanwhile.  The form it
+// replaces (four epilogue warps with TMA stores of 32 x 32 slabs) needed all SMs for its 148 us.
+// Warps: 0 = TMA producer of the operands, 1 = MMA issuer and TMEM owner, 2 = TMA producer of w and v, 3..18 = epilogue in
+// four sets of four warps; set s takes columns 16 s .. 16 s + 15 and 64 + 16 s .. of a tile.
+struct FcUpdParams {
+    CUtensorMap tmX, tmD;        // x [B][K] and dy [B][N], boxes of 64 columns x 64 rows
+    CUtensorMap tmW, tmV, tmS;   // fp32 w and v, bf16 copy of w: [N][K], boxes of 128 columns x kUpdRows rows, no swizzle
+    int n_tiles, tiles_total;    // tiles numbered with the k tile fastest
+    int steps, stages;           // 64-image steps of the reduction; ring depth
+    int N;
+    float lr, mu, d;             // d = lr * weight decay
+    float *w, *v, *g;            // g: nullptr unless the gradient is stored as well
+    int* status;
+};
+constexpr int kUpdThreads = 32 * 19, kUpdBN = 128, kUpdRows = 16, kUpdRing = 8;
+constexpr uint32_t kUpdStageBytes = 2 * 16384, kUpdWvBytes = 2 * kUpdRows * 512, kUpdShBytes = kUpdRows * 256;
+inline size_t fc_upd_smem_bytes(int stages) { return 1024 + (size_t)stages * kUpdStageBytes + kUpdRing * (kUpdWvBytes + kUpdShBytes) + 512; }
+
+template <int K>
+__global__ void __launch_bounds__(kUpdThreads, 1) fc_update_kernel(const __grid_constant__ FcUpdParams p) {
+    kn::pdl_trigger();
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const int stages = p.stages;
+    // barriers: full[8] @0, empty[8] @64, acc_full[2] @128, acc_empty[2] @144, wv_full[8] @176, wv_empty[8] @240; tmem slot @160,
+    // abort flag @168
+    const uint32_t wv0 = base + stages * kUpdStageBytes;
+    const uint32_t sh0 = wv0 + kUpdRing * kUpdWvBytes, bar_base = sh0 + kUpdRing * kUpdShBytes;
+    uint8_t* gen = smem_raw + (bar_base - raw);
+    volatile int* abort_flag = (volatile int*)(gen + 168);
+    volatile uint32_t* tmem_slot = (volatile uint32_t*)(gen + 160);
+    const uint32_t full0 = bar_base, empty0 = bar_base + 64u, accf0 = bar_base + 128u, acce0 = bar_base + 144u;
+    const uint32_t wvf0 = bar_base + 176u, wve0 = bar_base + 240u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kMt = K / 128;
+    constexpr uint32_t kCols = 2 * kUpdBN;
+
+    if (threadIdx.x == 0) {
+        *abort_flag = 0;
+        for (int s = 0; s < stages; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(accf0 + 8u * s, 1); mbar_init(acce0 + 8u * s, 16); }
+        for (int s = 0; s < kUpdRing; ++s) { mbar_init(wvf0 + 8u * s, 1); mbar_init(wve0 + 8u * s, 4); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tma_prefetch_desc(&p.tmX);
+        tma_prefetch_desc(&p.tmD);
+        tma_prefetch_desc(&p.tmW);
+        tma_prefetch_desc(&p.tmV);
+        tma_prefetch_desc(&p.tmS);
+    }
+    if (warp == 1) tmem_alloc(smem_u32((const void*)tmem_slot), kCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    kn::pdl_wait();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int st = 0; uint32_t ph = 0;
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < p.tiles_total && ok; tile += gridDim.x) {
+                const int k0 = (tile % kMt) * 128, n0 = (tile / kMt) * kUpdBN;
+                for (int i = 0; i < p.steps; ++i) {
+                    if (!(ok = mbar_wait(empty0 + 8u * st, ph ^ 1u, abort_flag))) break;
+                    const uint32_t sa = base + st * kUpdStageBytes, fb = full0 + 8u * st;
+                    mbar_expect_tx(fb, kUpdStageBytes);
+                    tma_load_2d(sa, &p.tmX, k0, 64 * i, fb);
+                    tma_load_2d(sa + 8192u, &p.tmX, k0 + 64, 64 * i, fb);
+                    tma_load_2d(sa + 16384u, &p.tmD, n0, 64 * i, fb);
+                    tma_load_2d(sa + 24576u, &p.tmD, n0 + 64, 64 * i, fb);
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        const uint32_t idesc = instr_desc(kUpdBN, 1, 1);
+        int st = 0; uint32_t ph = 0;
+        int ab = 0; uint32_t aph = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < p.tiles_total && ok; tile += gridDim.x) {
+            if (!(ok = mbar_wait_warp(acce0 + 8u * ab, aph ^ 1u, abort_flag))) break;
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(ab * kUpdBN);
+            for (int i = 0; i < p.steps; ++i) {
+                if (!(ok = mbar_wait_warp(full0 + 8u * st, ph, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t sa = base + st * kUpdStageBytes;
+                #pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    umma(d, smem_desc(sa + j * 2048u, 8192, 1024), smem_desc(sa + 16384u + j * 2048u, 8192, 1024), idesc, (i > 0 || j > 0) ? 1u : 0u);
+                umma_commit(empty0 + 8u * st);
+                if (++st == stages) { st = 0; ph ^= 1u; }
+            }
+            if (!ok) break;
+            umma_commit(accf0 + 8u * ab);
+            if (++ab == 2) { ab = 0; aph ^= 1u; }
+        }
+    } else if (warp == 2) {
+        // ------------------------------------------------------------ weights and momenta, kUpdRows rows of a tile per stage
+        if (lane == 0) {
+            int st = 0; uint32_t ph = 0;
+            bool ok = true;
+            for (int tile = blockIdx.x; tile < p.tiles_total && ok; tile += gridDim.x) {
+                const int k0 = (tile % kMt) * 128, n0 = (tile / kMt) * kUpdBN;
+                for (int c = 0; c < kUpdBN; c += kUpdRows) {
+                    if (!(ok = mbar_wait(wve0 + 8u * st, ph ^ 1u, abort_flag))) break;
+                    const uint32_t dst = wv0 + st * kUpdWvBytes, fb = wvf0 + 8u * st;
+                    mbar_expect_tx(fb, kUpdWvBytes);
+                    tma_load_2d(dst, &p.tmW, k0, n0 + c, fb);
+                    tma_load_2d(dst + kUpdWvBytes / 2, &p.tmV, k0, n0 + c, fb);
+                    if (++st == kUpdRing) { st = 0; ph ^= 1u; }
+                }
+            }
+        }
+    } else {
+        const int quad = warp & 3, set = (warp - 3) >> 2;            // TMEM lane quadrant; the set takes stages `set` and `set + 4` of a tile
+        const bool leader = ((warp - 3) & 3) == 0 && lane == 0;
+        int ab = 0; uint32_t aph = 0, ph = 0;
+        bool ok = true;
+        // (when a wait has expired a warp waits no more and stores nothing, but walks on to the end of its tile list: the four
+        // warps of a set must all arrive at its barrier)
+        for (int tile = blockIdx.x; tile < p.tiles_total; tile += gridDim.x) {
+            const int n0 = (tile / kMt) * kUpdBN, kl = quad * 32 + lane;
+            if (ok) ok = mbar_wait_warp(accf0 + 8u * ab, aph, abort_flag);
+            tc_fence_after();
+            const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * kUpdBN + set * 16);
+            uint32_t acc[2][16];
+            tmem_ld16(t0, acc[0]);
+            tmem_ld16(t0 + 64u, acc[1]);
+            tmem_ld_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acce0 + 8u * ab);
+            #pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int st = set + 4 * half;
+                if (ok) ok = mbar_wait_warp(wvf0 + 8u * st, ph, abort_flag);
+                const float* ws = (const float*)(smem_raw + (wv0 + st * kUpdWvBytes - raw)) + kl;
+                float wr[16], vr[16];
+                #pragma unroll
+                for (int j = 0; j < 16; ++j) { wr[j] = ws[j * 128]; vr[j] = ws[kUpdRows * 128 + j * 128]; }
+                fence_async_smem();          // these reads before the stage's refill by TMA
+                __syncwarp();
+                if (lane == 0) mbar_arrive(wve0 + 8u * st);
+                const int n = n0 + st * 16;
+                const uint32_t sp = sh0 + st * kUpdShBytes + 2u * kl;
+                const unsigned off = (unsigned)n * K + (unsigned)((tile % kMt) * 128 + kl);
+                #pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (ok && n + j < p.N) {
+                        const float g = __uint_as_float(acc[half][j]);
+                        if (p.g) __stcs(p.g + off + j * K, g);
+                        kn::sgd_step(wr[j], vr[j], g, p.d, p.lr, p.mu);
+                        __stcs(p.w + off + j * K, wr[j]);
+                        __stcs(p.v + off + j * K, vr[j]);
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(sp + j * 256u), "h"(__bfloat16_as_ushort(__float2bfloat16_rn(wr[j]))) : "memory");
+                    }
+                // the bf16 copy leaves through shared memory: as 64-byte stores it would cost a third of the store issue rate.  The
+                // two tiles of a set take turns: the store before this one has been read when the other tile is written next.
+                fence_async_smem();
+                if (leader) bulk_wait_read_0();
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory");
+                if (leader && ok) { tma_store_2d(&p.tmS, sh0 + st * kUpdShBytes, (tile % kMt) * 128, n); bulk_commit(); }
+            }
+            ph ^= 1u;
+            if (++ab == 2) { ab = 0; aph ^= 1u; }
+        }
+        if (leader) bulk_wait_all();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        if (threadIdx.x == 0 && p.status) atomicExch(p.status, 1);
+        long long t0 = clock64();
+        while (clock64() - t0 < 2000000LL) { }
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, kCols);
     }
 }
 

@@ -263,6 +263,7 @@ def test_fused_lrn_pool_forward_argmax_bit_exact(net, which, ta, tn, tp, targ, t
 def test_fused_lrn_pool_rows_per_block(batch):
     """The fused forward kernel with one, two and three output rows per block (the rule takes them at these batches; 27 and 13
     output rows leave a partial last block) on random activations: first and last image, values and argmax codes bit for bit."""
+    from paper_1412_2302_b200.alexnet import AlexNet
     n = AlexNet(batch=batch, seed=SEED, mean_image=synth.mean_image(SEED))
     for which, ta, tn, tp, targ, _, _, shp in FUSED:
         a = np.maximum(np.random.default_rng([batch, which]).standard_normal((batch,) + shp).astype(np.float32), 0) * 20

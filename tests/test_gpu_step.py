@@ -381,6 +381,33 @@ def test_fused_fc_update_gives_the_same_parameters():
     assert not np.array_equal(w0, w)
 
 
+@pytest.mark.parametrize("B", [1, 64, 65, 130])
+def test_fc_update_kernel_equals_gradient_then_update(B):
+    """The kernel that forms the FC weight gradients and updates the weights, at one, two and three 64-image steps with ragged
+    last ones (fc8's 1000 rows leave a partial tile at every batch): parameters, momentum and, with default flags, the
+    gradient must equal forward_backward followed by apply_update (the same sums in the same order)."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed = BASE + 21
+    w = synth.init_params(seed, variance_preserving=True, bias=0.1)
+    res = []
+    for flags, split in ((0, False), (A.FLAG_FUSED_FC_UPDATE, False), (0, True)):
+        net = make(B, seed=seed, flags=flags)
+        net.set_params(w)
+        for step in range(2):
+            load(net, 0, seed, step, B)
+            if split:
+                net.forward_backward(0)
+                net.apply_update(0, 1.0)
+            else:
+                net.train_step(0)
+        res.append([net.get_params(0, k) for k in ((0, 1) if flags else (0, 1, 2))])
+        net.close()
+    for got in res[:2]:
+        for a, b in zip(got, res[2]):
+            assert np.array_equal(a, b)
+    assert not np.array_equal(res[2][0], w)
+
+
 def test_fc_forward_chain_equals_three_launches():
     """ALEXNET_FLAG_FC_CHAIN: fc6 -> fc7 -> fc8 forward as one cooperative launch against the three per-layer launches:
     same units, same summation order, so activations, dropout masks, logits, losses and the parameters after three steps
