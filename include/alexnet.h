@@ -353,7 +353,7 @@ int alexnet_timeline_read(long long* host_out, int clear);
  * Such callers are, for example, a loop in the middle of overlapped steps,
  * where cudaMalloc / cudaFree would synchronise the device and serialise the
  * loader stream with the compute stream, or a process that has handed all free
- * HBM to the arena of alexnet_create.  The scratch of the two-stage reduction
+ * HBM to the arena of alexnet_create.  The scratch of the reduction
  * lives in a fixed 1 MiB array inside the library image, held by every GPU that
  * loads the library until the process exits; nothing is allocated or freed.
  *   dev_dy    device, bf16 [rows][channels], row-major, 16-byte aligned; read only
@@ -361,7 +361,7 @@ int alexnet_timeline_read(long long* host_out, int clear);
  *   channels  multiple of 8, at most 4096 (the fixed scratch); larger values are
  *             rejected with ALEXNET_ERR_ARG and a message
  *   dev_db    device, fp32 [channels]; written
- *   stream    cudaStream_t the two kernels are launched on (asynchronous)
+ *   stream    cudaStream_t the kernel is launched on (asynchronous)
  *   err       optional host buffer for an error message (may be NULL)
  * The first call on a device looks up the scratch address for that device;
  * make that call before any stream capture begins there.  All calls share the

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -56,6 +57,7 @@ class AlexNetError(RuntimeError):
 
 
 _lib = None
+_local = threading.local()
 
 
 def load_library():
@@ -371,10 +373,11 @@ def bias_grad_noalloc(dy, db, stream=None):
     [channels], written in place.  For callers that must not allocate device
     memory (see include/alexnet.h); channels is limited to 4096.  Raises
     AlexNetError with the library's message when the sizes are rejected."""
-    lib = load_library()
-    msg = ctypes.create_string_buffer(256)
-    rows, ch = int(dy.shape[0]), int(dy.shape[1])
-    rc = lib.alexnet_bias_grad_noalloc(_ptr(dy), rows, ch, _ptr(db),
-                                       ctypes.c_void_p(stream.cuda_stream if stream is not None else 0), msg, 256)
+    lib = _lib or load_library()
+    msg = getattr(_local, "msg", None)
+    if msg is None:
+        msg = _local.msg = ctypes.create_string_buffer(256)      # kept per thread: allocating it costs as much as the call
+    rows, ch = dy.shape
+    rc = lib.alexnet_bias_grad_noalloc(dy.data_ptr(), rows, ch, db.data_ptr(), stream.cuda_stream if stream is not None else None, msg, 256)
     if rc != OK:
         raise AlexNetError(rc, msg.value.decode())

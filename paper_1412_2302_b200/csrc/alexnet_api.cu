@@ -1831,7 +1831,7 @@ const char* alexnet_last_error(const alexnet_t* h) { return h ? h->err.c_str() :
 // serialise the loader stream with the compute stream), or a process that has
 // already given every free byte of HBM to the arena it passed to
 // alexnet_create.  For them this entry point keeps its scratch -- the per-split
-// partial column sums of the two-stage reduction -- in a fixed array that is
+// partial column sums of the reduction -- in a fixed array that is
 // part of the loaded library image.  Every GPU that loads the library holds
 // that array (kNoAllocSplits * kNoAllocMaxC floats = 1 MiB) until the process
 // exits.
@@ -1843,16 +1843,19 @@ const char* alexnet_last_error(const alexnet_t* h) { return h ? h->err.c_str() :
 // call before starting any stream capture on that device.
 //
 // All calls share the one array and it keeps whatever the last call left in it.
-// Nothing in it has to start at zero: the first stage writes every partial the
-// second stage reads, in the same call.  Two calls whose kernels overlap on the
-// GPU (different streams, no dependency) race on it; order them.
+// Nothing in it has to start at zero: a call writes every partial that it later
+// reads.  (The counters beside it, of finished row splits per 64 columns, start at
+// zero and are reset by every call.)  Two calls whose kernels overlap on the GPU
+// (different streams, no dependency) race on it; order them.
 namespace {
 constexpr int kNoAllocSplits = 64;
 constexpr int kNoAllocMaxC = 4096;
 static __device__ __align__(256) float g_noalloc_partials[kNoAllocSplits * kNoAllocMaxC];
+static __device__ unsigned g_noalloc_counters[kNoAllocMaxC / 64];      // finished row splits per 64 columns; zero between calls
 
 constexpr int kMaxDevices = 64;
 float* g_noalloc_ptr[kMaxDevices] = {nullptr};
+unsigned* g_noalloc_cnt[kMaxDevices] = {nullptr};
 
 void put_err(char* buf, size_t len, const char* msg) {
     if (buf && len) { snprintf(buf, len, "%s", msg); }
@@ -1877,19 +1880,23 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
     if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) { put_err(err, err_len, "bias_grad_noalloc: cudaGetDevice failed"); return ALEXNET_ERR_CUDA; }
     if (!g_noalloc_ptr[dev]) {
         float* p = nullptr;
-        e = cudaGetSymbolAddress((void**)&p, g_noalloc_partials);
-        if (e != cudaSuccess || !p) {
+        unsigned* q = nullptr;
+        e = cudaGetSymbolAddress((void**)&q, g_noalloc_counters);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&p, g_noalloc_partials);
+        if (e != cudaSuccess || !p || !q) {
             put_err(err, err_len, cudaGetErrorString(e));
             return ALEXNET_ERR_CUDA;
         }
+        g_noalloc_cnt[dev] = q;
         g_noalloc_ptr[dev] = p;
     }
-    float* scratch = g_noalloc_ptr[dev];
-    cudaStream_t st = (cudaStream_t)stream;
-    int splits = (int)std::min<int64_t>(kNoAllocSplits, std::max<int64_t>(1, rows / 256));
-    dim3 grid((channels + 63) / 64, splits);
-    launch_k(kn::colsum_kernel, grid, 256, 0, st, (const bf16*)dev_dy, (long long)rows, channels, scratch);
-    launch_k(kn::colsum_final_kernel, (channels + 127) / 128, 128, 0, st, scratch, splits, channels, dev_db);
+    // row splits: four blocks per SM in total, at least 64 rows each, as many as the scratch holds
+    const int groups = (channels + 63) / 64;
+    int64_t splits = std::min<int64_t>(4 * 148 / groups, rows / 64);
+    splits = std::min<int64_t>(splits, kNoAllocSplits * kNoAllocMaxC / channels);
+    splits = std::max<int64_t>(splits, 1);
+    launch_k(kn::bias_grad_kernel, dim3(groups, (unsigned)splits), 256, 0, (cudaStream_t)stream, (const bf16*)dev_dy, (long long)rows, channels,
+             g_noalloc_ptr[dev], g_noalloc_cnt[dev], dev_db);
     e = cudaGetLastError();
     if (e != cudaSuccess) { put_err(err, err_len, cudaGetErrorString(e)); return ALEXNET_ERR_CUDA; }
     return ALEXNET_OK;

@@ -727,6 +727,83 @@ __global__ void colsum_scalar_kernel(const __nv_bfloat16* __restrict__ dy, int r
     db[c] = s;
 }
 
+// The same column sums in one launch, for the allocation-free entry point: grid (ceil(C/64), row splits), a block sums 64 columns of
+// its rows (eight 16-byte loads of a thread in flight), and the block of a column group that finishes last adds the
+// group's partials in a fixed order (a counter per group, reset for the next call), so the result does not depend on which
+// block that is.  HBM-bound (L2-bound where dy fits); 25088 x 384 took 12.2 us per call as two launches with one load in
+// flight per thread, 7.6 us in this form, about half of it the launch.
+__global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
+                                                        unsigned* __restrict__ counters, float* __restrict__ db) {
+    pdl_sync();
+    __shared__ __align__(16) float red[16][68];
+    __shared__ bool last;
+    const int tid = threadIdx.x, cc = tid & 7, rl = tid >> 3;
+    const int c0 = blockIdx.x * 64 + cc * 8;
+    const long long per = (rows + gridDim.y - 1) / gridDim.y;
+    const long long r0 = (long long)blockIdx.y * per, r1 = min(rows, r0 + per);
+    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (c0 < C) {
+        for (long long r = r0 + rl; r < r1; r += 32 * 8) {
+            uint4 u[8];
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                u[q] = make_uint4(0u, 0u, 0u, 0u);
+                if (r + 32 * q < r1) u[q] = __ldg((const uint4*)(dy + (r + 32 * q) * C + c0));
+            }
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                float f[8];
+                unpack8(u[q], f);
+                #pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i] += f[i];
+            }
+        }
+    }
+    #pragma unroll
+    for (int i = 0; i < 8; ++i) {                // the four row lanes of a warp
+        acc[i] += __shfl_xor_sync(~0u, acc[i], 8);
+        acc[i] += __shfl_xor_sync(~0u, acc[i], 16);
+    }
+    if ((tid & 31) < 8) {
+        #pragma unroll
+        for (int i = 0; i < 8; ++i) red[tid >> 5][cc * 8 + i] = acc[i];
+    }
+    __syncthreads();
+    const int splits = gridDim.y, c = blockIdx.x * 64 + tid;
+    if (tid < 64 && c < C) {
+        float s = 0.f;
+        #pragma unroll
+        for (int w = 0; w < 8; ++w) s += red[w][tid];
+        if (splits == 1) db[c] = s;
+        else partial[(size_t)blockIdx.y * C + c] = s;
+    }
+    if (splits == 1) return;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(counters + blockIdx.x, 1u) == (unsigned)splits - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int q4 = tid & 15, zl = tid >> 4, cq = blockIdx.x * 64 + 4 * q4;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (cq < C) {
+        #pragma unroll 4
+        for (int z = zl; z < splits; z += 16) {
+            const float4 t = __ldcg((const float4*)(partial + (size_t)z * C + cq));
+            a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
+        }
+    }
+    *(float4*)&red[zl][4 * q4] = a;
+    __syncthreads();
+    if (tid < 64 && c < C) {
+        float s = 0.f;
+        #pragma unroll
+        for (int w = 0; w < 16; ++w) s += red[w][tid];
+        db[c] = s;
+    }
+    if (tid == 0) counters[blockIdx.x] = 0u;
+}
+
 // ------------------------------------------------------ softmax cross-entropy
 // one block per sample: p = softmax(z), loss_n = -log p[label], dz = (p - onehot)/B as bf16
 __global__ void softmax_xent_kernel(const float* __restrict__ z, const int32_t* __restrict__ labels,
