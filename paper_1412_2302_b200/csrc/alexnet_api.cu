@@ -5,6 +5,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -164,6 +165,7 @@ struct Replica {
     bool n_stale[2], dn_stale[2];
     // plans
     Plan conv_fwd[5][2], conv_bwd[5], conv_wg[5][2], fc_fwd[3], fc_bwd[3];
+    std::vector<Plan> eval_conv[2];    // per slot: the forward convolutions of every chunk of an evaluation from host memory
     Plan conv_bwd_beside[5];    // the same data gradients on the SMs that the FC updates leave free (conv3-5)
     Plan fc_wg_plain[3];    // the FC weight gradient stored (alexnet_forward_backward)
     Plan fc_upd[3];         // ... with the momentum update of the FC weights; it also stores the gradient unless the handle was
@@ -190,6 +192,13 @@ struct alexnet {
     cudaEvent_t ev_fork[kBranches] = {};   // the inputs of branch b are ready on the compute stream
     bool fc_grads_on_branches = false;     // the last backward pass ran the FC weight gradients on branches 0-2: ev_side_done[0..2]
                                            // then complete as soon as those gradients exist, long before the pass ends
+    // copies of losses (alexnet_loss_async) leave on a stream of their own as soon as the loss exists, beside the backward pass
+    cudaStream_t loss_stream = nullptr;
+    cudaEvent_t ev_loss_stored = nullptr;
+    bool loss_at_fork = false;             // the loss of the last pass exists at ev_fork[2] (that pass was forked)
+    std::vector<cudaEvent_t> ev_chunk;     // the copy of chunk c of an evaluation batch is done
+    kn::HostResult* host_result = nullptr; // mapped host memory: results of the calls that wait (one at a time per handle)
+    uint32_t result_seq = 0;
     cudaEvent_t ev_backward_done = nullptr;   // recorded on the compute stream after every backward pass
     size_t ws_conv_off[5] = {};            // floats: each conv layer's split partials have their own region of the workspace
     float* bias_partial = nullptr;         // [5][kBiasPartial] bias-gradient partials of the conv weight-gradient kernels
@@ -489,10 +498,10 @@ int conv_out_map(alexnet* h, tc::ConvParams& p, const void* out, int ldo, long l
     return make_tm_out(h, &p.tmOut, out, false, (uint64_t)ldo, (uint64_t)M, 1, (uint64_t)ldo * 2, (uint64_t)ldo * 2 * (uint64_t)M);
 }
 
-int plan_conv_fwd(alexnet* h, Plan& P, const ConvL& c, const bf16* in, const bf16* wsh, const float* bias, bf16* out) {
+int plan_conv_fwd(alexnet* h, Plan& P, const ConvL& c, const bf16* in, const bf16* wsh, const float* bias, bf16* out, int images) {
     memset(&P, 0, sizeof(P));
     tc::ConvParams& p = P.c;
-    const long long M = (long long)h->B * c.gin.Hp * c.gin.Wp;
+    const long long M = (long long)images * c.gin.Hp * c.gin.Wp;
     const int gp = c.gin.Wp;
     p.kh = p.kw = c.k; p.chunks = (c.cig + 63) / 64; p.kk = c.cig == 48 ? 3 : 4;
     const ConvShape sh = choose_conv_shape(h, M, c.cog, c.groups, p.kh, p.kw, p.chunks, p.kk);
@@ -713,7 +722,7 @@ int build_plans(alexnet* h, int r) {
         const ConvL& c = L.conv[l];
         for (int s = 0; s < 2; ++s) {
             const bf16* x = l == 0 ? R.x0[s] : in[l];
-            if ((rc = plan_conv_fwd(h, R.conv_fwd[l][s], c, x, R.shadow + c.w_off, R.w + c.b_off, out[l]))) return rc;
+            if ((rc = plan_conv_fwd(h, R.conv_fwd[l][s], c, x, R.shadow + c.w_off, R.w + c.b_off, out[l], h->B))) return rc;
             if ((rc = plan_conv_wg(h, R.conv_wg[l][s], l, c, dyv[l], x))) return rc;
         }
         if ((rc = plan_conv_bwd(h, R.conv_bwd[l], c, dyv[l], R.wt + c.wt_off, maskv[l], dxv[l]))) return rc;
@@ -732,6 +741,31 @@ int build_plans(alexnet* h, int r) {
         if ((rc = plan_fc_upd(h, R.fc_upd[l], f, fdy[l], fx[l], g, R.w + f.w_off, R.v + f.w_off, R.shadow + f.w_off))) return rc;
     }
     plan_fc_chain(h, r);
+    return ALEXNET_OK;
+}
+
+// An evaluation whose images come over PCIe works in chunks of images: the convolution layers of one chunk run while the next is
+// copied.  A chunk of n images takes about 85 + 1.2 n us (eight dependent launches and the work) and its copy 3.6 n us, so
+// from about 40 images on the copies are the longer side; what is left behind the last copy is one chunk's time.
+constexpr int kEvalChunk = 40;
+int eval_chunks(int B) { return std::max(1, B / kEvalChunk); }
+inline int chunk_begin(int B, int chunks, int c) { return (int)((long long)B * c / chunks); }
+int build_eval_plans(alexnet* h, int r, int slot) {
+    Replica& R = h->rep[r];
+    const Layout& L = h->L;
+    const int chunks = eval_chunks(h->B);
+    std::vector<Plan> plans((size_t)chunks * 5);
+    const bf16* in[5] = {R.x0[slot], R.p1, R.p2, R.a3, R.a4};
+    bf16* out[5] = {R.a1, R.a2, R.a3, R.a4, R.a5};
+    for (int c = 0; c < chunks; ++c) {
+        const int i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
+        for (int l = 0; l < 5; ++l) {
+            const ConvL& q = L.conv[l];
+            const size_t off = (size_t)i0 * q.gin.Hp * q.gin.Wp;      // input and output share a grid
+            if (int rc = plan_conv_fwd(h, plans[(size_t)c * 5 + l], q, in[l] + off * q.cin, R.shadow + q.w_off, R.w + q.b_off, out[l] + off * q.cout, n)) return rc;
+        }
+    }
+    R.eval_conv[slot].swap(plans);
     return ALEXNET_OK;
 }
 
@@ -902,14 +936,16 @@ void op_lrn_bwd(alexnet* h, int r, int which, cudaStream_t st) {
 }
 struct PoolGeo { int C, Hpi, Wpi, Hi, Wi, Ho, Wo, Hpo, Wpo; };
 const PoolGeo kPool[3] = {{96, 57, 57, 55, 55, 27, 27, 29, 29}, {256, 29, 29, 27, 27, 13, 13, 14, 14}, {256, 14, 14, 13, 13, 6, 6, 6, 6}};
-void op_pool_fwd(alexnet* h, int r, int which, cudaStream_t st) {
+void op_pool_fwd(alexnet* h, int r, int which, cudaStream_t st, int i0 = 0, int images = 0) {
+    if (!images) images = h->B;
     Replica& R = h->rep[r];
     const PoolGeo& g = kPool[which];
     const bf16* x[3] = {R.n1, R.n2, R.a5};
     bf16* y[3] = {R.p1, R.p2, R.p5};
     uint8_t* a[3] = {R.arg1, R.arg2, R.arg5};
-    const dim3 grid(nblk((long long)g.Wo * (g.C / 8), 256), g.Ho, h->B);
-    launch_k(kn::pool_fwd_kernel, grid, 256, 0, st, x[which], y[which], a[which], g.C / 8, g.Hpi, g.Wpi, g.Ho, g.Wo, g.Hpo, g.Wpo);
+    const dim3 grid(nblk((long long)g.Wo * (g.C / 8), 256), g.Ho, images);
+    launch_k(kn::pool_fwd_kernel, grid, 256, 0, st, x[which] + (size_t)i0 * g.Hpi * g.Wpi * g.C, y[which] + (size_t)i0 * g.Hpo * g.Wpo * g.C,
+             a[which] + (size_t)i0 * g.Ho * g.Wo * g.C, g.C / 8, g.Hpi, g.Wpi, g.Ho, g.Wo, g.Hpo, g.Wpo);
     h->launches++;
 }
 void op_pool_bwd(alexnet* h, int r, int which, cudaStream_t st) {
@@ -931,7 +967,8 @@ void op_pool_bwd(alexnet* h, int r, int which, cudaStream_t st) {
 #define LRN_POOL_FWD_2(B75) kn::lrn_pool_fwd_kernel<32, 16, 27, 27, B75, 3>
 #define POOL_LRN_BWD_1(B75) kn::pool_lrn_bwd_kernel<12, 55, 55, B75>
 #define POOL_LRN_BWD_2(B75) kn::pool_lrn_bwd_kernel<32, 27, 27, B75>
-void op_lrn_pool_fwd(alexnet* h, int r, int which, cudaStream_t st) {
+void op_lrn_pool_fwd(alexnet* h, int r, int which, cudaStream_t st, int i0 = 0, int images = 0) {
+    if (!images) images = h->B;
     Replica& R = h->rep[r];
     const PoolGeo& g = kPool[which];
     const bool b75 = h->cfg.lrn_beta == 0.75f;
@@ -939,11 +976,12 @@ void op_lrn_pool_fwd(alexnet* h, int r, int which, cudaStream_t st) {
     // batch 1 / 8 / 32 / 512, LRN1 4.1 / 6.4 / 12.3 / 128 us by this rule (6.2 / 6.6 / 12.3 / 128 with three everywhere, 154
     // with one row at 512, where every second input row would be normalised twice)
     int opr = 1;
-    while (opr < 3 && (long long)nblk(g.Ho, opr) * 2 * h->B * 10 > (which == 0 ? 4 : 3) * h->sm_count * 11) ++opr;
-    const dim3 grid(nblk(g.Ho, opr), 2, h->B);
+    while (opr < 3 && (long long)nblk(g.Ho, opr) * 2 * images * 10 > (which == 0 ? 4 : 3) * h->sm_count * 11) ++opr;
+    const dim3 grid(nblk(g.Ho, opr), 2, images);
     const int nt = which == 0 ? 28 * 6 : 14 * 16;
     auto k = which == 0 ? (b75 ? LRN_POOL_FWD_1(true) : LRN_POOL_FWD_1(false)) : (b75 ? LRN_POOL_FWD_2(true) : LRN_POOL_FWD_2(false));
-    launch_k(k, grid, nt, 0, st, which ? R.a2 : R.a1, which ? R.p2 : R.p1, which ? R.arg2 : R.arg1, opr, g.Hpi, g.Wpi,
+    launch_k(k, grid, nt, 0, st, (which ? R.a2 : R.a1) + (size_t)i0 * g.Hpi * g.Wpi * g.C, (which ? R.p2 : R.p1) + (size_t)i0 * g.Hpo * g.Wpo * g.C,
+             (which ? R.arg2 : R.arg1) + (size_t)i0 * g.Ho * g.Wo * g.C, opr, g.Hpi, g.Wpi,
              g.Hpo, g.Wpo, h->alpha_eff, h->cfg.lrn_beta, h->cfg.lrn_k);
     h->launches++;
     R.n_stale[which] = true;
@@ -1014,12 +1052,13 @@ bool op_fc_chain(alexnet* h, int r, uint64_t step, cudaStream_t st, bool eval) {
     h->launches++;
     return true;
 }
-void op_fc8_softmax(alexnet* h, int r, int slot, cudaStream_t st) {
+void op_fc8_softmax(alexnet* h, int r, int slot, cudaStream_t st, bool eval) {
     Replica& R = h->rep[r];
     const FcL& f = h->L.fc[2];
     const Plan& P = R.fc_fwd[2];
-    launch_k(kn::fc8_softmax_xent_kernel, h->B, 256, 0, st, h->ws, P.c.splits, P.c.split_stride, R.w + f.b_off, R.z, R.labels[slot], R.dz,
-             R.loss_n, R.loss, h->status + 8, h->B, f.N);
+    launch_k(eval ? kn::fc8_softmax_xent_kernel<true> : kn::fc8_softmax_xent_kernel<false>, h->B, 256, 0, st, h->ws, P.c.splits, P.c.split_stride,
+             R.w + f.b_off, R.z, R.labels[slot], R.dz, R.loss_n, R.loss, h->status + 8, h->B, f.N, (int32_t*)(h->status + 4), h->status,
+             h->host_result, h->result_seq);
     h->launches++;
 }
 // The conv split reduction may ride in the update launch when that launch takes the conv filters and every bias in one go
@@ -1091,34 +1130,56 @@ void op_average(alexnet* h, cudaStream_t st) {
     h->launches++;
     refresh_transposed_both(h, st);
 }
-void op_preprocess(alexnet* h, int r, int slot, uint64_t step, cudaStream_t st, bool eval = false) {
+// labels != nullptr: taken along by the kernel (see label_source)
+void op_preprocess(alexnet* h, int r, int slot, uint64_t step, cudaStream_t st, bool eval = false, const int32_t* labels = nullptr, int i0 = 0,
+                   int images = 0) {
     Replica& R = h->rep[r];
+    if (!images) images = h->B;
     kn::ColorAug aug = h->color;
     aug.key = kn::stream_key(h->cfg.seed, 10, r, step);
-    const dim3 grid(57, h->B);
-    if (aug.sigma != 0.f && !eval)
-        launch_k(kn::preprocess_kernel<true>, grid, 256, 0, st, R.stage[slot], h->mean, R.x0[slot], R.cf[slot], h->B,
-                 kn::stream_key(h->cfg.seed, 1, r, step), 0, aug);
-    else
-        launch_k(kn::preprocess_kernel<false>, grid, 256, 0, st, R.stage[slot], h->mean, R.x0[slot], R.cf[slot], h->B,
-                 kn::stream_key(h->cfg.seed, 1, r, step), eval ? 1 : 0, aug);
+    const bool augment = aug.sigma != 0.f && !eval;
+    launch_k(augment ? kn::preprocess_kernel<true> : kn::preprocess_kernel<false>, dim3(57, images), 256, 0, st, R.stage[slot], h->mean, R.x0[slot],
+             R.cf[slot], labels, R.labels[slot], i0, kn::stream_key(h->cfg.seed, 1, r, step), eval ? 1 : 0, aug);
     h->launches++;
 }
+// the address under which a kernel on this device can read the caller's labels, or nullptr (then they are copied)
+const int32_t* label_source(const int32_t* labels) {
+    cudaPointerAttributes at{};
+    int dev = 0;
+    if (((uintptr_t)labels & 3) || cudaPointerGetAttributes(&at, labels) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type == cudaMemoryTypeHost || (at.type == cudaMemoryTypeDevice && at.device == dev)) return (const int32_t*)at.devicePointer;
+    return nullptr;
+}
 
-void forward(alexnet* h, int r, int slot, cudaStream_t st, bool eval) {
+void forward_fc(alexnet* h, int r, int slot, cudaStream_t st, bool eval) {
     Replica& R = h->rep[r];
     const uint64_t step = R.slot_step[slot];
+    if (!R.chain_mode || !op_fc_chain(h, r, step, st, eval)) {
+        op_fc_fwd(h, r, 0, step, st, eval, false, true); op_fc_fwd(h, r, 1, step, st, eval, false, true);
+        op_fc_fwd(h, r, 2, step, st, eval, true, true);
+    }
+    op_fc8_softmax(h, r, slot, st, eval);
+}
+void forward(alexnet* h, int r, int slot, cudaStream_t st, bool eval) {
     // conv1 may directly follow the kernel that wrote its weights (the update of the step before): it waits in full.  Its
     // CTAs hold every SM until it ends, so no later kernel of the pass can start (and read weights) before that writer is done.
     op_conv_fwd(h, r, 0, slot, st); op_lrn_pool_fwd(h, r, 0, st);
     op_conv_fwd(h, r, 1, slot, st, true); op_lrn_pool_fwd(h, r, 1, st);
     op_conv_fwd(h, r, 2, slot, st, true); op_conv_fwd(h, r, 3, slot, st, true); op_conv_fwd(h, r, 4, slot, st, true);
     op_pool_fwd(h, r, 2, st);
-    if (!R.chain_mode || !op_fc_chain(h, r, step, st, eval)) {
-        op_fc_fwd(h, r, 0, step, st, eval, false, true); op_fc_fwd(h, r, 1, step, st, eval, false, true);
-        op_fc_fwd(h, r, 2, step, st, eval, true, true);
-    }
-    op_fc8_softmax(h, r, slot, st);
+    forward_fc(h, r, slot, st, eval);
+}
+// the convolution layers of one chunk of an evaluation batch
+void forward_conv_chunk(alexnet* h, int r, int slot, int c, int chunks, cudaStream_t st) {
+    const std::vector<Plan>& P = h->rep[r].eval_conv[slot];
+    const int i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
+    launch_gemm(h, P[5 * c], st); op_lrn_pool_fwd(h, r, 0, st, i0, n);
+    launch_gemm(h, P[5 * c + 1], st, true); op_lrn_pool_fwd(h, r, 1, st, i0, n);
+    launch_gemm(h, P[5 * c + 2], st, true); launch_gemm(h, P[5 * c + 3], st, true); launch_gemm(h, P[5 * c + 4], st, true);
+    op_pool_fwd(h, r, 2, st, i0, n);
 }
 // update: the FC weights are updated here, by their weight-gradient kernels (the rest of the parameters by op_update)
 void forward_backward(alexnet* h, int r, int slot, cudaStream_t st, bool update, bool defer_conv_reduce) {
@@ -1160,12 +1221,29 @@ void forward_backward(alexnet* h, int r, int slot, cudaStream_t st, bool update,
             cudaEventRecord(h->ev_side_done[b], h->side[b]);
             cudaStreamWaitEvent(st, h->ev_side_done[b], 0);
         }
+    h->loss_at_fork = used[2];
     h->fc_grads_on_branches = used[0] && used[1] && used[2] && !update;
     if (h->ev_backward_done) cudaEventRecord(h->ev_backward_done, st);
 }
 
 int check_status(alexnet* h) {
     if (h->latched) return h->latched;
+    return ALEXNET_OK;
+}
+// Waits for the kernel that publishes result `result_seq` (nothing is queued behind it that the caller needs).  The stream is
+// asked now and then, so that a failed launch or a fault ends the wait with its error.
+int wait_result(alexnet* h, kn::HostResult* out) {
+    volatile kn::HostResult* p = h->host_result;
+    for (unsigned spins = 1; p->seq != h->result_seq; ++spins) {
+        if (spins % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(h->cs);
+        if (e == cudaErrorNotReady) continue;
+        if (e != cudaSuccess) return fail(h, ALEXNET_ERR_CUDA, std::string("waiting for a result: ") + cudaGetErrorString(e));
+        if (p->seq != h->result_seq) return fail(h, ALEXNET_ERR_CUDA, "the stream is idle and the result has not arrived");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    out->top1 = p->top1; out->top5 = p->top5; out->loss = p->loss;
+    if (p->status) { h->latched = ALEXNET_ERR_DEVICE_TIMEOUT; return fail(h, ALEXNET_ERR_DEVICE_TIMEOUT, "a bounded device-side wait expired"); }
     return ALEXNET_OK;
 }
 int poll_status(alexnet* h) {  // after a synchronisation
@@ -1276,6 +1354,10 @@ void teardown(alexnet* h) {
         if (h->ev_fork[b]) cudaEventDestroy(h->ev_fork[b]);
     }
     for (cudaEvent_t e : h->prof_ev) cudaEventDestroy(e);
+    if (h->loss_stream) { cudaStreamSynchronize(h->loss_stream); cudaStreamDestroy(h->loss_stream); }
+    if (h->ev_loss_stored) cudaEventDestroy(h->ev_loss_stored);
+    for (cudaEvent_t e : h->ev_chunk) cudaEventDestroy(e);
+    if (h->host_result) cudaFreeHost(h->host_result);
     if (h->ev_backward_done) cudaEventDestroy(h->ev_backward_done);
     for (int r = 0; r < h->cfg.replicas; ++r)
         for (int s = 0; s < 2; ++s) {
@@ -1356,6 +1438,10 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
         CKC(cudaEventCreateWithFlags(&h->ev_fork[b], cudaEventDisableTiming));
     }
     CKC(cudaEventCreateWithFlags(&h->ev_backward_done, cudaEventDisableTiming));
+    CKC(cudaStreamCreateWithFlags(&h->loss_stream, cudaStreamNonBlocking));
+    CKC(cudaEventCreateWithFlags(&h->ev_loss_stored, cudaEventDisableTiming));
+    CKC(cudaHostAlloc((void**)&h->host_result, sizeof(kn::HostResult), cudaHostAllocMapped | cudaHostAllocPortable));
+    memset((void*)h->host_result, 0, sizeof(kn::HostResult));
     // pad positions of every grid must be zero from the start; gradients and momentum start at zero
     CKC(cudaMemsetAsync(h->arena, 0, need, h->cs));
     if (host_mean_image) CKC(cudaMemcpyAsync(h->mean, host_mean_image, 256 * 256 * 3 * sizeof(float), cudaMemcpyHostToDevice, h->cs));
@@ -1400,8 +1486,9 @@ int alexnet_load_batch_async(alexnet_t* h, int replica, const uint8_t* images, c
     const int s = R.next_load;
     if (R.consumed_valid[s]) CK(cudaStreamWaitEvent(h->ls, R.consumed[s], 0));
     CK(cudaMemcpyAsync(R.stage[s], images, (size_t)h->B * 196608, cudaMemcpyDefault, h->ls));
-    CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
-    op_preprocess(h, replica, s, step, h->ls);
+    const int32_t* lsrc = label_source(labels);
+    if (!lsrc) CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
+    op_preprocess(h, replica, s, step, h->ls, false, lsrc);
     CK(cudaEventRecord(R.ready[s], h->ls));
     R.slot_step[s] = step;
     R.last_slot = s; R.next_load ^= 1; R.loaded++;
@@ -1430,9 +1517,13 @@ static int step_impl(alexnet_t* h, int replica, float* host_loss, bool with_upda
     R.last_slot = s; R.next_train ^= 1; R.loaded--;
     CK(cudaGetLastError());
     if (host_loss) {
-        CK(cudaMemcpyAsync(host_loss, R.loss, sizeof(float), cudaMemcpyDeviceToHost, h->cs));
-        CK(cudaStreamSynchronize(h->cs));
-        return poll_status(h);
+        launch_k(kn::store_result_kernel, 1, 1, 0, h->cs, (const float*)R.loss, (const int*)h->status, h->host_result, ++h->result_seq);
+        h->launches++;
+        CK(cudaGetLastError());
+        CK(cudaStreamSynchronize(h->cs));      // the call promises a finished step
+        kn::HostResult res;
+        if (int rc = wait_result(h, &res)) return rc;
+        *host_loss = res.loss;
     }
     return ALEXNET_OK;
 }
@@ -1558,8 +1649,17 @@ int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out) {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, loss_out) == cudaSuccess && at.devicePointer != nullptr &&
         (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)) {
-        launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
+        // A store to host memory takes 7-13 us beside a batch upload.  The loss exists since before the backward pass, so the store
+        // runs there, on a stream of its own, and the compute stream only waits for its (long past) end.
+        const bool early = h->loss_at_fork;
+        cudaStream_t st = early ? h->loss_stream : h->cs;
+        if (early) CK(cudaStreamWaitEvent(st, h->ev_fork[2], 0));
+        launch_k(kn::store_value_kernel, 1, 1, 0, st, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
         h->launches++;
+        if (early) {
+            CK(cudaEventRecord(h->ev_loss_stored, st));
+            CK(cudaStreamWaitEvent(h->cs, h->ev_loss_stored, 0));
+        }
         CK(cudaGetLastError());
         return ALEXNET_OK;
     }
@@ -1577,29 +1677,42 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     if (R.loaded != 0) return fail(h, ALEXNET_ERR_STATE, "eval_batch: a loaded training batch is waiting for its train_step");
     const int s = R.next_load;      // the free slot the next training load would use; it stays free afterwards
     if (R.consumed_valid[s]) CK(cudaStreamWaitEvent(h->ls, R.consumed[s], 0));
-    CK(cudaMemcpyAsync(R.stage[s], images, (size_t)h->B * 196608, cudaMemcpyDefault, h->ls));
-    CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
-    op_preprocess(h, replica, s, 0, h->ls, true);
-    CK(cudaEventRecord(R.ready[s], h->ls));
+    const int32_t* lsrc = label_source(labels);
+    if (!lsrc) CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
     R.slot_step[s] = 0; R.last_slot = s;
-    CK(cudaStreamWaitEvent(h->cs, R.ready[s], 0));
-    forward(h, replica, s, h->cs, true);
-    int32_t* counts = (int32_t*)(h->status + 4);    // two counters in the status block
-    CK(cudaMemsetAsync(counts, 0, 2 * sizeof(int32_t), h->cs));
-    launch_k(kn::topk_count_kernel, h->B, 256, 0, h->cs, R.z, R.labels[s], 1000, counts);
-    h->launches++;
+    ++h->result_seq;
+    h->loss_at_fork = false;
+    // the copies run on the copy stream, everything else (preprocessing too) on the compute stream
+    cudaPointerAttributes at{};
+    const bool on_device = cudaPointerGetAttributes(&at, images) == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
+    cudaGetLastError();
+    const int chunks = on_device || h->prof ? 1 : eval_chunks(h->B);
+    if (chunks > 1 && R.eval_conv[s].empty())
+        if (int rc = build_eval_plans(h, replica, s)) return rc;
+    while ((int)h->ev_chunk.size() < chunks) {
+        cudaEvent_t e;
+        CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        h->ev_chunk.push_back(e);
+    }
+    for (int c = 0; c < chunks; ++c) {
+        const size_t i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
+        CK(cudaMemcpyAsync(R.stage[s] + i0 * 196608, images + i0 * 196608, n * 196608, cudaMemcpyDefault, h->ls));
+        CK(cudaEventRecord(h->ev_chunk[c], h->ls));
+        CK(cudaStreamWaitEvent(h->cs, h->ev_chunk[c], 0));
+        op_preprocess(h, replica, s, 0, h->cs, true, lsrc, (int)i0, (int)n);
+        if (chunks > 1) forward_conv_chunk(h, replica, s, c, chunks, h->cs);
+    }
+    if (chunks > 1) forward_fc(h, replica, s, h->cs, true);
+    else forward(h, replica, s, h->cs, true);
     CK(cudaEventRecord(R.consumed[s], h->cs));
     R.consumed_valid[s] = true;
-    int32_t hc[2] = {0, 0};
-    float loss = 0.f;
-    CK(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, h->cs));
-    CK(cudaMemcpyAsync(&loss, R.loss, sizeof(float), cudaMemcpyDeviceToHost, h->cs));
-    CK(cudaStreamSynchronize(h->cs));
     CK(cudaGetLastError());
-    if (host_top1) *host_top1 = hc[0];
-    if (host_top5) *host_top5 = hc[1];
-    if (host_loss) *host_loss = loss;
-    return poll_status(h);
+    kn::HostResult res;
+    if (int rc = wait_result(h, &res)) return rc;
+    if (host_top1) *host_top1 = res.top1;
+    if (host_top5) *host_top5 = res.top5;
+    if (host_loss) *host_loss = res.loss;
+    return ALEXNET_OK;
 }
 
 int alexnet_replica_average(alexnet_t* h) {
@@ -1738,6 +1851,7 @@ int alexnet_run_op(alexnet_t* h, int replica, int op, int iters) {
     Replica& R = h->rep[replica];
     const int slot = R.last_slot;
     cudaStream_t st = h->cs;
+    h->loss_at_fork = false;      // SOFTMAX writes the loss
     for (int it = 0; it < iters; ++it) {
         if (op <= ALEXNET_OP_CONV5_FWD) op_conv_fwd(h, replica, op - ALEXNET_OP_CONV1_FWD, slot, st);
         else if (op <= ALEXNET_OP_CONV5_BWD_DATA) op_conv_bwd(h, replica, op - ALEXNET_OP_CONV2_BWD_DATA + 1, st);

@@ -64,15 +64,18 @@ __device__ __forceinline__ float normal_draw(uint64_t key, uint64_t idx) {
 // One block = one image and four rows of the 228-padded crop (one row `by` of the space-to-depth grid): the four source rows
 // of the uint8 image (768 bytes each) and of the mean image (768 floats each) come to shared memory in coalesced loads, then
 // thread (bx, dy) forms its 12 values (4 pixels x 3 colours) from there and stores 24 contiguous bytes; a warp writes 768
-// contiguous bytes.  grid: (57, B), 256 threads.
+// contiguous bytes.  grid: (57, images), 256 threads; image n0 + blockIdx.y of the batch.  labels_src != nullptr: the labels travel with
+// the images (from device or mapped host memory, four bytes per image: cheaper than a copy of their own in the stream).
 template <bool AUG>
 __global__ void __launch_bounds__(256) preprocess_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mean,
                                                          __nv_bfloat16* __restrict__ out, int32_t* __restrict__ cf_out,
-                                                         int B, uint64_t key, int eval_mode, const ColorAug aug) {
+                                                         const int32_t* __restrict__ labels_src, int32_t* __restrict__ labels_dst,
+                                                         int n0, uint64_t key, int eval_mode, const ColorAug aug) {
     pdl_sync();
     __shared__ uint4 s_img[4][49];        // rows padded by 16 bytes: the four rows start in different banks
     __shared__ float s_mean[4][769];      // row pitch = 1 mod 32 words: the warp's 8 bx x 4 dy reads (12 words apart per bx) hit 32 banks
-    const int by = blockIdx.x, n = blockIdx.y, tid = threadIdx.x;
+    const int by = blockIdx.x, n = n0 + blockIdx.y, tid = threadIdx.x;
+    if (labels_src && by == 0 && tid == 32) labels_dst[n] = labels_src[n];
     const uint64_t r = draw(key, (uint64_t)n);
     // evaluation: the centre 227 x 227 window, never flipped
     const int ox = eval_mode ? 14 : (int)((r & 0xFFFF) % 30), oy = eval_mode ? 14 : (int)(((r >> 16) & 0xFFFF) % 30);
@@ -835,15 +838,34 @@ __global__ void softmax_xent_kernel(const float* __restrict__ z, const int32_t* 
     }
     if (tid == 0) loss_n[n] = -(zr[lab] - mx - logf(sum));
 }
+// What a call that waits for the GPU reads: written by the last kernel of the call to mapped host memory, seq last, so that the
+// host polls one word instead of queueing copies behind the kernels (two copies, a synchronisation and a third
+// copy of the status word took 60 us of the 205 us of a one-image evaluation).
+struct HostResult { int32_t top1, top5; float loss; int32_t status; uint32_t seq; };
+__device__ __forceinline__ void publish_result(volatile HostResult* out, int top1, int top5, float loss, int status, uint32_t seq) {
+    out->top1 = top1; out->top5 = top5; out->loss = loss; out->status = status;
+    __threadfence_system();
+    out->seq = seq;
+}
+__global__ void store_result_kernel(const float* __restrict__ loss, const int* __restrict__ status, HostResult* out, uint32_t seq) {
+    pdl_sync();
+    publish_result(out, 0, 0, *loss, *(volatile const int*)status, seq);
+}
 // The training step's form of the three kernels fc_reduce_fwd (fc8), softmax_xent and mean in one launch: block n adds the
 // split-K partials of its row of logits in split order, adds the bias, stores z (fp32 logits), then softmax, loss_n and dz as
 // above; the block that finishes last (a counter in global memory, reset for the next launch) averages loss_n in index order,
 // so the result does not depend on which block that is.  Same arithmetic as the separate kernels.
+// EVAL: also counts the samples whose label is among the top 1 / top 5 logits (rank of the label = logits strictly greater than
+// it plus equal logits with a smaller class index; integer atomics, so the order does not matter) and the last block
+// publishes the counts, the loss and the status word.
+template <bool EVAL>
 __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __restrict__ ws, int splits, long long split_stride,
                                                                const float* __restrict__ bias, float* __restrict__ z,
                                                                const int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ dz,
                                                                float* __restrict__ loss_n, float* __restrict__ loss_mean,
-                                                               int* __restrict__ done_counter, int B, int N) {
+                                                               int* __restrict__ done_counter, int B, int N,
+                                                               int32_t* __restrict__ counts, const int* __restrict__ status,
+                                                               HostResult* host_out, uint32_t seq) {
     pdl_sync();
     __shared__ float red[32];
     __shared__ __align__(16) float zs[1024];
@@ -897,6 +919,21 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
         const float pj = expf(zs[j] - mx) * inv;
         dz[(size_t)n * N + j] = __float2bfloat16_rn((pj - (j == lab ? 1.f : 0.f)) * invB);
     }
+    if (EVAL) {
+        const float zl = zs[lab];
+        int c = 0;
+        for (int j = tid; j < N; j += 256) c += (zs[j] > zl) || (zs[j] == zl && j < lab);
+        const int rank = __reduce_add_sync(~0u, c);
+        __syncthreads();
+        if ((tid & 31) == 0) red[tid >> 5] = __int_as_float(rank);
+        __syncthreads();
+        if (tid == 0) {
+            int k = 0;
+            for (int w = 0; w < 8; ++w) k += __float_as_int(red[w]);
+            if (k < 1) atomicAdd(counts, 1);
+            if (k < 5) atomicAdd(counts + 1, 1);
+        }
+    }
     if (tid == 0) {
         loss_n[n] = -(zs[lab] - mx - logf(sum));
         __threadfence();
@@ -916,6 +953,10 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
         for (int w = 0; w < 8; ++w) t += red[w];
         *loss_mean = t / (float)B;
         *done_counter = 0;
+        if (EVAL) {
+            const int t1 = atomicExch(counts, 0), t5 = atomicExch(counts + 1, 0);      // zero again for the next call
+            publish_result(host_out, t1, t5, t / (float)B, *(volatile const int*)status, seq);
+        }
     }
 }
 // one float to wherever dst points (device memory, or pinned host memory mapped into the device's address space): the
@@ -923,7 +964,6 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
 __global__ void store_value_kernel(const float* __restrict__ src, float* __restrict__ dst) {
     pdl_sync();
     *dst = *src;
-    __threadfence_system();
 }
 __global__ void mean_kernel(const float* __restrict__ v, int n, float* __restrict__ out) {
     pdl_sync();
@@ -937,31 +977,6 @@ __global__ void mean_kernel(const float* __restrict__ v, int n, float* __restric
         float t = 0.f;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
         *out = t / (float)n;
-    }
-}
-
-// top-1 / top-5 counting: one block per sample.  rank of the label = logits strictly greater than it plus equal
-// logits with a smaller class index; the sample counts for top-k when rank < k.  counts[0] += top-1, counts[1] += top-5
-// (integer atomics: the result does not depend on the order).
-__global__ void topk_count_kernel(const float* __restrict__ z, const int32_t* __restrict__ labels, int N, int32_t* __restrict__ counts) {
-    pdl_sync();
-    __shared__ int red[32];
-    const int n = blockIdx.x, lab = labels[n];
-    const float* zr = z + (size_t)n * N;
-    const float zl = zr[lab];
-    int c = 0;
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
-        const float v = zr[j];
-        c += (v > zl) || (v == zl && j < lab);
-    }
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(~0u, c, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int rank = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) rank += red[w];
-        if (rank < 1) atomicAdd(counts, 1);
-        if (rank < 5) atomicAdd(counts + 1, 1);
     }
 }
 
