@@ -192,10 +192,6 @@ struct alexnet {
     cudaEvent_t ev_fork[kBranches] = {};   // the inputs of branch b are ready on the compute stream
     bool fc_grads_on_branches = false;     // the last backward pass ran the FC weight gradients on branches 0-2: ev_side_done[0..2]
                                            // then complete as soon as those gradients exist, long before the pass ends
-    // copies of losses (alexnet_loss_async) leave on a stream of their own as soon as the loss exists, beside the backward pass
-    cudaStream_t loss_stream = nullptr;
-    cudaEvent_t ev_loss_stored = nullptr;
-    bool loss_at_fork = false;             // the loss of the last pass exists at ev_fork[2] (that pass was forked)
     std::vector<cudaEvent_t> ev_chunk;     // the copy of chunk c of an evaluation batch is done
     kn::HostResult* host_result = nullptr; // mapped host memory: results of the calls that wait (one at a time per handle)
     uint32_t result_seq = 0;
@@ -1221,7 +1217,6 @@ void forward_backward(alexnet* h, int r, int slot, cudaStream_t st, bool update,
             cudaEventRecord(h->ev_side_done[b], h->side[b]);
             cudaStreamWaitEvent(st, h->ev_side_done[b], 0);
         }
-    h->loss_at_fork = used[2];
     h->fc_grads_on_branches = used[0] && used[1] && used[2] && !update;
     if (h->ev_backward_done) cudaEventRecord(h->ev_backward_done, st);
 }
@@ -1354,8 +1349,6 @@ void teardown(alexnet* h) {
         if (h->ev_fork[b]) cudaEventDestroy(h->ev_fork[b]);
     }
     for (cudaEvent_t e : h->prof_ev) cudaEventDestroy(e);
-    if (h->loss_stream) { cudaStreamSynchronize(h->loss_stream); cudaStreamDestroy(h->loss_stream); }
-    if (h->ev_loss_stored) cudaEventDestroy(h->ev_loss_stored);
     for (cudaEvent_t e : h->ev_chunk) cudaEventDestroy(e);
     if (h->host_result) cudaFreeHost(h->host_result);
     if (h->ev_backward_done) cudaEventDestroy(h->ev_backward_done);
@@ -1438,8 +1431,6 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
         CKC(cudaEventCreateWithFlags(&h->ev_fork[b], cudaEventDisableTiming));
     }
     CKC(cudaEventCreateWithFlags(&h->ev_backward_done, cudaEventDisableTiming));
-    CKC(cudaStreamCreateWithFlags(&h->loss_stream, cudaStreamNonBlocking));
-    CKC(cudaEventCreateWithFlags(&h->ev_loss_stored, cudaEventDisableTiming));
     CKC(cudaHostAlloc((void**)&h->host_result, sizeof(kn::HostResult), cudaHostAllocMapped | cudaHostAllocPortable));
     memset((void*)h->host_result, 0, sizeof(kn::HostResult));
     // pad positions of every grid must be zero from the start; gradients and momentum start at zero
@@ -1486,9 +1477,8 @@ int alexnet_load_batch_async(alexnet_t* h, int replica, const uint8_t* images, c
     const int s = R.next_load;
     if (R.consumed_valid[s]) CK(cudaStreamWaitEvent(h->ls, R.consumed[s], 0));
     CK(cudaMemcpyAsync(R.stage[s], images, (size_t)h->B * 196608, cudaMemcpyDefault, h->ls));
-    const int32_t* lsrc = label_source(labels);
-    if (!lsrc) CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
-    op_preprocess(h, replica, s, step, h->ls, false, lsrc);
+    CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
+    op_preprocess(h, replica, s, step, h->ls);
     CK(cudaEventRecord(R.ready[s], h->ls));
     R.slot_step[s] = step;
     R.last_slot = s; R.next_load ^= 1; R.loaded++;
@@ -1649,17 +1639,8 @@ int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out) {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, loss_out) == cudaSuccess && at.devicePointer != nullptr &&
         (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)) {
-        // A store to host memory takes 7-13 us beside a batch upload.  The loss exists since before the backward pass, so the store
-        // runs there, on a stream of its own, and the compute stream only waits for its (long past) end.
-        const bool early = h->loss_at_fork;
-        cudaStream_t st = early ? h->loss_stream : h->cs;
-        if (early) CK(cudaStreamWaitEvent(st, h->ev_fork[2], 0));
-        launch_k(kn::store_value_kernel, 1, 1, 0, st, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
+        launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
         h->launches++;
-        if (early) {
-            CK(cudaEventRecord(h->ev_loss_stored, st));
-            CK(cudaStreamWaitEvent(h->cs, h->ev_loss_stored, 0));
-        }
         CK(cudaGetLastError());
         return ALEXNET_OK;
     }
@@ -1681,7 +1662,6 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     if (!lsrc) CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
     R.slot_step[s] = 0; R.last_slot = s;
     ++h->result_seq;
-    h->loss_at_fork = false;
     // the copies run on the copy stream, everything else (preprocessing too) on the compute stream
     cudaPointerAttributes at{};
     const bool on_device = cudaPointerGetAttributes(&at, images) == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
@@ -1851,7 +1831,6 @@ int alexnet_run_op(alexnet_t* h, int replica, int op, int iters) {
     Replica& R = h->rep[replica];
     const int slot = R.last_slot;
     cudaStream_t st = h->cs;
-    h->loss_at_fork = false;      // SOFTMAX writes the loss
     for (int it = 0; it < iters; ++it) {
         if (op <= ALEXNET_OP_CONV5_FWD) op_conv_fwd(h, replica, op - ALEXNET_OP_CONV1_FWD, slot, st);
         else if (op <= ALEXNET_OP_CONV5_BWD_DATA) op_conv_bwd(h, replica, op - ALEXNET_OP_CONV2_BWD_DATA + 1, st);

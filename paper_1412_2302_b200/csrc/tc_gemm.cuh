@@ -344,52 +344,69 @@ __device__ __forceinline__ void epi_chunk(const P& p, uint32_t* v, bool zero, bo
 // tensor are clipped by TMA.  Each epilogue warp owns one kEpiStageBytes tile: before rewriting it the warp waits
 // until the previous store has finished reading it (wait_group.read 0), which the TMEM loads and the arithmetic of
 // the next slab overlap.
+// An SM has only four or eight epilogue warps, so a slab is a latency chain and not a throughput problem: all its TMEM
+// columns are read before the first wait, with the bias of the first half in flight beside them, pairs of columns are
+// added as packed fp32, and one conversion instruction applies the ReLU and packs.  The ReLU mask of a backward slab is
+// fetched by the caller one slab ahead.
 constexpr uint32_t kEpiStageBytes = 4096;
+__device__ __forceinline__ uint32_t cvt_relu_bf16x2(float lo, float hi) {
+    uint32_t d; asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo)); return d;
+}
+__device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
+    uint32_t d; asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo)); return d;
+}
+// the 128 bytes of the ReLU mask under a lane's row of a slab; mp == nullptr: a row outside the tensor
+__device__ __forceinline__ void epi_mask_load(const uint4* mp, uint4* mk) {
+    #pragma unroll
+    for (int q = 0; q < 8; ++q) mk[q] = mp ? __ldg(mp + q) : make_uint4(0u, 0u, 0u, 0u);
+}
 template <typename P>
-__device__ __forceinline__ void epi_slab(const P& p, uint32_t tmem_addr, bool pad_row, long long row_off, int col0, int g,
+__device__ __forceinline__ void epi_slab(const P& p, uint32_t tmem_addr, bool pad_row, int col0, int g, uint4* mk, const uint4* next_mask,
                                          int x, int y, int z, uint32_t stage, int lane) {
     uint32_t w[32];   // the packed 128-byte row
     if (p.epi == EPI_F32) {
         tmem_ld32(tmem_addr, w);
         tmem_ld_wait();
     } else {
-        const float* bp = p.bias ? p.bias + g * p.out_gx + col0 : nullptr;
-        const uint4* mp = p.mask ? (const uint4*)(p.mask + row_off + col0) : nullptr;
+        uint32_t v[64];
+        tmem_ld32(tmem_addr, v);
+        tmem_ld32(tmem_addr + 32u, v + 32);
+        const float4* bp = p.bias ? (const float4*)(p.bias + g * p.out_gx + col0) : nullptr;
+        float4 b[8];
+        if (bp) {
+            #pragma unroll
+            for (int q = 0; q < 8; ++q) b[q] = __ldg(bp + q);
+        }
+        tmem_ld_wait();
         #pragma unroll
         for (int half = 0; half < 2; ++half) {
-            uint32_t v[32];
-            tmem_ld32(tmem_addr + 32u * half, v);
-            tmem_ld_wait();
-            #pragma unroll
-            for (int qq = 0; qq < 4; ++qq) {       // four 16-byte chunks of eight columns
-                const int q = 4 * half + qq;
-                float f[8];
+            if (bp) {
                 #pragma unroll
-                for (int k = 0; k < 8; ++k) f[k] = __uint_as_float(v[8 * qq + k]);
-                if (bp) {
-                    const float4 b0 = __ldg((const float4*)(bp + 8 * q)), b1 = __ldg((const float4*)(bp + 8 * q + 4));
-                    f[0] += b0.x; f[1] += b0.y; f[2] += b0.z; f[3] += b0.w; f[4] += b1.x; f[5] += b1.y; f[6] += b1.z; f[7] += b1.w;
-                }
-                if (p.relu) {
+                for (int q = 0; q < 8; ++q) {
+                    uint32_t* u = v + 32 * half + 4 * q;
+                    float f[4];
+                    kn::un2(kn::add2(kn::mk2(__uint_as_float(u[0]), __uint_as_float(u[1])), kn::mk2(b[q].x, b[q].y)), f[0], f[1]);
+                    kn::un2(kn::add2(kn::mk2(__uint_as_float(u[2]), __uint_as_float(u[3])), kn::mk2(b[q].z, b[q].w)), f[2], f[3]);
                     #pragma unroll
-                    for (int k = 0; k < 8; ++k) f[k] = fmaxf(f[k], 0.f);
-                }
-                if (mp) {
-                    const uint4 mv = __ldg(mp + q);
-                    const __nv_bfloat162* mh = (const __nv_bfloat162*)&mv;
-                    #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float2 m2 = __bfloat1622float2(mh[k]);
-                        f[2 * k] = m2.x > 0.f ? f[2 * k] * p.mask_scale : 0.f;
-                        f[2 * k + 1] = m2.y > 0.f ? f[2 * k + 1] * p.mask_scale : 0.f;
-                    }
-                }
-                #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    __nv_bfloat162 hh = __floats2bfloat162_rn(pad_row ? 0.f : f[2 * k], pad_row ? 0.f : f[2 * k + 1]);
-                    w[4 * q + k] = *(uint32_t*)&hh;
+                    for (int k = 0; k < 4; ++k) u[k] = __float_as_uint(f[k]);
+                    if (half == 0) b[q] = __ldg(bp + 8 + q);
                 }
             }
+            #pragma unroll
+            for (int k = 16 * half; k < 16 * half + 16; ++k) {
+                const float lo = __uint_as_float(v[2 * k]), hi = __uint_as_float(v[2 * k + 1]);
+                w[k] = p.relu ? cvt_relu_bf16x2(lo, hi) : cvt_bf16x2(lo, hi);
+            }
+        }
+        if (mk) {      // a masked value is kept or zero (mask_scale is 1 in every layer that stores bf16 this way)
+            const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f);
+            #pragma unroll
+            for (int k = 0; k < 32; ++k) w[k] &= __hgt2_mask(((const __nv_bfloat162*)mk)[k], zero2);
+            epi_mask_load(next_mask, mk);
+        }
+        if (pad_row) {
+            #pragma unroll
+            for (int k = 0; k < 32; ++k) w[k] = 0u;
         }
     }
     if (lane == 0) bulk_wait_read_0();
@@ -608,7 +625,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
             if (p.tma_store) {
                 const int slab = p.epi == EPI_F32 ? 32 : 64;
                 for (int c = 0; c < p.BN; c += slab) {
-                    epi_slab(p, t0 + (uint32_t)c, pad_row, row_off, n0 + c, g, g * p.out_gx * (p.mode != MODE_MNMN) + n0 + c,
+                    epi_slab(p, t0 + (uint32_t)c, pad_row, n0 + c, g, nullptr, nullptr, g * p.out_gx * (p.mode != MODE_MNMN) + n0 + c,
                              m0 + quad * 32 + (p.mode == MODE_MNMN ? g * p.out_gx : 0), tc.z,
                              epi_stage0 + (uint32_t)quad * kEpiStageBytes, lane);
                 }
@@ -984,15 +1001,41 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             const int m0 = tc.m_tile * tile_rows + row0, n0 = tc.n_tile * BN, g = tc.g;
             const int a_begin = tc.z * per;
             const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
+            // with two sets of epilogue warps, the (row half, slab) units of the tile alternate between the sets
+            const bool staged = p.tma_store && !zc;
+            const int slab = p.epi == EPI_F32 ? 32 : 64, nslab = (BN + slab - 1) / slab, units = MH * nslab, first = E == 2 ? eset : 0;
+            uint4 mk[8];
+            if (staged && p.mask && first < units) {
+                const int row = m0 + (first / nslab) * 128 + r;
+                epi_mask_load(row < p.M_total ? (const uint4*)(p.mask + (long long)row * p.ldo + g * p.out_gx + n0 + (first % nslab) * slab) : nullptr, mk);
+            }
             TL(const long long ce0 = clock64();)
             ok = mbar_wait(accf0 + 8u * ab, aph, abort_flag);
             TL(if (ew == 0 && lane == 0) tl[8] += clock64() - ce0;)
             if (!ok) break;
             tc_fence_after();
-            // with two sets of epilogue warps, the (row half, slab) units of the tile alternate between the sets
+            if (staged) {
+                #pragma unroll 1
+                for (int u = first; u < units; u += E) {
+                    const int h = u / nslab, c = (u - h * nslab) * slab, row = m0 + h * 128 + r;
+                    bool pad_row = false;
+                    if (p.Hp > 0) {
+                        const int x = row % p.Wp, y = (row / p.Wp) % p.Hp;
+                        pad_row = (x >= p.W) || (y >= p.H);
+                    }
+                    const uint4* next = nullptr;
+                    if (p.mask && u + E < units) {
+                        const int h2 = (u + E) / nslab, row2 = m0 + h2 * 128 + r;
+                        if (row2 < p.M_total) next = (const uint4*)(p.mask + (long long)row2 * p.ldo + g * p.out_gx + n0 + (u + E - h2 * nslab) * slab);
+                    }
+                    epi_slab(p, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * acc_cols + h * BN + c), pad_row, n0 + c, g,
+                             p.mask ? mk : nullptr, next, g * p.out_gx + n0 + c, m0 + h * 128 + quad * 32, tc.z,
+                             epi_stage0 + (uint32_t)ew * kEpiStageBytes, lane);
+                }
+            }
             int unit = 0;
             #pragma unroll 1
-            for (int h = 0; h < MH; ++h) {
+            for (int h = 0; h < MH && !staged; ++h) {
                 const int row = m0 + h * 128 + r;
                 const bool row_ok = row < p.M_total;
                 bool pad_row = false;
@@ -1012,13 +1055,6 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                         const uint32_t rowp = ring_a + (uint32_t)(r * kZcPitch + c) * 4u;
                         #pragma unroll
                         for (int q = 0; q < 8; ++q) st_shared_v4(rowp + 16u * q, v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                    }
-                } else if (p.tma_store) {
-                    const int slab = p.epi == EPI_F32 ? 32 : 64;
-                    for (int c = 0; c < BN; c += slab, ++unit) {
-                        if (E == 2 && (unit & 1) != eset) continue;
-                        epi_slab(p, t0 + (uint32_t)c, pad_row, row_off, n0 + c, g, g * p.out_gx + n0 + c, m0 + h * 128 + quad * 32,
-                                 tc.z, epi_stage0 + (uint32_t)ew * kEpiStageBytes, lane);
                     }
                 } else {
                     for (int c = 0; c < BN; c += 16, ++unit) {
