@@ -183,15 +183,20 @@ struct alexnet {
     Layout L;
     int B;
     cudaStream_t cs, ls;   // compute, loader
-    // The independent branches of the backward pass - the weight gradient (+ update) of FC layer l (branch l) and the weight
-    // gradient + split reduction of conv layer l (branch 3 + l) - each run on a stream of their own (owned by the handle),
-    // forked from the compute stream when their inputs exist and joined before the update.
-    static const int kBranches = 8;
-    cudaStream_t side[kBranches] = {};
-    cudaEvent_t ev_side_done[kBranches] = {};
-    cudaEvent_t ev_fork[kBranches] = {};   // the inputs of branch b are ready on the compute stream
-    bool fc_grads_on_branches = false;     // the last backward pass ran the FC weight gradients on branches 0-2: ev_side_done[0..2]
-                                           // then complete as soon as those gradients exist, long before the pass ends
+    // The independent branches of the backward pass run on streams of the handle, forked from the compute stream when their inputs
+    // exist and joined before the update: the FC weight gradients (+ update) on side[0], the conv weight gradients on
+    // side[1] and side[2] in turn, so that one can fill the SMs that the tail of another leaves.
+    // No more than that: with the caller's streams and the default stream the process stays within the eight hardware queues of
+    // a context.  With a stream per branch (eight) some of them shared a queue with one another or with the copy stream and
+    // waited for work they do not depend on: 430 against 411 us per step at batch 8, 527 against 510 at 32, larger batches alike.
+    static const int kSides = 3;
+    cudaStream_t side[kSides] = {};
+    cudaEvent_t ev_side_done[kSides] = {};
+    static const int kForks = 9;           // fork points of a pass: FC layers 0-2, conv layers 3-7, fc8's bias 8
+    cudaEvent_t ev_fork[kForks] = {};
+    cudaEvent_t ev_fc_grads = nullptr;     // side[0]: the FC weight gradients are stored
+    bool fc_grads_on_branches = false;     // the last backward pass ran the FC weight gradients on side[0]: ev_fc_grads
+                                           // then completes as soon as those gradients exist, long before the pass ends
     std::vector<cudaEvent_t> ev_chunk;     // the copy of chunk c of an evaluation batch is done
     kn::HostResult* host_result = nullptr; // mapped host memory: results of the calls that wait (one at a time per handle)
     uint32_t result_seq = 0;
@@ -1188,36 +1193,36 @@ void forward_backward(alexnet* h, int r, int slot, cudaStream_t st, bool update,
     // tensor-bound work; each branch has its own region of the split workspace and of the bias partials.  `st` joins all
     // branches before it returns.  Per-kernel profiling keeps everything on one stream.
     const bool fork = h->side[0] != nullptr && !h->prof;
-    bool used[alexnet::kBranches] = {};
-    auto branch = [&](int b) -> cudaStream_t {       // fork branch b from `st` here
+    bool used[alexnet::kSides] = {};
+    auto branch = [&](int f, int side) -> cudaStream_t {       // fork point f: stream `side` goes on from here
         if (!fork) return st;
-        cudaEventRecord(h->ev_fork[b], st);
-        cudaStreamWaitEvent(h->side[b], h->ev_fork[b], 0);
-        used[b] = true;
-        return h->side[b];
+        cudaEventRecord(h->ev_fork[f], st);
+        cudaStreamWaitEvent(h->side[side], h->ev_fork[f], 0);
+        used[side] = true;
+        return h->side[side];
     };
     // the data gradient reads the layer's weights, so it comes first when the weight-gradient kernel updates them in place
     for (int l = 2; l >= 0; --l) {
         if (update) op_fc_bwd(h, r, l, st);
-        op_fc_wg(h, r, l, update, branch(l));
+        op_fc_wg(h, r, l, update, branch(l, 0));
         if (!update) op_fc_bwd(h, r, l, st);
-        if (l == 2) op_fc_bias(h, r, l, branch(3));
+        if (l == 2) op_fc_bias(h, r, l, branch(8, 2));
     }
+    if (fork) cudaEventRecord(h->ev_fc_grads, h->side[0]);
     op_pool_bwd(h, r, 2, st);
     // (the transposed bf16 filters that the data gradients read are written between steps only: they may load early)
-    op_conv_wg(h, r, 4, slot, branch(3 + 4), !defer_conv_reduce); op_conv_bwd(h, r, 4, st, true, update && fork);
-    op_conv_wg(h, r, 3, slot, branch(3 + 3), !defer_conv_reduce); op_conv_bwd(h, r, 3, st, true, update && fork);
-    op_conv_wg(h, r, 2, slot, branch(3 + 2), !defer_conv_reduce); op_conv_bwd(h, r, 2, st, true, update && fork);
-    op_pool_lrn_bwd(h, r, 1, st);
-    op_conv_wg(h, r, 1, slot, branch(3 + 1), !defer_conv_reduce); op_conv_bwd(h, r, 1, st, true);
-    op_pool_lrn_bwd(h, r, 0, st);
-    op_conv_wg(h, r, 0, slot, branch(3 + 0), !defer_conv_reduce);
-    for (int b = 0; b < alexnet::kBranches; ++b)
+    for (int l = 4; l >= 0; --l) {
+        op_conv_wg(h, r, l, slot, branch(3 + l, 1 + l % 2), !defer_conv_reduce);
+        if (l == 0) break;
+        op_conv_bwd(h, r, l, st, true, update && fork && l >= 2);
+        if (l <= 2) op_pool_lrn_bwd(h, r, l - 1, st);
+    }
+    for (int b = 0; b < alexnet::kSides; ++b)
         if (used[b]) {
             cudaEventRecord(h->ev_side_done[b], h->side[b]);
             cudaStreamWaitEvent(st, h->ev_side_done[b], 0);
         }
-    h->fc_grads_on_branches = used[0] && used[1] && used[2] && !update;
+    h->fc_grads_on_branches = used[0] && !update;
     if (h->ev_backward_done) cudaEventRecord(h->ev_backward_done, st);
 }
 
@@ -1343,11 +1348,13 @@ inline uint16_t f2bf(float f) {
 // everything the handle owns: streams, events (null where never created); shared by alexnet_destroy and the failure paths
 // of alexnet_create
 void teardown(alexnet* h) {
-    for (int b = 0; b < alexnet::kBranches; ++b) {
+    for (int b = 0; b < alexnet::kSides; ++b) {
         if (h->side[b]) { cudaStreamSynchronize(h->side[b]); cudaStreamDestroy(h->side[b]); }
         if (h->ev_side_done[b]) cudaEventDestroy(h->ev_side_done[b]);
-        if (h->ev_fork[b]) cudaEventDestroy(h->ev_fork[b]);
     }
+    for (cudaEvent_t e : h->ev_fork)
+        if (e) cudaEventDestroy(e);
+    if (h->ev_fc_grads) cudaEventDestroy(h->ev_fc_grads);
     for (cudaEvent_t e : h->prof_ev) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_chunk) cudaEventDestroy(e);
     if (h->host_result) cudaFreeHost(h->host_result);
@@ -1421,15 +1428,16 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
         CKC(cudaGetDevice(&dev));
         CKC(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
     }
-    // The FC updates (branches 0-2) are the longest work beside the chain and need few SMs: their streams go first, so that
-    // they start as soon as their inputs exist instead of behind the chain's queue (batch 8: 440 -> 430 us per step).
+    // The FC updates are the longest work beside the chain and need few SMs: their stream goes first, so that they start as soon as
+    // their inputs exist instead of behind the chain's queue (batch 8: 440 -> 430 us per step).
     int prio_low = 0, prio_high = 0;
     CKC(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
-    for (int b = 0; b < alexnet::kBranches; ++b) {
-        CKC(cudaStreamCreateWithPriority(&h->side[b], cudaStreamNonBlocking, b < 3 ? std::max(prio_high, -2) : 0));
+    for (int b = 0; b < alexnet::kSides; ++b) {
+        CKC(cudaStreamCreateWithPriority(&h->side[b], cudaStreamNonBlocking, b == 0 ? std::max(prio_high, -2) : 0));
         CKC(cudaEventCreateWithFlags(&h->ev_side_done[b], cudaEventDisableTiming));
-        CKC(cudaEventCreateWithFlags(&h->ev_fork[b], cudaEventDisableTiming));
     }
+    for (cudaEvent_t& e : h->ev_fork) CKC(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    CKC(cudaEventCreateWithFlags(&h->ev_fc_grads, cudaEventDisableTiming));
     CKC(cudaEventCreateWithFlags(&h->ev_backward_done, cudaEventDisableTiming));
     CKC(cudaHostAlloc((void**)&h->host_result, sizeof(kn::HostResult), cudaHostAllocMapped | cudaHostAllocPortable));
     memset((void*)h->host_result, 0, sizeof(kn::HostResult));
@@ -1571,7 +1579,7 @@ int alexnet_stream_wait_fc_gradients(alexnet_t* h, void* stream) {
     if (int rc = check_status(h)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     if (h->fc_grads_on_branches) {
-        for (int b = 0; b < 3; ++b) CK(cudaStreamWaitEvent(st, h->ev_side_done[b], 0));
+        CK(cudaStreamWaitEvent(st, h->ev_fc_grads, 0));
     } else {
         CK(cudaStreamWaitEvent(st, h->ev_backward_done, 0));
     }
