@@ -383,7 +383,8 @@ int make_tm_rows(alexnet* h, CUtensorMap* tm, const void* ptr, bool f32, uint64_
 
 void finish_plan(const alexnet* h, Plan& P) {
     tc::GemmParams& p = P.p;
-    const int stage_bytes = tc::kABytes + tc::b_stage_bytes(p.mode, p.BN);
+    if (p.a_bytes == 0) p.a_bytes = tc::kABytes;
+    const int stage_bytes = p.a_bytes + tc::b_stage_bytes(p.mode, p.BN);
     int stages = (227 * 1024 - 2048 - 4 * (int)tc::kEpiStageBytes) / stage_bytes;
     if (stages > tc::kMaxStages) stages = tc::kMaxStages;
     p.stages = stages;
@@ -392,7 +393,7 @@ void finish_plan(const alexnet* h, Plan& P) {
     p.splits = (p.steps_total + per - 1) / per;
     p.steps_per_split = per;
     p.tiles_total = p.m_tiles * p.n_tiles * p.groups * p.taps_grid * p.splits;
-    P.smem = tc::smem_bytes(p.mode, p.BN, stages);
+    P.smem = tc::smem_bytes(stage_bytes, stages);
     P.grid = std::min(p.tiles_total, h->sm_count);   // persistent: one CTA per SM walks the tile list
     P.valid = true;
 }
@@ -582,6 +583,7 @@ int plan_conv_wg(alexnet* h, Plan& P, int l, const ConvL& c, const bf16* dy, con
     P.valid = true;
     return ALEXNET_OK;
 }
+uint32_t fc_box_rows(int B) { return (uint32_t)std::min(128, (B + 7) / 8 * 8); }
 int plan_fc_fwd(alexnet* h, Plan& P, const FcL& f, const bf16* x, const bf16* wsh, const float* bias, bool with_epilogue) {
     memset(&P, 0, sizeof(P));
     tc::ConvParams& p = P.c;
@@ -592,12 +594,15 @@ int plan_fc_fwd(alexnet* h, Plan& P, const FcL& f, const bf16* x, const bf16* ws
     p.M_total = B; p.m_tiles = (B + 127) / 128; p.n_tiles = (f.N + p.BN - 1) / p.BN;
     p.groups = 1; p.splits = fc_fwd_splits(f, B);
     p.asteps_total = p.chunks;
-    p.a_box_rows = 128;
-    p.halo_shift[0] = 0; p.tap_off[0] = 0; p.tap_off[1] = 128;   // the second chunk's box follows the first in the stage
+    // The activation boxes hold the batch's rows and no more (whole 8-row swizzle groups): the instructions read 128 rows all the
+    // same, but what lies under the rows past the batch never reaches an output, and the shared memory that a small batch
+    // leaves goes to more weight stages in flight.
+    p.a_box_rows = fc_box_rows(B);
+    p.halo_shift[0] = 0; p.tap_off[0] = 0; p.tap_off[1] = p.a_box_rows;   // the second chunk's box follows the first in the stage
     p.epi = tc::EPI_F32; p.n_valid = f.N; p.ldo = f.N; p.split_stride = (long long)B * f.N;
     p.mask_scale = 1.f; p.out = h->ws; p.status = h->status;
     int rc;
-    if ((rc = make_tm(h, &p.tmA, x, f.K, B, (uint64_t)f.K * 2, 128))) return rc;
+    if ((rc = make_tm(h, &p.tmA, x, f.K, B, (uint64_t)f.K * 2, p.a_box_rows))) return rc;
     if ((rc = make_tm(h, &p.tmB, wsh, f.K, f.N, (uint64_t)f.K * 2, p.BN))) return rc;
     p.tma_store = 1;
     if ((rc = make_tm_out(h, &p.tmOut, h->ws, true, (uint64_t)f.N, (uint64_t)B, (uint64_t)p.splits, (uint64_t)f.N * 4,
@@ -626,7 +631,8 @@ int plan_fc_bwd(alexnet* h, Plan& P, const FcL& f, const bf16* dy, const bf16* w
     p.n_valid = f.K; p.ldo = f.K; p.split_stride = (long long)B * f.K;
     p.out = h->ws; p.status = h->status;
     int rc;
-    if ((rc = make_tm(h, &p.tmA, dy, f.N, B, (uint64_t)f.N * 2, 128))) return rc;
+    p.a_bytes = fc_box_rows(B) * 128;      // (see plan_fc_fwd)
+    if ((rc = make_tm(h, &p.tmA, dy, f.N, B, (uint64_t)f.N * 2, fc_box_rows(B)))) return rc;
     if ((rc = make_tm(h, &p.tmB, wsh, f.K, f.N, (uint64_t)f.K * 2, 64))) return rc;
     p.tma_store = 1;
     if ((rc = make_tm_out(h, &p.tmOut, h->ws, true, (uint64_t)f.K, (uint64_t)B, (uint64_t)p.splits, (uint64_t)f.K * 4,
@@ -690,7 +696,9 @@ void plan_fc_chain(alexnet* h, int r) {
         if (!R.fc_fwd[l].valid || c.m_tiles != 1 || c.BN != 128 || c.cpg != 2 || c.kk != 4 || c.kh != 1 || c.tiles_total != grid ||
             c.n_valid % 4 || (l < 2 ? c.zcluster != tc::kChainCluster : c.zcluster != 0)) return;
         tc::FcChainLayer& y = q.L[l];
-        y.tmA = c.tmA; y.tmB = c.tmB;
+        const bf16* xs[3] = {R.p5, R.f6, R.f7};
+        if (make_tm(h, &y.tmA, xs[l], f.K, h->B, (uint64_t)f.K * 2, 128)) return;
+        y.tmB = c.tmB;
         y.n_tiles = c.n_tiles; y.splits = c.splits; y.per = c.asteps_per_split; y.asteps_total = c.asteps_total; y.n_valid = c.n_valid;
         y.cluster_reduce = l < 2;
         y.relu = l < 2; y.bias = R.w + f.b_off; y.out = outs[l]; y.keep = keeps[l];

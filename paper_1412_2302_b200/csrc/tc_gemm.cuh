@@ -64,6 +64,7 @@ struct GemmParams {
     int steps_total;   // k-steps over the whole reduction (split evenly over `splits`)
     int steps_per_split;
     int stages;        // smem ring depth
+    int a_bytes;       // A part of a stage: kABytes, or less when a K-major A has fewer than 128 rows (a multiple of 1024)
     int a_x0, a_gx;    // A column origin and per-group column stride
     int b_gx;          // MODE_MNMN: B per-group column stride
     int b_tap_rows, b_g_rows;  // MODE_KK: B row = tap*b_tap_rows + g*b_g_rows + n0
@@ -441,9 +442,7 @@ constexpr int kABytes = 128 * 128;  // 128 rows x 64 bf16, or 2 boxes of 64 x 64
 __host__ __device__ inline int b_stage_bytes(int mode, int BN) {
     return mode == MODE_KK ? BN * 128 : ((BN + 63) / 64) * 8192;
 }
-inline size_t smem_bytes(int mode, int BN, int stages) {
-    return 1024 + (size_t)stages * (kABytes + b_stage_bytes(mode, BN)) + 4 * kEpiStageBytes + 512;
-}
+inline size_t smem_bytes(int stage_bytes, int stages) { return 1024 + (size_t)stages * stage_bytes + 4 * kEpiStageBytes + 512; }
 
 // position of a CTA in the tile list; tiles are numbered with m fastest, then
 // n tile, group, tap (weight gradients), k split
@@ -477,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const int bbytes = b_stage_bytes(p.mode, p.BN);
-    const int stage_bytes = kABytes + bbytes;
+    const int stage_bytes = p.a_bytes + bbytes;
     const int stages = p.stages;
     // epilogue staging (4 warps x kEpiStageBytes), then barriers: full[8] @0, empty[8] @64, acc_full[2] @128,
     // acc_empty[2] @144, tmem slot @160, abort flag @168
@@ -530,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                         const uint32_t sa = base + st * stage_bytes, fb = full0 + 8u * st;
                         mbar_expect_tx(fb, tx);
                         tma_load_2d(sa, &p.tmA, xa + ch * 64, m0 + p.shift[tap], fb);
-                        tma_load_2d(sa + kABytes, &p.tmB, ch * 64, tap * p.b_tap_rows + yb, fb);
+                        tma_load_2d(sa + p.a_bytes, &p.tmB, ch * 64, tap * p.b_tap_rows + yb, fb);
                         if (++ch == p.chunks) { ch = 0; ++tap; }
                         if (++st == stages) { st = 0; ph ^= 1u; }
                     }
@@ -541,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                         const int q = (s_begin + i) * 64;
                         mbar_expect_tx(fb, tx);
                         tma_load_2d(sa, &p.tmA, q, m0, fb);
-                        for (int j = 0; j < nb; ++j) tma_load_2d(sa + kABytes + j * 8192, &p.tmB, n0 + 64 * j, q, fb);
+                        for (int j = 0; j < nb; ++j) tma_load_2d(sa + p.a_bytes + j * 8192, &p.tmB, n0 + 64 * j, q, fb);
                         if (++st == stages) { st = 0; ph ^= 1u; }
                     }
                 } else {
@@ -553,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                         mbar_expect_tx(fb, tx);
                         tma_load_2d(sa, &p.tmA, xa, q, fb);
                         tma_load_2d(sa + 8192, &p.tmA, xa + 64, q, fb);
-                        for (int j = 0; j < nb; ++j) tma_load_2d(sa + kABytes + j * 8192, &p.tmB, xb + 64 * j, q + sh, fb);
+                        for (int j = 0; j < nb; ++j) tma_load_2d(sa + p.a_bytes + j * 8192, &p.tmB, xb + 64 * j, q + sh, fb);
                         if (++st == stages) { st = 0; ph ^= 1u; }
                     }
                 }
@@ -580,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                 for (int i = 0; i < nsteps; ++i) {
                     if (!(ok = mbar_wait_warp(full0 + 8u * st, ph, abort_flag))) break;
                     tc_fence_after();
-                    const uint32_t sa = base + st * stage_bytes, sb = sa + kABytes;
+                    const uint32_t sa = base + st * stage_bytes, sb = sa + p.a_bytes;
                     #pragma unroll 4
                     for (int j = 0; j < kk; ++j)
                         umma(d, smem_desc(sa + j * a_adv, a_lbo, 1024), smem_desc(sb + j * b_adv, b_lbo, 1024),
