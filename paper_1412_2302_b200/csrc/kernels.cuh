@@ -466,17 +466,20 @@ struct PoolLrnBwdGeo {
     static constexpr int HALO = CPR == 32 ? 0 : 1, PER = 32 - 2 * HALO, NP = (WI + 1) / 2, NJ = (HI + 1) / 2;
     static constexpr int TOT = NJ * NP * CPR, WARPS = (TOT + PER - 1) / PER, BLOCKS = (WARPS + 3) / 4;
 };
-// the eight gradients of a window where its argmax equals the tap, as fp32
-__device__ __forceinline__ void tap_select(const uint4& g, const uint2& ab, uint32_t tap, float* f) {
+// the eight gradients of a window where its argmax equals the tap, else zero (four words of two bf16 channels)
+__device__ __forceinline__ void tap_words(const uint4& g, const uint2& ab, uint32_t tap, uint32_t* v) {
     const uint32_t T = tap * 0x01010101u;
     const uint32_t m0 = (ab.x ^ T) + 0x7f7f7f7fu, m1 = (ab.y ^ T) + 0x7f7f7f7fu;      // sign bit of a byte: not this tap (bytes are < 16)
     const uint32_t w[4] = {g.x, g.y, g.z, g.w};
     #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const uint32_t m = i < 2 ? m0 : m1;
-        const uint32_t v = w[i] & ~prmt(m, m, (i & 1) ? 0xbbaau : 0x9988u);          // sign-replicated bytes
-        f[2 * i] = bf_lo(v); f[2 * i + 1] = bf_hi(v);
+        v[i] = w[i] & ~prmt(m, m, (i & 1) ? 0xbbaau : 0x9988u);          // sign-replicated bytes
     }
+}
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 r = __hadd2(*(const __nv_bfloat162*)&a, *(const __nv_bfloat162*)&b);
+    return *(const uint32_t*)&r;
 }
 template <int CPR, int WI, int HI, bool B75>
 __global__ void __launch_bounds__(128, 5) pool_lrn_bwd_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ dp,
@@ -510,30 +513,33 @@ __global__ void __launch_bounds__(128, 5) pool_lrn_bwd_kernel(const __nv_bfloat1
     const f2 al2 = mk2(alpha, alpha), k2 = mk2(k, k), mc2 = mk2(-2.f * alpha * beta, -2.f * alpha * beta);
     #pragma unroll
     for (int r = 0; r < 2; ++r) {
+        // dn of the row's even and odd pixel, two channels per word.  Three of the four pixels of a block get one or two terms: a
+        // packed bf16 sum is then the fp32 sum rounded to bf16 (exact, or its smaller term is far below half a unit in the last
+        // place); only the pixel of four windows adds in fp32.
         f2 g[8];
         {
-            float e0[8], o0[8], t[8];
+            uint32_t e[4], o[4], t[4];
+            tap_words(wd[0][0], wa[0][0], 3 * r, e);             // window (j, i): taps (r, 0) and (r, 1)
+            tap_words(wd[0][0], wa[0][0], 3 * r + 1, o);
+            tap_words(wd[0][1], wa[0][1], 3 * r + 2, t);         // window (j, i-1): tap (r, 2) on the even pixel
             if (r == 0) {                                        // windows of row j-1: their last filter row
-                tap_select(wd[1][0], wa[1][0], 6, e0);
-                tap_select(wd[1][0], wa[1][0], 7, o0);
-                tap_select(wd[1][1], wa[1][1], 8, t);
+                uint32_t a6[4], a7[4], a8[4];
+                tap_words(wd[1][0], wa[1][0], 6, a6);
+                tap_words(wd[1][0], wa[1][0], 7, a7);
+                tap_words(wd[1][1], wa[1][1], 8, a8);
                 #pragma unroll
-                for (int c = 0; c < 8; ++c) g[c] = mk2(e0[c] + t[c], o0[c]);
+                for (int c = 0; c < 4; ++c) {
+                    const float lo = ((bf_lo(a6[c]) + bf_lo(a8[c])) + bf_lo(e[c])) + bf_lo(t[c]);
+                    const float hi = ((bf_hi(a6[c]) + bf_hi(a8[c])) + bf_hi(e[c])) + bf_hi(t[c]);
+                    e[c] = pack_bf(lo, hi);
+                    o[c] = add_bf16x2(a7[c], o[c]);
+                }
+            } else {
+                #pragma unroll
+                for (int c = 0; c < 4; ++c) e[c] = add_bf16x2(e[c], t[c]);
             }
-            tap_select(wd[0][0], wa[0][0], 3 * r, e0);           // window (j, i): taps (r, 0) and (r, 1)
-            tap_select(wd[0][0], wa[0][0], 3 * r + 1, o0);
-            tap_select(wd[0][1], wa[0][1], 3 * r + 2, t);        // window (j, i-1): tap (r, 2) on the even pixel
             #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const f2 v = mk2(e0[c], o0[c]);
-                g[c] = add2(r == 0 ? add2(g[c], v) : v, mk2(t[c], 0.f));
-            }
-            // rounded to bf16, as pool_bwd_kernel stores it
-            uint4 q0, q1;
-            pack_pair(g, q0, q1);
-            const uint32_t b0[4] = {q0.x, q0.y, q0.z, q0.w}, b1[4] = {q1.x, q1.y, q1.z, q1.w};
-            #pragma unroll
-            for (int c = 0; c < 4; ++c) { g[2 * c] = mk2(bf_lo(b0[c]), bf_lo(b1[c])); g[2 * c + 1] = mk2(bf_hi(b0[c]), bf_hi(b1[c])); }
+            for (int c = 0; c < 4; ++c) { g[2 * c] = mk2(bf_lo(e[c]), bf_lo(o[c])); g[2 * c + 1] = mk2(bf_hi(e[c]), bf_hi(o[c])); }
         }
         uint32_t w0[6] = {__shfl_up_sync(0xffffffffu, av[r][0].w, 1), av[r][0].x, av[r][0].y, av[r][0].z, av[r][0].w, __shfl_down_sync(0xffffffffu, av[r][0].x, 1)};
         uint32_t w1[6] = {__shfl_up_sync(0xffffffffu, av[r][1].w, 1), av[r][1].x, av[r][1].y, av[r][1].z, av[r][1].w, __shfl_down_sync(0xffffffffu, av[r][1].x, 1)};
