@@ -965,9 +965,9 @@ void op_pool_bwd(alexnet* h, int r, int which, cudaStream_t st) {
     const uint8_t* a[3] = {R.arg1, R.arg2, R.arg5};
     const bf16* relu[3] = {nullptr, nullptr, R.a5};
     bf16* dx[3] = {R.dn1, R.dn2, R.da5};
-    const dim3 grid(nblk((long long)g.Wpi * (g.C / 8), 256), g.Hpi, h->B);
+    const dim3 grid(nblk((long long)((g.Wpi + 1) / 2) * (g.C / 8), 256), (g.Hpi + 1) / 2, h->B);
     launch_k(kn::pool_bwd_kernel, grid, 256, 0, st, dy[which], a[which], relu[which], dx[which], g.C / 8, g.Hpi, g.Wpi,
-                                              g.Hi, g.Wi, g.Ho, g.Wo, g.Hpo, g.Wpo);
+                                              g.Ho, g.Wo, g.Hpo, g.Wpo);
     h->launches++;
 }
 // fused LRN + pool kernels, instantiated for the two LRN layers: {vectors per pixel, vectors per block, W, H, output rows

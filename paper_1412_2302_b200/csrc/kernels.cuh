@@ -247,49 +247,6 @@ __global__ void __launch_bounds__(256) pool_fwd_kernel(const __nv_bfloat16* __re
     ab.y = bi[4] | (bi[5] << 8) | (bi[6] << 16) | (bi[7] << 24);
     ((uint2*)arg)[((size_t)(n * Ho + oy) * Wo + ox) * cpr + ch] = ab;
 }
-// dx[y][x] = sum over the (up to 4) windows containing (y,x) whose argmax points at it; optional ReLU mask.
-// grid: (ceil(Wpi*cpr / 256), Hpi, B); one thread = 8 channels of one input pixel (pad pixels get zero).
-__device__ __forceinline__ void pool_bwd8(const __nv_bfloat16* __restrict__ dy, const uint8_t* __restrict__ arg, float* acc,
-                                          int n, int y, int x, int ch, int cpr, int Ho, int Wo, int Hpo, int Wpo) {
-    const int oy_lo = max(0, (y - 1) >> 1), oy_hi = min(Ho - 1, y >> 1);
-    const int ox_lo = max(0, (x - 1) >> 1), ox_hi = min(Wo - 1, x >> 1);
-    for (int oy = oy_lo; oy <= oy_hi; ++oy)
-        for (int ox = ox_lo; ox <= ox_hi; ++ox) {
-            const unsigned code = (unsigned)((y - 2 * oy) * 3 + (x - 2 * ox)) * 0x01010101u;
-            const uint2 ab = __ldg((const uint2*)arg + ((size_t)(n * Ho + oy) * Wo + ox) * cpr + ch);
-            float f[8];
-            unpack8(__ldg((const uint4*)dy + ((size_t)(n * Hpo + oy) * Wpo + ox) * cpr + ch), f);
-            // byte-wise equality of the eight argmax codes with this pixel's code
-            const unsigned e0 = ab.x ^ code, e1 = ab.y ^ code;
-            #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (((e0 >> (8 * q)) & 0xFFu) == 0u) acc[q] += f[q];
-                if (((e1 >> (8 * q)) & 0xFFu) == 0u) acc[q + 4] += f[q + 4];
-            }
-        }
-}
-__global__ void __launch_bounds__(256) pool_bwd_kernel(const __nv_bfloat16* __restrict__ dy, const uint8_t* __restrict__ arg,
-                                                       const __nv_bfloat16* __restrict__ relu_src, __nv_bfloat16* __restrict__ dx,
-                                                       int cpr, int Hpi, int Wpi, int Hi, int Wi, int Ho, int Wo, int Hpo, int Wpo) {
-    pdl_sync();
-    const unsigned i = blockIdx.x * 256u + threadIdx.x;
-    if (i >= (unsigned)(Wpi * cpr)) return;
-    const int x = i / cpr, ch = i - x * cpr;
-    const int y = blockIdx.y, n = blockIdx.z;
-    const size_t t = ((size_t)(n * Hpi + y) * Wpi + x) * cpr + ch;
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (y < Hi && x < Wi) {
-        pool_bwd8(dy, arg, acc, n, y, x, ch, cpr, Ho, Wo, Hpo, Wpo);
-        if (relu_src) {
-            float m[8];
-            unpack8(__ldg((const uint4*)relu_src + t), m);
-            #pragma unroll
-            for (int q = 0; q < 8; ++q) acc[q] = m[q] > 0.f ? acc[q] : 0.f;
-        }
-    }
-    ((uint4*)dx)[t] = pack8(acc);
-}
-
 // ------------------------------------------------- LRN + pool fused (the training step)
 // Geometry is a template parameter (the network's two LRN layers): CPR 16-byte vectors per pixel, input WI x HI.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
@@ -301,7 +258,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // SM and cycle), not by HBM, and packing halves the arithmetic instructions.  Window sums take pair sums shared by
 // neighbouring channels.  Measured at batch 128 (back to back), this form against one thread per pixel vector with the
 // pooling gradient scattered through shared memory: forward 40.4 -> 36.6 us (LRN1) and 27.6 -> 24.8 (LRN2), backward 79.1 ->
-// 55 and 48.9 -> 35; at batch 512 forward 141 -> 128 and 97 -> 83.  Same arithmetic in the same order as the single-operation kernels.
+// 53.5 and 48.9 -> 34; at batch 512 forward 141 -> 128 and 97 -> 83.  Same arithmetic in the same order as the single-operation kernels.
 typedef unsigned long long f2;
 __device__ __forceinline__ f2 mk2(float lo, float hi) { f2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
 __device__ __forceinline__ void un2(f2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
@@ -452,20 +409,6 @@ __global__ void __launch_bounds__((WI + 1) / 2 * CV, MINB) lrn_pool_fwd_kernel(c
         }
     }
 }
-// Backward: da = LRN'(a, dn), dn = maxpool'(dp, arg).  One thread = eight channels of a 2 x 2 block of pixels (rows 2j, 2j+1,
-// columns 2i, 2i+1).  The four windows (j-1..j, i-1..i) are the only ones that reach these pixels, in nine (window, tap)
-// combinations, so dn is gathered in registers: four argmax bytes are compared with a tap at once, the byte masks select
-// the bf16 gradients, and the up to four terms of a pixel are added in fp32 in a fixed order.  No shared memory, no
-// barriers, no divergent loops.  dn is rounded to bf16, as pool_bwd_kernel stores it.  Then s^-beta and tt = dn a s^(-beta-1) for the row's pixel pair; the tt of the two channels on
-// either side come from the neighbouring lanes, which hold the neighbouring channel vectors: where a pixel is not a whole
-// warp (CPR = 12) the first and last lane of a warp only compute for their neighbours (30 of 32 lanes store).  The ReLU
-// mask of the convolution that produced a is applied to the packed result.  Pad positions are not written: they are zero.
-// grid: (ceil(warps per image / 4), B), 128 threads.
-template <int CPR, int WI, int HI>
-struct PoolLrnBwdGeo {
-    static constexpr int HALO = CPR == 32 ? 0 : 1, PER = 32 - 2 * HALO, NP = (WI + 1) / 2, NJ = (HI + 1) / 2;
-    static constexpr int TOT = NJ * NP * CPR, WARPS = (TOT + PER - 1) / PER, BLOCKS = (WARPS + 3) / 4;
-};
 // the eight gradients of a window where its argmax equals the tap, else zero (four words of two bf16 channels)
 __device__ __forceinline__ void tap_words(const uint4& g, const uint2& ab, uint32_t tap, uint32_t* v) {
     const uint32_t T = tap * 0x01010101u;
@@ -481,6 +424,92 @@ __device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
     const __nv_bfloat162 r = __hadd2(*(const __nv_bfloat162*)&a, *(const __nv_bfloat162*)&b);
     return *(const uint32_t*)&r;
 }
+// halves of a word of two bf16 that are greater than zero, as 16-bit masks
+__device__ __forceinline__ uint32_t positive_mask(uint32_t w) {
+    return __hgt2_mask(*(const __nv_bfloat162*)&w, __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
+}
+// dx[y][x] = sum over the (up to 4) windows containing (y,x) whose argmax points at it; optional ReLU mask.  One thread = eight
+// channels of the 2 x 2 input pixels (2j, 2i) .. (2j+1, 2i+1): their nine taps lie in four windows, so a window's gradients and codes are
+// read four times in all instead of nine, and all of a thread's loads are in flight together.  A pixel of one or two terms stays
+// packed bf16 (one rounding, as in fp32 followed by the conversion).  Windows cover valid pixels only, so pad pixels get zero.
+// Measured (pool5): one thread per pixel and a loop over its windows 10.5 us at batch 128 and 36.0 at 512, this form 7.2 and 22.2
+// (HBM floor 4.3 and 17).
+// grid: (ceil(ceil(Wpi / 2) * cpr / 256), ceil(Hpi / 2), B).
+__global__ void __launch_bounds__(256) pool_bwd_kernel(const __nv_bfloat16* __restrict__ dy, const uint8_t* __restrict__ arg,
+                                                       const __nv_bfloat16* __restrict__ relu_src, __nv_bfloat16* __restrict__ dx,
+                                                       int cpr, int Hpi, int Wpi, int Ho, int Wo, int Hpo, int Wpo) {
+    pdl_sync();
+    const unsigned q = blockIdx.x * 256u + threadIdx.x;
+    if (q >= (unsigned)((Wpi + 1) / 2 * cpr)) return;
+    const int i = q / cpr, ch = q - i * cpr;
+    const int j = blockIdx.y, n = blockIdx.z;
+    uint4 d[2][2], rl[2][2]; uint2 ab[2][2];            // windows (j - dj, i - di); the pixels' ReLU source
+    #pragma unroll
+    for (int dj = 0; dj < 2; ++dj)
+        #pragma unroll
+        for (int di = 0; di < 2; ++di) {
+            const int oy = j - dj, ox = i - di;
+            d[dj][di] = make_uint4(0, 0, 0, 0);
+            ab[dj][di] = make_uint2(0, 0);
+            if (oy >= 0 && oy < Ho && ox >= 0 && ox < Wo) {
+                ab[dj][di] = __ldg((const uint2*)arg + ((size_t)(n * Ho + oy) * Wo + ox) * cpr + ch);
+                d[dj][di] = __ldg((const uint4*)dy + ((size_t)(n * Hpo + oy) * Wpo + ox) * cpr + ch);
+            }
+        }
+    const size_t t0 = ((size_t)(n * Hpi + 2 * j) * Wpi + 2 * i) * cpr + ch;
+    #pragma unroll
+    for (int r = 0; r < 2; ++r)
+        #pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            rl[r][s] = make_uint4(0, 0, 0, 0);
+            if (relu_src && 2 * j + r < Hpi && 2 * i + s < Wpi) rl[r][s] = __ldg((const uint4*)relu_src + t0 + (size_t)(r * Wpi + s) * cpr);
+        }
+    uint32_t g[2][2][4], u[4], v[4], w[4];
+    tap_words(d[0][0], ab[0][0], 0, g[0][0]);
+    tap_words(d[0][1], ab[0][1], 2, u);
+    tap_words(d[1][0], ab[1][0], 6, v);
+    tap_words(d[1][1], ab[1][1], 8, w);
+    #pragma unroll
+    for (int c = 0; c < 4; ++c)
+        g[0][0][c] = pack_bf(((bf_lo(w[c]) + bf_lo(v[c])) + bf_lo(u[c])) + bf_lo(g[0][0][c]),
+                             ((bf_hi(w[c]) + bf_hi(v[c])) + bf_hi(u[c])) + bf_hi(g[0][0][c]));
+    tap_words(d[0][0], ab[0][0], 1, g[0][1]);
+    tap_words(d[1][0], ab[1][0], 7, u);
+    tap_words(d[0][0], ab[0][0], 3, g[1][0]);
+    tap_words(d[0][1], ab[0][1], 5, v);
+    tap_words(d[0][0], ab[0][0], 4, g[1][1]);
+    #pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        g[0][1][c] = add_bf16x2(u[c], g[0][1][c]);
+        g[1][0][c] = add_bf16x2(v[c], g[1][0][c]);
+    }
+    #pragma unroll
+    for (int r = 0; r < 2; ++r)
+        #pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            if (2 * j + r >= Hpi || 2 * i + s >= Wpi) continue;
+            uint4 o = make_uint4(g[r][s][0], g[r][s][1], g[r][s][2], g[r][s][3]);
+            if (relu_src) {
+                const uint4 m = rl[r][s];
+                o.x &= positive_mask(m.x); o.y &= positive_mask(m.y); o.z &= positive_mask(m.z); o.w &= positive_mask(m.w);
+            }
+            ((uint4*)dx)[t0 + (size_t)(r * Wpi + s) * cpr] = o;
+        }
+}
+// Backward: da = LRN'(a, dn), dn = maxpool'(dp, arg).  One thread = eight channels of a 2 x 2 block of pixels (rows 2j, 2j+1,
+// columns 2i, 2i+1).  The four windows (j-1..j, i-1..i) are the only ones that reach these pixels, in nine (window, tap)
+// combinations, so dn is gathered in registers: four argmax bytes are compared with a tap at once, the byte masks select
+// the bf16 gradients, and the up to four terms of a pixel are added in fp32 in a fixed order.  No shared memory, no
+// barriers, no divergent loops.  dn is rounded to bf16, as pool_bwd_kernel stores it.  Then s^-beta and tt = dn a s^(-beta-1) for the row's pixel pair; the tt of the two channels on
+// either side come from the neighbouring lanes, which hold the neighbouring channel vectors: where a pixel is not a whole
+// warp (CPR = 12) the first and last lane of a warp only compute for their neighbours (30 of 32 lanes store).  The ReLU
+// mask of the convolution that produced a is applied to the packed result.  Pad positions are not written: they are zero.
+// grid: (ceil(warps per image / 4), B), 128 threads.
+template <int CPR, int WI, int HI>
+struct PoolLrnBwdGeo {
+    static constexpr int HALO = CPR == 32 ? 0 : 1, PER = 32 - 2 * HALO, NP = (WI + 1) / 2, NJ = (HI + 1) / 2;
+    static constexpr int TOT = NJ * NP * CPR, WARPS = (TOT + PER - 1) / PER, BLOCKS = (WARPS + 3) / 4;
+};
 template <int CPR, int WI, int HI, bool B75>
 __global__ void __launch_bounds__(128, 5) pool_lrn_bwd_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ dp,
                                                            const uint8_t* __restrict__ arg, __nv_bfloat16* __restrict__ da,
