@@ -1147,7 +1147,7 @@ void op_preprocess(alexnet* h, int r, int slot, uint64_t step, cudaStream_t st, 
     kn::ColorAug aug = h->color;
     aug.key = kn::stream_key(h->cfg.seed, 10, r, step);
     const bool augment = aug.sigma != 0.f && !eval;
-    launch_k(augment ? kn::preprocess_kernel<true> : kn::preprocess_kernel<false>, dim3(57, images), 256, 0, st, R.stage[slot], h->mean, R.x0[slot],
+    launch_k(augment ? kn::preprocess_kernel<true> : kn::preprocess_kernel<false>, dim3(images, 57), 256, 0, st, R.stage[slot], h->mean, R.x0[slot],
              R.cf[slot], labels, R.labels[slot], i0, kn::stream_key(h->cfg.seed, 1, r, step), eval ? 1 : 0, aug);
     h->launches++;
 }
