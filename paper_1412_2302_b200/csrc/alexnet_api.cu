@@ -754,10 +754,13 @@ int build_plans(alexnet* h, int r) {
 }
 
 // An evaluation whose images come over PCIe works in chunks of images: the convolution layers of one chunk run while the next is
-// copied.  A chunk of n images takes about 85 + 1.2 n us (eight dependent launches and the work) and its copy 3.6 n us, so
-// from about 40 images on the copies are the longer side; what is left behind the last copy is one chunk's time.
-constexpr int kEvalChunk = 40;
-int eval_chunks(int B) { return std::max(1, B / kEvalChunk); }
+// copied (3.6 us per image); what is left behind the last copy is one chunk's time and the FC layers.  A chunk's dependent launches
+// cost a fixed time and small grids fill the machine badly, so chunks below about 50 images take longer than the copy they should
+// hide behind and the delay adds up from chunk to chunk, while two chunks can be smaller, since only the first has to keep up.
+// Measured, chunks of at least 40 / 54 / 64 / 80 / 100 images: 256 images 1301 / 1207 / 1206 / 1233 / 1308 us, 512 images 2299 / 2231 /
+// 2180 / 2199 / 2234; two chunks against one: 72 images 537 -> 520, 64 488 -> 468, 56 452 -> 441, 48 411 -> 419.
+constexpr int kEvalChunk = 64, kEvalTwoChunks = 56;
+int eval_chunks(int B) { return std::max(B >= kEvalTwoChunks ? 2 : 1, B / kEvalChunk); }
 inline int chunk_begin(int B, int chunks, int c) { return (int)((long long)B * c / chunks); }
 int build_eval_plans(alexnet* h, int r, int slot) {
     Replica& R = h->rep[r];

@@ -61,3 +61,28 @@ def test_eval_batch_against_oracle(inverted):
     t1b, t5b, _ = net.eval_batch(0, torch.from_numpy(img).pin_memory(), torch.from_numpy(lab).pin_memory())
     assert 0 <= t1b <= t5b <= B
     net.close()
+
+
+@pytest.mark.parametrize("B", [55, 56, 57, 129, 193])
+def test_eval_in_chunks_agrees_with_one_pass(B):
+    """Images in host memory are evaluated in chunks (one up to 55 images, then two, more from 192 on; 57, 129 and 193 do not
+    divide evenly), images on the device in one pass.  Both compute the same sums in fp32, in an order that depends on the tile
+    numbering, and each is within TOL of the oracle by the test above: the logits agree within 2 TOL, the mean loss to the
+    same relative bound, and the counts are exact for the logits of each."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed = synth.BASE_SEED + 32
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    net.set_params(synth.init_params(seed, variance_preserving=True, bias=0.1))
+    gen = torch.Generator().manual_seed(B)
+    img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen)
+    lab = torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen)
+    got = {}
+    for where, im, lb in (("host", img.pin_memory(), lab.pin_memory()), ("device", img.cuda(), lab.cuda())):
+        torch.cuda.synchronize()
+        t1, t5, loss = net.eval_batch(0, im, lb)
+        z = net.get_tensor("Z").reshape(B, 1000)
+        assert t1 == int(O.topk_correct(z, lab.numpy(), 1).sum()) and t5 == int(O.topk_correct(z, lab.numpy(), 5).sum()), where
+        got[where] = z, loss
+    assert rel(got["host"][0], got["device"][0]) < 2 * TOL
+    assert abs(got["host"][1] - got["device"][1]) < 2 * TOL * max(1.0, abs(got["device"][1]))
+    net.close()
