@@ -3,6 +3,7 @@
 #include "../../include/alexnet.h"
 
 #include <cudaTypedefs.h>
+#include <cxxabi.h>
 
 #include <algorithm>
 #include <atomic>
@@ -16,6 +17,17 @@
 #include "kernels.cuh"
 #include "tc_gemm.cuh"
 
+// The first launch of this thread that the runtime refused since somebody last asked (launches_ok below), and its kernel: a
+// refused launch leaves the rest of a pass running on old data, so the call that made it has to end with an error that
+// says which kernel it was.
+namespace {
+thread_local cudaError_t g_launch_error = cudaSuccess;
+thread_local const void* g_launch_kernel = nullptr;
+void note_launch(cudaError_t e, const void* kernel) {
+    if (e != cudaSuccess && g_launch_error == cudaSuccess) { g_launch_error = e; g_launch_kernel = kernel; }
+}
+}  // namespace
+
 // Every kernel is launched with programmatic stream serialization: its blocks may become resident while the kernel
 // before it in the stream drains, and run their set-up; each kernel waits (griddepcontrol.wait) before it touches
 // global memory, so the data dependencies of the stream order are kept.
@@ -27,7 +39,7 @@ void launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cuda
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = &at; lc.numAttrs = 1;
-    cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
+    note_launch(cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...), (const void*)kernel);
 }
 
 // The same as a grid of clusters of two (an odd grid: as single CTAs): the two CTAs of a cluster take the two SMs of one TPC.  A kernel whose CTAs take a
@@ -44,7 +56,7 @@ void launch_paired(void (*kernel)(KArgs...), int grid, dim3 block, size_t smem, 
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = 2; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     lc.attrs = at; lc.numAttrs = grid % 2 == 0 ? 2 : 1;
-    cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
+    note_launch(cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...), (const void*)kernel);
 }
 
 namespace {
@@ -226,6 +238,27 @@ namespace {
 
 int fail(alexnet* h, int code, const std::string& msg) { if (h) h->err = msg; return code; }
 #define CK(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) return fail(h, ALEXNET_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); } while (0)
+
+// "kernel: error" of the launch noted above (empty: none), which is then forgotten
+std::string take_launch_error() {
+    if (g_launch_error == cudaSuccess) return std::string();
+    const char* sym = nullptr;
+    if (cudaFuncGetName(&sym, g_launch_kernel) != cudaSuccess || !sym) sym = "a kernel";
+    int st = 0;
+    char* plain = abi::__cxa_demangle(sym, nullptr, nullptr, &st);
+    const std::string msg = std::string("launch of ") + (plain ? plain : sym) + ": " + cudaGetErrorString(g_launch_error);
+    free(plain);
+    g_launch_error = cudaSuccess;
+    return msg;
+}
+// at the end of every call that launches: the launches were accepted and nothing before them has failed
+int launches_ok(alexnet* h) {
+    const std::string msg = take_launch_error();
+    const cudaError_t e = cudaGetLastError();
+    if (!msg.empty()) return fail(h, ALEXNET_ERR_CUDA, msg);
+    if (e != cudaSuccess) return fail(h, ALEXNET_ERR_CUDA, std::string("an earlier call on the GPU: ") + cudaGetErrorString(e));
+    return ALEXNET_OK;
+}
 
 struct Carver {
     uint8_t* base; size_t off;
@@ -810,7 +843,7 @@ void launch_gemm(alexnet* h, const Plan& P0, cudaStream_t st, bool early_weights
         at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[1].val.programmaticStreamSerializationAllowed = 1;
         lc.attrs = at; lc.numAttrs = 2;
-        cudaLaunchKernelEx(&lc, tc::conv_kernel<2>, P.c);
+        note_launch(cudaLaunchKernelEx(&lc, tc::conv_kernel<2>, P.c), (const void*)tc::conv_kernel<2>);
     }
     else if (P.conv && P.c.zcluster) {
         cudaLaunchConfig_t lc{};
@@ -821,7 +854,7 @@ void launch_gemm(alexnet* h, const Plan& P0, cudaStream_t st, bool early_weights
         at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[1].val.programmaticStreamSerializationAllowed = 1;
         lc.attrs = at; lc.numAttrs = 2;
-        cudaLaunchKernelEx(&lc, tc::conv_kernel<1>, P.c);
+        note_launch(cudaLaunchKernelEx(&lc, tc::conv_kernel<1>, P.c), (const void*)tc::conv_kernel<1>);
     }
     else if (P.conv) launch_k(tc::conv_kernel<1>, P.grid, tc::conv_threads(P.c), P.smem, st, P.c);
     else launch_k(tc::gemm_kernel, P.grid, tc::kThreads, P.smem, st, P.p);
@@ -1474,7 +1507,7 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
         if (rc) return create_fail(h, rc, "alexnet_create: " + h->err);
     }
     CKC(cudaStreamSynchronize(h->cs));
-    CKC(cudaGetLastError());
+    if (int rc = launches_ok(h)) return create_fail(h, rc, "alexnet_create: " + h->err);
     *out = h;
     return ALEXNET_OK;
 }
@@ -1499,6 +1532,7 @@ int alexnet_load_batch_async(alexnet_t* h, int replica, const uint8_t* images, c
     CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
     op_preprocess(h, replica, s, step, h->ls);
     CK(cudaEventRecord(R.ready[s], h->ls));
+    if (int rc = launches_ok(h)) return rc;
     R.slot_step[s] = step;
     R.last_slot = s; R.next_load ^= 1; R.loaded++;
     return ALEXNET_OK;
@@ -1524,11 +1558,11 @@ static int step_impl(alexnet_t* h, int replica, float* host_loss, bool with_upda
     if (with_update) op_update(h, replica, h->cs, false, 1.f, defer ? s : -1);
     R.grad_pending = !with_update;
     R.last_slot = s; R.next_train ^= 1; R.loaded--;
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     if (host_loss) {
         launch_k(kn::store_result_kernel, 1, 1, 0, h->cs, (const float*)R.loss, (const int*)h->status, h->host_result, ++h->result_seq);
         h->launches++;
-        CK(cudaGetLastError());
+        if (int rc = launches_ok(h)) return rc;
         CK(cudaStreamSynchronize(h->cs));      // the call promises a finished step
         kn::HostResult res;
         if (int rc = wait_result(h, &res)) return rc;
@@ -1550,7 +1584,7 @@ int alexnet_apply_update(alexnet_t* h, int replica, float grad_scale) {
     if (!R.grad_pending) return fail(h, ALEXNET_ERR_STATE, "apply_update: no pending gradient (call alexnet_forward_backward first)");
     op_update(h, replica, h->cs, true, grad_scale);
     R.grad_pending = false;
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1562,7 +1596,7 @@ int alexnet_update_and_average(alexnet_t* h) {
         return fail(h, ALEXNET_ERR_STATE, "update_and_average: both replicas need a pending gradient (alexnet_forward_backward)");
     op_update_average(h, h->cs);
     h->rep[0].grad_pending = h->rep[1].grad_pending = false;
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1603,7 +1637,7 @@ int alexnet_scale_and_refresh(alexnet_t* h, int replica, float scale) {
     if (int rc = check_status(h)) return rc;
     if (shared_weights(h) && replica == 1) return ALEXNET_OK;      // replica 0's call has done the shared copy
     op_scale_refresh(h, replica, scale, h->cs);
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1634,7 +1668,7 @@ int alexnet_average_received(alexnet_t* h, int replica, const float* const* dev_
     launch_k(kn::average_received_kernel, 1184, 256, 0, h->cs, R.w, R.v, R.shadow, rl, h->L.n_total / 4, 1.f / (float)count);
     h->launches++;
     refresh_shadows(h, replica, false, h->cs);
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1644,7 +1678,7 @@ int alexnet_debug_expire_wait(alexnet_t* h, long long budget_cycles) {
     const long long budget = std::min<long long>(200000000LL, std::max<long long>(10000LL, budget_cycles));
     launch_k(tc::wait_probe_kernel, 1, 32, 0, h->cs, h->status, budget);
     h->launches++;
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1660,7 +1694,7 @@ int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out) {
         (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)) {
         launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
         h->launches++;
-        CK(cudaGetLastError());
+        if (int rc = launches_ok(h)) return rc;
         return ALEXNET_OK;
     }
     cudaGetLastError();      // (an unregistered host pointer makes the query fail on some drivers: not an error here)
@@ -1705,7 +1739,7 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     else forward(h, replica, s, h->cs, true);
     CK(cudaEventRecord(R.consumed[s], h->cs));
     R.consumed_valid[s] = true;
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     kn::HostResult res;
     if (int rc = wait_result(h, &res)) return rc;
     if (host_top1) *host_top1 = res.top1;
@@ -1719,7 +1753,7 @@ int alexnet_replica_average(alexnet_t* h) {
     if (int rc = check_status(h)) return rc;
     if (h->cfg.replicas < 2 || shared_weights(h)) return ALEXNET_OK;     // one copy: nothing to average
     op_average(h, h->cs);
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -1731,6 +1765,7 @@ int alexnet_get_params(alexnet_t* h, int replica, int which, float* host_out, si
     const float* src = which == 0 ? R.w : which == 1 ? R.v : R.g;
     launch_k(kn::params_gather_kernel, 1184, 256, 0, h->cs, src, h->canon_tmp, h->L.segs, kCanonCount);
     h->launches++;
+    if (int rc = launches_ok(h)) return rc;
     CK(cudaMemcpyAsync(host_out, h->canon_tmp, n * sizeof(float), cudaMemcpyDeviceToHost, h->cs));
     CK(cudaStreamSynchronize(h->cs));
     return poll_status(h);
@@ -1747,6 +1782,7 @@ int alexnet_set_params(alexnet_t* h, int replica, int which, const float* host_i
     launch_k(kn::params_scatter_kernel, 1184, 256, 0, h->cs, dst, h->canon_tmp, h->L.segs, kCanonCount);
     h->launches++;
     if (which == 0) refresh_shadows(h, replica, true, h->cs);
+    if (int rc = launches_ok(h)) return rc;
     CK(cudaStreamSynchronize(h->cs));
     return ALEXNET_OK;
 }
@@ -1771,6 +1807,7 @@ int alexnet_get_tensor(alexnet_t* h, int replica, int tensor_id, float* out, siz
         if (tensor_id == ALEXNET_T_DN1 && R.dn_stale[0]) op_pool_bwd(h, replica, 0, h->cs);
         if (tensor_id == ALEXNET_T_DN2 && R.dn_stale[1]) op_pool_bwd(h, replica, 1, h->cs);
     }
+    if (int rc = launches_ok(h)) return rc;
     std::vector<uint8_t> raw(tensor_dev_bytes(T, B));
     CK(cudaStreamSynchronize(h->cs));
     CK(cudaStreamSynchronize(h->ls));
@@ -1878,7 +1915,7 @@ int alexnet_run_op(alexnet_t* h, int replica, int op, int iters) {
                 return fail(h, ALEXNET_ERR_STATE, "the FC forward chain is not available in this configuration");
         }
     }
-    CK(cudaGetLastError());
+    if (int rc = launches_ok(h)) return rc;
     return ALEXNET_OK;
 }
 
@@ -2009,7 +2046,8 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
     splits = std::max<int64_t>(splits, 1);
     launch_k(kn::bias_grad_kernel, dim3(groups, (unsigned)splits), 256, 0, (cudaStream_t)stream, (const bf16*)dev_dy, (long long)rows, channels,
              g_noalloc_ptr[dev], g_noalloc_cnt[dev], dev_db);
+    const std::string refused = take_launch_error();
     e = cudaGetLastError();
-    if (e != cudaSuccess) { put_err(err, err_len, cudaGetErrorString(e)); return ALEXNET_ERR_CUDA; }
+    if (!refused.empty() || e != cudaSuccess) { put_err(err, err_len, refused.empty() ? cudaGetErrorString(e) : refused.c_str()); return ALEXNET_ERR_CUDA; }
     return ALEXNET_OK;
 }

@@ -856,3 +856,27 @@ def test_batch1024_largest_configuration_sampled_forward():
     for k, (o, n, _) in off.items():
         assert np.abs(gc[o:o + n]).max() > 0, k
     net.close()
+
+
+def test_refused_launch_names_its_kernel():
+    """A launch that the runtime refuses (here: into a stream whose capture a synchronisation has invalidated, so that nothing
+    reaches the GPU) ends the call that made it with an error that names the kernel, and the handle works on afterwards."""
+    import ctypes
+    from paper_1412_2302_b200 import alexnet as A
+    net = make(1, seed=BASE + 14)
+    net.set_params(synth.init_params(BASE + 14))
+    w = net.get_params(0, 0)
+    rt, stream, graph = ctypes.CDLL("libcudart.so.12"), ctypes.c_void_p(net.compute_stream.cuda_stream), ctypes.c_void_p()
+    torch.cuda.synchronize()
+    assert rt.cudaStreamBeginCapture(stream, 2) == 0                 # relaxed mode
+    assert rt.cudaStreamSynchronize(stream) != 0                     # not permitted: the capture is invalid from here on
+    with pytest.raises(A.AlexNetError) as e:
+        net.scale_and_refresh(0, 0.5)
+    assert e.value.code == A.ERR_CUDA and "scale_refresh_kernel" in str(e.value)
+    assert rt.cudaStreamEndCapture(stream, ctypes.byref(graph)) != 0 and not graph.value
+    rt.cudaGetLastError()
+    net.sync()
+    assert np.array_equal(net.get_params(0, 0), w)
+    net.scale_and_refresh(0, 0.5)
+    assert np.array_equal(net.get_params(0, 0), 0.5 * w)
+    net.close()
