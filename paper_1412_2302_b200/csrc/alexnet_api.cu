@@ -1389,6 +1389,33 @@ inline uint16_t f2bf(float f) {
     return (uint16_t)(u >> 16);
 }
 
+// Every kernel of the library.  The runtime loads a kernel's code when it is first asked for it, by default at its first
+// launch, which in a training step means in the middle of a pass that already runs on five streams and overlaps its launches;
+// alexnet_create asks for all of them instead, so that no pass loads code (and the first pass costs what later ones cost).
+const void* const kKernels[] = {
+    (const void*)kn::preprocess_kernel<false>, (const void*)kn::preprocess_kernel<true>,
+    (const void*)kn::lrn_fwd_kernel, (const void*)kn::lrn_bwd_kernel, (const void*)kn::pool_fwd_kernel, (const void*)kn::pool_bwd_kernel,
+    (const void*)LRN_POOL_FWD_1(false), (const void*)LRN_POOL_FWD_1(true), (const void*)LRN_POOL_FWD_2(false), (const void*)LRN_POOL_FWD_2(true),
+    (const void*)POOL_LRN_BWD_1(false), (const void*)POOL_LRN_BWD_1(true), (const void*)POOL_LRN_BWD_2(false), (const void*)POOL_LRN_BWD_2(true),
+    (const void*)kn::fc_reduce_fwd_kernel, (const void*)kn::fc_reduce_bwd_kernel, (const void*)kn::wgrad_reduce_kernel,
+    (const void*)kn::colsum_kernel, (const void*)kn::colsum_final_kernel, (const void*)kn::colsum_scalar_kernel, (const void*)kn::bias_grad_kernel,
+    (const void*)kn::softmax_xent_kernel, (const void*)kn::mean_kernel, (const void*)kn::fc8_softmax_xent_kernel<false>,
+    (const void*)kn::fc8_softmax_xent_kernel<true>, (const void*)kn::store_result_kernel, (const void*)kn::store_value_kernel,
+    (const void*)kn::sgd_update_kernel, (const void*)kn::sgd_update_conv_kernel, (const void*)kn::replica_average_kernel,
+    (const void*)kn::sgd_update_average_kernel, (const void*)kn::sgd_update_average_shared_kernel, (const void*)kn::scale_refresh_kernel,
+    (const void*)kn::average_received_kernel, (const void*)kn::shadow_kernel, (const void*)kn::conv_transpose_shadow_kernel,
+    (const void*)kn::params_gather_kernel, (const void*)kn::params_scatter_kernel, (const void*)init_kernel,
+    (const void*)tc::gemm_kernel, (const void*)tc::conv_kernel<1>, (const void*)tc::conv_kernel<2>, (const void*)tc::wgrad_kernel,
+    (const void*)tc::fc_update_kernel<9216>, (const void*)tc::fc_update_kernel<4096>, (const void*)tc::fc_chain_kernel,
+    (const void*)tc::wait_probe_kernel};
+cudaError_t load_kernels() {
+    for (const void* k : kKernels) {
+        cudaFuncAttributes at;
+        if (const cudaError_t e = cudaFuncGetAttributes(&at, k)) return e;
+    }
+    return cudaSuccess;
+}
+
 // everything the handle owns: streams, events (null where never created); shared by alexnet_destroy and the failure paths
 // of alexnet_create
 void teardown(alexnet* h) {
@@ -1460,6 +1487,7 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
     CKC(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres));
     if (!fn || qres != cudaDriverEntryPointSuccess) return create_fail(h, ALEXNET_ERR_CUDA, "alexnet_create: the driver has no cuTensorMapEncodeTiled");
     h->encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+    CKC(load_kernels());
     CKC(cudaFuncSetAttribute(tc::gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     CKC(cudaFuncSetAttribute(tc::conv_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     CKC(cudaFuncSetAttribute(tc::conv_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));

@@ -71,3 +71,19 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(B, "LIB", str(tmp_path / "nothing.so"))
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         A.load_library()
+
+
+def test_every_kernel_is_loaded_with_the_handle():
+    """alexnet_create loads the code of every kernel (no pass may load code between its launches): the list it walks names each
+    `__global__` function of the sources."""
+    csrc = os.path.join(ROOT, "paper_1412_2302_b200", "csrc")
+    api = open(os.path.join(csrc, "alexnet_api.cu")).read()
+    listed = api.split("const void* const kKernels[] = {", 1)[1].split("};", 1)[0]
+    for macro, body in re.findall(r"#define (\w+)\(B75\) (.*)", api):
+        listed = listed.replace(macro, body)
+    names = set()
+    for f in ("kernels.cuh", "tc_gemm.cuh", "alexnet_api.cu"):
+        names |= set(re.findall(r"__global__[^;{]*?\b(\w+_kernel)\(", open(os.path.join(csrc, f)).read()))
+    assert len(names) > 30 and {"conv_kernel", "wgrad_reduce_kernel", "init_kernel"} <= names
+    for n in sorted(names):
+        assert re.search(r"\b%s\b" % n, listed), n
