@@ -152,7 +152,9 @@ int alexnet_train_step(alexnet_t* h, int replica, float* host_loss);
  * float) and return without waiting: the host can read step i's loss while
  * step i+1 runs.  The value is there once the compute stream has reached this
  * point (alexnet_sync, or an event the caller records on that stream after
- * the call); loss_out must stay valid until then.  Errors: ARG, CUDA. */
+ * the call); loss_out must stay valid until then.  The value is NaN when a
+ * bounded device-side wait has expired before that point (the calls that wait
+ * for the GPU then report DEVICE_TIMEOUT).  Errors: ARG, CUDA. */
 int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out);
 
 /* Evaluation of one minibatch, the measurement behind the paper's reported

@@ -1720,13 +1720,17 @@ int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out) {
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, loss_out) == cudaSuccess && at.devicePointer != nullptr &&
         (at.type == cudaMemoryTypeHost || at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged)) {
-        launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (float*)at.devicePointer);
+        launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (const int*)h->status, (float*)at.devicePointer);
         h->launches++;
         if (int rc = launches_ok(h)) return rc;
         return ALEXNET_OK;
     }
     cudaGetLastError();      // (an unregistered host pointer makes the query fail on some drivers: not an error here)
-    CK(cudaMemcpyAsync(loss_out, h->rep[replica].loss, sizeof(float), cudaMemcpyDefault, h->cs));
+    float* staged = h->rep[replica].loss + 1;      // (the slot behind the loss is the copy's source, so that it too carries an expired wait)
+    launch_k(kn::store_value_kernel, 1, 1, 0, h->cs, (const float*)h->rep[replica].loss, (const int*)h->status, staged);
+    h->launches++;
+    if (int rc = launches_ok(h)) return rc;
+    CK(cudaMemcpyAsync(loss_out, staged, sizeof(float), cudaMemcpyDefault, h->cs));
     return ALEXNET_OK;
 }
 

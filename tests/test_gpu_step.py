@@ -495,6 +495,30 @@ def test_loss_async_delivers_the_step_loss():
     net.close()
 
 
+def test_loss_async_reports_an_expired_wait():
+    """A loop that reads only the losses of alexnet_loss_async sees NaN once a bounded wait has run out (the self-test's warp: a
+    barrier nothing arrives on, about a millisecond), whatever kind of memory the loss goes to."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed, B = BASE + 15, 2
+    net = make(B, seed=seed)
+    net.set_params(synth.init_params(seed))
+    pinned, device, pageable = torch.zeros(2).pin_memory(), torch.zeros(1, device="cuda"), np.zeros(1, np.float32)
+    torch.cuda.synchronize()
+    load(net, 0, seed, 0, B)
+    net.train_step(0)
+    net.loss_async(0, pinned[:1])
+    net.debug_expire_wait(2_000_000)
+    for out in (pinned[1:], device, pageable):
+        net.loss_async(0, out)
+    net.compute_stream.synchronize()
+    assert np.isfinite(float(pinned[0])) and float(pinned[0]) > 0
+    assert np.isnan(float(pinned[1])) and np.isnan(float(device[0])) and np.isnan(pageable[0])
+    with pytest.raises(A.AlexNetError) as e:
+        net.sync()
+    assert e.value.code == A.ERR_DEVICE_TIMEOUT
+    net.close()
+
+
 def test_multi_stream_step_is_deterministic():
     """The backward pass forks its independent branches onto streams of their own; the result may not depend on how the
     kernels interleave: three runs of four steps (fused FC update) give bit-identical parameters and momentum."""
