@@ -392,7 +392,12 @@ template <int CPR, int CV, int WI, int HI, bool B75, int MINB>
 __global__ void __launch_bounds__((WI + 1) / 2 * CV, MINB) lrn_pool_fwd_kernel(const __nv_bfloat16* __restrict__ a, __nv_bfloat16* __restrict__ y,
                                                                                uint8_t* __restrict__ arg, int opr, int Hpi, int Wpi, int Hpo,
                                                                                int Wpo, float alpha, float beta, float k) {
-    pdl_sync();
+    // Waits first and lets the next launch start afterwards, unlike every other kernel: when a block of the next kernel runs, conv1
+    // (the kernel before this one) has completed, and with it whatever wrote the weights before the pass.  The
+    // convolution and FC kernels behind this one rely on that when they load weights before their own wait.
+    // (Nothing is lost: batch 8 and 128 and an evaluation of one image take what they took with the trigger first.)
+    pdl_wait();
+    pdl_trigger();
     constexpr int NP = (WI + 1) / 2, NT = NP * CV, WO = (WI - 3) / 2 + 1, HO = (HI - 3) / 2 + 1;
     __shared__ uint4 xch[2][2][NT];           // [parity of the output row][value / filter row of the maximum][thread]
     const int n = blockIdx.z, c0 = blockIdx.y * CV, oy0 = opr * blockIdx.x, oy1 = min(HO, oy0 + opr);

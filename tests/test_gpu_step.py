@@ -408,6 +408,31 @@ def test_fc_update_kernel_equals_gradient_then_update(B):
     assert not np.array_equal(res[2][0], w)
 
 
+@pytest.mark.parametrize("B", [1, 2, 3])
+def test_queued_small_steps_equal_waited_for_steps(B):
+    """At batches of one to three images conv1 and the kernel behind it leave SMs free, on which the next convolution may load its
+    filters while the update of the step before still runs, unless something orders it behind: forty steps queued without
+    a wait must give the parameters of forty steps each of which is waited for, bit for bit."""
+    seed = BASE + 27
+    img = torch.from_numpy(synth.images(seed, 0, 0, B)).cuda(); lab = torch.from_numpy(synth.labels(seed, 0, 0, B)).cuda()
+    w = synth.init_params(seed, variance_preserving=True, bias=0.1)
+    torch.cuda.synchronize()
+    res = []
+    for wait in (True, False):
+        net = make(B, seed=seed, lr=1e-4)
+        net.set_params(w)
+        for step in range(40):
+            net.load_batch_async(0, img, lab, step)
+            net.train_step(0)
+            if wait:
+                net.sync()
+        net.sync()
+        res.append((net.get_params(0, 0), net.get_params(0, 1)))
+        net.close()
+    assert np.isfinite(res[0][0]).all() and not np.array_equal(res[0][0], w)
+    assert np.array_equal(res[0][0], res[1][0]) and np.array_equal(res[0][1], res[1][1])
+
+
 def test_fc_forward_chain_equals_three_launches():
     """ALEXNET_FLAG_FC_CHAIN: fc6 -> fc7 -> fc8 forward as one cooperative launch against the three per-layer launches:
     same units, same summation order, so activations, dropout masks, logits, losses and the parameters after three steps
