@@ -370,7 +370,8 @@ int alexnet_timeline_read(long long* host_out, int clear);
  * make that call before any stream capture begins there.  All calls share the
  * scratch, which keeps the last call's contents (nothing in it needs clearing:
  * each call overwrites what it later reads), so calls whose kernels could run
- * at the same time on one GPU race: order them on one stream or with events. */
+ * at the same time on one GPU race and may leave wrong sums in their own dev_db
+ * (later calls are not affected): order them on one stream or with events. */
 int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32_t channels, float* dev_db, void* stream,
                               char* err, size_t err_len);
 

@@ -2027,18 +2027,22 @@ const char* alexnet_last_error(const alexnet_t* h) { return h ? h->err.c_str() :
 //
 // All calls share the one array and it keeps whatever the last call left in it.
 // Nothing in it has to start at zero: a call writes every partial that it later
-// reads.  (The counters beside it, of finished row splits per 64 columns, start at
-// zero and are reset by every call.)  Two calls whose kernels overlap on the GPU
-// (different streams, no dependency) race on it; order them.
+// reads, and the counters beside it (of finished row splits per 64 columns) carry
+// the number of the call, so that a call starts from zero whatever it finds.  (A
+// captured call keeps its number in every replay: a memset node before it clears
+// the counters instead.)  Two calls whose kernels overlap on the GPU (different
+// streams, no dependency) race on it and may both give wrong sums, but later calls
+// do not suffer from it; order them.
 namespace {
 constexpr int kNoAllocSplits = 64;
 constexpr int kNoAllocMaxC = 4096;
 static __device__ __align__(256) float g_noalloc_partials[kNoAllocSplits * kNoAllocMaxC];
-static __device__ unsigned g_noalloc_counters[kNoAllocMaxC / 64];      // finished row splits per 64 columns; zero between calls
+static __device__ unsigned long long g_noalloc_counters[kNoAllocMaxC / 64];      // call number << 16 | finished row splits of 64 columns
 
 constexpr int kMaxDevices = 64;
 float* g_noalloc_ptr[kMaxDevices] = {nullptr};
-unsigned* g_noalloc_cnt[kMaxDevices] = {nullptr};
+unsigned long long* g_noalloc_cnt[kMaxDevices] = {nullptr};
+std::atomic<unsigned long long> g_noalloc_calls{0};
 
 void put_err(char* buf, size_t len, const char* msg) {
     if (buf && len) { snprintf(buf, len, "%s", msg); }
@@ -2063,7 +2067,7 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
     if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) { put_err(err, err_len, "bias_grad_noalloc: cudaGetDevice failed"); return ALEXNET_ERR_CUDA; }
     if (!g_noalloc_ptr[dev]) {
         float* p = nullptr;
-        unsigned* q = nullptr;
+        unsigned long long* q = nullptr;
         e = cudaGetSymbolAddress((void**)&q, g_noalloc_counters);
         if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&p, g_noalloc_partials);
         if (e != cudaSuccess || !p || !q) {
@@ -2078,8 +2082,13 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
     int64_t splits = std::min<int64_t>(4 * 148 / groups, rows / 64);
     splits = std::min<int64_t>(splits, kNoAllocSplits * kNoAllocMaxC / channels);
     splits = std::max<int64_t>(splits, 1);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing((cudaStream_t)stream, &capture);
+    if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone)
+        e = cudaMemsetAsync(g_noalloc_cnt[dev], 0, groups * sizeof(unsigned long long), (cudaStream_t)stream);
+    if (e != cudaSuccess) { cudaGetLastError(); put_err(err, err_len, cudaGetErrorString(e)); return ALEXNET_ERR_CUDA; }
     launch_k(kn::bias_grad_kernel, dim3(groups, (unsigned)splits), 256, 0, (cudaStream_t)stream, (const bf16*)dev_dy, (long long)rows, channels,
-             g_noalloc_ptr[dev], g_noalloc_cnt[dev], dev_db);
+             g_noalloc_ptr[dev], g_noalloc_cnt[dev], ++g_noalloc_calls, dev_db);
     const std::string refused = take_launch_error();
     e = cudaGetLastError();
     if (!refused.empty() || e != cudaSuccess) { put_err(err, err_len, refused.empty() ? cudaGetErrorString(e) : refused.c_str()); return ALEXNET_ERR_CUDA; }

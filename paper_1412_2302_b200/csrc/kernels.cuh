@@ -839,11 +839,15 @@ __global__ void colsum_scalar_kernel(const __nv_bfloat16* __restrict__ dy, int r
 
 // The same column sums in one launch, for the allocation-free entry point: grid (ceil(C/64), row splits), a block sums 64 columns of
 // its rows (eight 16-byte loads of a thread in flight), and the block of a column group that finishes last adds the
-// group's partials in a fixed order (a counter per group, reset for the next call), so the result does not depend on which
-// block that is.  HBM-bound (L2-bound where dy fits); 25088 x 384 took 12.2 us per call as two launches with one load in
-// flight per thread, 7.6 us in this form, about half of it the launch.
+// group's partials in a fixed order, so the result does not depend on which block that is.  A group counts its finished
+// blocks in the low 16 bits of a word whose upper bits are the number of the launch: the first block of a launch sets the
+// word to its number and a count of zero (a maximum: every later block of the launch leaves the count alone), so a launch
+// owes nothing to what an earlier one left there, be it one that overlapped another or one that died.  HBM-bound (L2-bound
+// where dy fits); 25088 x 384 took 12.2 us per call as two launches with one load in flight per thread, 7.6 us in this form,
+// about half of it the launch.
 __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
-                                                        unsigned* __restrict__ counters, float* __restrict__ db) {
+                                                        unsigned long long* __restrict__ counters, unsigned long long launch,
+                                                        float* __restrict__ db) {
     pdl_sync();
     __shared__ __align__(16) float red[16][68];
     __shared__ bool last;
@@ -890,7 +894,10 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
     if (splits == 1) return;
     __threadfence();
     __syncthreads();
-    if (tid == 0) last = atomicAdd(counters + blockIdx.x, 1u) == (unsigned)splits - 1u;
+    if (tid == 0) {
+        atomicMax(counters + blockIdx.x, launch << 16);
+        last = atomicAdd(counters + blockIdx.x, 1ull) == (launch << 16) + (unsigned)splits - 1u;
+    }
     __syncthreads();
     if (!last) return;
     __threadfence();
@@ -911,7 +918,6 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
         for (int w = 0; w < 16; ++w) s += red[w][tid];
         db[c] = s;
     }
-    if (tid == 0) counters[blockIdx.x] = 0u;
 }
 
 // ------------------------------------------------------ softmax cross-entropy

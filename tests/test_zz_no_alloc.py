@@ -85,3 +85,35 @@ def test_bias_grad_noalloc_against_host_column_sums():
         msg = __import__("ctypes").create_string_buffer(256)
         rc = A.load_library().alexnet_bias_grad_noalloc(A._ptr(x), bad_rows, bad_c, A._ptr(torch.zeros(bad_c, device="cuda")), None, msg, 256)
         assert rc == A.ERR_ARG and word in msg.value.decode(), (bad_rows, bad_c, msg.value)
+
+
+def test_bias_grad_noalloc_after_calls_that_overlapped():
+    """Calls that overlap on the GPU (two streams, no order between them, different numbers of row splits) may spoil their own
+    sums, as the header says, and nothing else: the ordered calls that follow are exact, eager ones as well as the replay of
+    one captured before."""
+    from paper_1412_2302_b200 import alexnet as A
+    gen = torch.Generator().manual_seed(29)
+    x, y, z = ((torch.randint(-64, 65, (rows, 64), generator=gen) / 64.0).to(torch.bfloat16).cuda() for rows in (150000, 9000, 6500))
+    db = [torch.empty(64, device="cuda") for _ in range(3)]
+    st = [torch.cuda.Stream(), torch.cuda.Stream()]
+    A.bias_grad_noalloc(z, db[2], stream=st[0])                      # set up before the capture
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=st[0]):
+        A.bias_grad_noalloc(z, db[2], stream=st[0])
+    for _ in range(20):
+        for _ in range(4):
+            A.bias_grad_noalloc(x, db[0], stream=st[0])
+            A.bias_grad_noalloc(y, db[1], stream=st[1])
+        torch.cuda.synchronize()
+        db[2].fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(db[2].cpu().numpy().astype(np.float64), host_colsum(z))
+        for t, out in ((y, db[1]), (x, db[0]), (y, db[1])):
+            out.fill_(float("nan"))
+            torch.cuda.synchronize()
+            A.bias_grad_noalloc(t, out, stream=st[0])
+            torch.cuda.synchronize()
+            # multiples of 1/64: the fp32 sums are exact
+            assert np.array_equal(out.cpu().numpy().astype(np.float64), host_colsum(t))
