@@ -377,7 +377,7 @@ def bias_grad_noalloc(dy, db, stream=None):
     msg = getattr(_local, "msg", None)
     if msg is None:
         msg = _local.msg = ctypes.create_string_buffer(256)      # kept per thread: allocating it costs as much as the call
-    rows, ch = dy.shape
-    rc = lib.alexnet_bias_grad_noalloc(dy.data_ptr(), rows, ch, db.data_ptr(), stream.cuda_stream if stream is not None else None, msg, 256)
+    shape = dy.shape
+    rc = lib.alexnet_bias_grad_noalloc(dy.data_ptr(), int(shape[0]), int(shape[1]), db.data_ptr(), stream.cuda_stream if stream is not None else None, msg, 256)
     if rc != OK:
         raise AlexNetError(rc, msg.value.decode())

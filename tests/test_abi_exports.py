@@ -87,3 +87,16 @@ def test_every_kernel_is_loaded_with_the_handle():
     assert len(names) > 30 and {"conv_kernel", "wgrad_reduce_kernel", "init_kernel"} <= names
     for n in sorted(names):
         assert re.search(r"\b%s\b" % n, listed), n
+
+
+def test_bias_grad_noalloc_takes_trailing_dimensions(lib):
+    """The binding reads the first two sizes of dy and passes them on ([rows, channels, 1, 1] of a convolution's output is as good
+    as [rows, channels]); here the NULL pointer is what the library refuses, before it looks for a GPU."""
+    class Dy:
+        shape = (4, 8, 1, 1)
+
+        def data_ptr(self):
+            return 0
+    with pytest.raises(A.AlexNetError, match="NULL pointer") as e:
+        A.bias_grad_noalloc(Dy(), Dy())
+    assert e.value.code == A.ERR_ARG
