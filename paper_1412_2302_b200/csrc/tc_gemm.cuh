@@ -347,14 +347,15 @@ __device__ __forceinline__ void epi_chunk(const P& p, uint32_t* v, bool zero, bo
 // the next slab overlap.
 // An SM has only four or eight epilogue warps, so a slab is a latency chain and not a throughput problem: all its TMEM
 // columns are read before the first wait, with the bias of the first half in flight beside them, pairs of columns are
-// added as packed fp32, and one conversion instruction applies the ReLU and packs.  The ReLU mask of a backward slab is
-// fetched by the caller one slab ahead.
+// added as packed fp32, and the ReLU is applied to the packed result.  The ReLU mask of a backward slab is fetched by the
+// caller one slab ahead.
 constexpr uint32_t kEpiStageBytes = 4096;
-__device__ __forceinline__ uint32_t cvt_relu_bf16x2(float lo, float hi) {
-    uint32_t d; asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo)); return d;
-}
 __device__ __forceinline__ uint32_t cvt_bf16x2(float lo, float hi) {
     uint32_t d; asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo)); return d;
+}
+// with the ReLU of every other path, fmaxf(x, 0): the maximum drops a NaN (the conversion's own .relu would keep it)
+__device__ __forceinline__ uint32_t cvt_relu_bf16x2(float lo, float hi) {
+    uint32_t d; asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(cvt_bf16x2(lo, hi)), "r"(0u)); return d;
 }
 // the 128 bytes of the ReLU mask under a lane's row of a slab; mp == nullptr: a row outside the tensor
 __device__ __forceinline__ void epi_mask_load(const uint4* mp, uint4* mk) {

@@ -259,6 +259,37 @@ def test_fused_lrn_pool_forward_argmax_bit_exact(net, which, ta, tn, tp, targ, t
     assert np.array_equal(net.get_tensor(targ).reshape(arg.shape).astype(np.uint8), arg)     # bit exact
 
 
+@pytest.mark.parametrize("batch", [2, 40])
+@pytest.mark.parametrize("flags", [0, 16, 32])
+def test_relu_turns_nan_into_zero_in_every_tile_shape(batch, flags):
+    """ReLU is max(x, 0) with the maximum that drops a NaN, whatever tile shape (and epilogue) a layer's batch and the CTA-pair
+    flags give: with one NaN in the input, the outputs whose window contains it are zero and all others keep their bits."""
+    from paper_1412_2302_b200.alexnet import AlexNet
+    n = AlexNet(batch=batch, seed=SEED, mean_image=synth.mean_image(SEED), flags=flags)
+    n.set_params((np.random.default_rng(12).integers(-64, 65, size=n.param_count) / 256.0).astype(np.float32))
+    for name, tin, tout, shp in CONVS:
+        x = synth.bf16_grid(SEED, tag(name), (batch,) + shp, -1, 1)
+        res = []
+        for bad in (False, True):
+            if bad:
+                x[batch - 1, 1, 7, 6] = np.nan       # (channel 1: the first group)
+            n.set_tensor(tin, x)
+            n.run_op(name.upper() + "_FWD")
+            n.sync()
+            res.append(n.get_tensor(tout).reshape(batch, O.CONV[name]["cout"], -1, 55 if name == "conv1" else shp[2]))
+        clean, got = res
+        assert not np.isnan(got).any(), name
+        if name == "conv1":                          # (its zero-padded 12 x 12 filter reaches one row and column further)
+            hit = np.s_[batch - 1, :, 0:2, 0:2]
+        else:
+            k = 2 if name == "conv2" else 1
+            hit = np.s_[batch - 1, :O.CONV[name]["cout"] // O.CONV[name]["g"], 7 - k:8 + k, 6 - k:7 + k]
+        assert (clean[hit] > 0).any() and (got[hit] == 0).all(), name
+        clean[hit] = got[hit] = 0
+        assert np.array_equal(clean, got), name
+    n.close()
+
+
 @pytest.mark.parametrize("batch", [1, 20, 40])
 def test_fused_lrn_pool_rows_per_block(batch):
     """The fused forward kernel with one, two and three output rows per block (the rule takes them at these batches; 27 and 13
