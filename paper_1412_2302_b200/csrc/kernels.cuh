@@ -410,7 +410,8 @@ __global__ void __launch_bounds__((WI + 1) / 2 * CV, MINB) lrn_pool_fwd_kernel(c
     const int lane = threadIdx.x & 31;
     const bool has_l = ch > 0, has_r = ch < CPR - 1;
     const bool ld_l = has_l && (lane == 0 || cv == 0), ld_r = has_r && (lane == 31 || threadIdx.x == NT - 1 || cv == CV - 1);
-    const unsigned mask = __activemask();      // the last warp of a block may be partial
+    // the lanes that exist: the last warp of a block may be partial
+    const unsigned mask = NT % 32 && threadIdx.x >= NT / 32 * 32 ? (1u << NT % 32) - 1u : ~0u;
     uint4 v0, v1; uint32_t l0 = 0u, l1 = 0u, r0 = 0u, r1 = 0u;
     auto fetch = [&]() {
         v0 = __ldg(ap); v1 = __ldg(ap + CPR);
