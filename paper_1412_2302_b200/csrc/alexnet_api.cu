@@ -177,7 +177,6 @@ struct Replica {
     bool n_stale[2], dn_stale[2];
     // plans
     Plan conv_fwd[5][2], conv_bwd[5], conv_wg[5][2], fc_fwd[3], fc_bwd[3];
-    std::vector<Plan> eval_conv[2];    // per slot: the forward convolutions of every chunk of an evaluation from host memory
     Plan conv_bwd_beside[5];    // the same data gradients on the SMs that the FC updates leave free (conv3-5)
     Plan fc_wg_plain[3];    // the FC weight gradient stored (alexnet_forward_backward)
     Plan fc_upd[3];         // ... with the momentum update of the FC weights; it also stores the gradient unless the handle was
@@ -496,6 +495,7 @@ void finish_conv_plan(const alexnet* h, Plan& P) {
     c.splits = (c.asteps_total + per - 1) / per;
     c.asteps_per_split = per;
     c.tiles_total = c.m_tiles * c.n_tiles * c.groups * c.splits;
+    c.m_tile0 = 0; c.m_tiles_all = c.m_tiles;
     if (c.cpg < 1) c.cpg = 1;
     if (c.cg < 1) c.cg = 1;
     const size_t a_bytes = (size_t)c.MH * c.cpg * c.a_box_rows * 128, b_bytes = (size_t)(c.BN / c.cg) * 128;
@@ -533,10 +533,10 @@ int conv_out_map(alexnet* h, tc::ConvParams& p, const void* out, int ldo, long l
     return make_tm_out(h, &p.tmOut, out, false, (uint64_t)ldo, (uint64_t)M, 1, (uint64_t)ldo * 2, (uint64_t)ldo * 2 * (uint64_t)M);
 }
 
-int plan_conv_fwd(alexnet* h, Plan& P, const ConvL& c, const bf16* in, const bf16* wsh, const float* bias, bf16* out, int images) {
+int plan_conv_fwd(alexnet* h, Plan& P, const ConvL& c, const bf16* in, const bf16* wsh, const float* bias, bf16* out) {
     memset(&P, 0, sizeof(P));
     tc::ConvParams& p = P.c;
-    const long long M = (long long)images * c.gin.Hp * c.gin.Wp;
+    const long long M = (long long)h->B * c.gin.Hp * c.gin.Wp;
     const int gp = c.gin.Wp;
     p.kh = p.kw = c.k; p.chunks = (c.cig + 63) / 64; p.kk = c.cig == 48 ? 3 : 4;
     const ConvShape sh = choose_conv_shape(h, M, c.cog, c.groups, p.kh, p.kw, p.chunks, p.kk);
@@ -764,7 +764,7 @@ int build_plans(alexnet* h, int r) {
         const ConvL& c = L.conv[l];
         for (int s = 0; s < 2; ++s) {
             const bf16* x = l == 0 ? R.x0[s] : in[l];
-            if ((rc = plan_conv_fwd(h, R.conv_fwd[l][s], c, x, R.shadow + c.w_off, R.w + c.b_off, out[l], h->B))) return rc;
+            if ((rc = plan_conv_fwd(h, R.conv_fwd[l][s], c, x, R.shadow + c.w_off, R.w + c.b_off, out[l]))) return rc;
             if ((rc = plan_conv_wg(h, R.conv_wg[l][s], l, c, dyv[l], x))) return rc;
         }
         if ((rc = plan_conv_bwd(h, R.conv_bwd[l], c, dyv[l], R.wt + c.wt_off, maskv[l], dxv[l]))) return rc;
@@ -790,29 +790,11 @@ int build_plans(alexnet* h, int r) {
 // copied (3.6 us per image); what is left behind the last copy is one chunk's time and the FC layers.  A chunk's dependent launches
 // cost a fixed time and small grids fill the machine badly, so chunks below about 50 images take longer than the copy they should
 // hide behind and the delay adds up from chunk to chunk, while two chunks can be smaller, since only the first has to keep up.
-// Measured, chunks of at least 40 / 54 / 64 / 80 / 100 images: 256 images 1301 / 1207 / 1206 / 1233 / 1308 us, 512 images 2299 / 2231 /
-// 2180 / 2199 / 2234; two chunks against one: 72 images 537 -> 520, 64 488 -> 468, 56 452 -> 441, 48 411 -> 419.
-constexpr int kEvalChunk = 64, kEvalTwoChunks = 56;
+// Measured, 3 / 4 / 5 chunks: 256 images 1238 / 1217 / 1310 us; 4 / 5 / 6: 320 images 1495 / 1483 / 1574; 7 / 8 / 9: 512 images 2201 / 2195 /
+// 2259; one / two: 56 images 450 / 473, 64 487 / 503, 72 538 / 524, 80 572 / 545.
+constexpr int kEvalChunk = 64, kEvalTwoChunks = 68;
 int eval_chunks(int B) { return std::max(B >= kEvalTwoChunks ? 2 : 1, B / kEvalChunk); }
 inline int chunk_begin(int B, int chunks, int c) { return (int)((long long)B * c / chunks); }
-int build_eval_plans(alexnet* h, int r, int slot) {
-    Replica& R = h->rep[r];
-    const Layout& L = h->L;
-    const int chunks = eval_chunks(h->B);
-    std::vector<Plan> plans((size_t)chunks * 5);
-    const bf16* in[5] = {R.x0[slot], R.p1, R.p2, R.a3, R.a4};
-    bf16* out[5] = {R.a1, R.a2, R.a3, R.a4, R.a5};
-    for (int c = 0; c < chunks; ++c) {
-        const int i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
-        for (int l = 0; l < 5; ++l) {
-            const ConvL& q = L.conv[l];
-            const size_t off = (size_t)i0 * q.gin.Hp * q.gin.Wp;      // input and output share a grid
-            if (int rc = plan_conv_fwd(h, plans[(size_t)c * 5 + l], q, in[l] + off * q.cin, R.shadow + q.w_off, R.w + q.b_off, out[l] + off * q.cout, n)) return rc;
-        }
-    }
-    R.eval_conv[slot].swap(plans);
-    return ALEXNET_OK;
-}
 
 // ---------------------------------------------------------------- launches
 inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
@@ -1219,14 +1201,33 @@ void forward(alexnet* h, int r, int slot, cudaStream_t st, bool eval) {
     op_pool_fwd(h, r, 2, st);
     forward_fc(h, r, slot, st, eval);
 }
-// the convolution layers of one chunk of an evaluation batch
-void forward_conv_chunk(alexnet* h, int r, int slot, int c, int chunks, cudaStream_t st) {
-    const std::vector<Plan>& P = h->rep[r].eval_conv[slot];
-    const int i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
-    launch_gemm(h, P[5 * c], st); op_lrn_pool_fwd(h, r, 0, st, i0, n);
-    launch_gemm(h, P[5 * c + 1], st, true); op_lrn_pool_fwd(h, r, 1, st, i0, n);
-    launch_gemm(h, P[5 * c + 2], st, true); launch_gemm(h, P[5 * c + 3], st, true); launch_gemm(h, P[5 * c + 4], st, true);
-    op_pool_fwd(h, r, 2, st, i0, n);
+// How far the convolution layers of an evaluation in chunks have come: the m tiles done of each layer, and the images complete behind it
+struct ConvProgress { int tiles[5], images[5]; };
+// The convolution layers as far as `avail` images in X0 allow.  The tiles are those of the whole batch's launches, with their
+// shapes and their order of summation, so that the chunks do not show in the results.  A layer takes the tiles whose rows are
+// all there; a tile that ends beyond them waits for the next chunk, and with it the image that it ends in.  (A halo reaches
+// into rows that are not there yet for pad positions only, and these are stored as zeros.)
+// Launches planned per chunk with tile shapes of its own, which sum in an order of their own, are up to 2% faster (256 images 1206
+// us against 1220, 128 720 against 735); computing the tiles at a boundary with both chunks is not (1229 us, 100 images 642
+// against 632).
+void forward_conv_chunk(alexnet* h, int r, int slot, int avail, ConvProgress& q, cudaStream_t st) {
+    for (int l = 0; l < 5; ++l) {
+        Plan P = h->rep[r].conv_fwd[l][slot];
+        const Grid& g = h->L.conv[l].gin;              // input and output share a grid
+        const long long rows = (long long)g.Hp * g.Wp, tile_rows = 128LL * P.c.MH * P.c.cg;
+        const int t0 = q.tiles[l], t1 = avail == h->B ? P.c.m_tiles : (int)(avail * rows / tile_rows);
+        if (t1 > t0) {
+            P.c.m_tile0 = t0; P.c.m_tiles = t1 - t0;
+            P.c.tiles_total = P.c.m_tiles * P.c.n_tiles * P.c.groups;
+            P.grid = P.c.cg * std::min(P.c.tiles_total, h->sm_count / P.c.cg);
+            launch_gemm(h, P, st, l > 0);
+        }
+        if (avail < h->B) avail = (int)(t1 * tile_rows / rows);
+        const int i0 = q.images[l], n = avail - i0;
+        if (n > 0 && l < 2) op_lrn_pool_fwd(h, r, l, st, i0, n);
+        if (n > 0 && l == 4) op_pool_fwd(h, r, 2, st, i0, n);
+        q.tiles[l] = t1; q.images[l] = avail;
+    }
 }
 // update: the FC weights are updated here, by their weight-gradient kernels (the rest of the parameters by op_update)
 void forward_backward(alexnet* h, int r, int slot, cudaStream_t st, bool update, bool defer_conv_reduce) {
@@ -1754,20 +1755,19 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     const bool on_device = cudaPointerGetAttributes(&at, images) == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
     cudaGetLastError();
     const int chunks = on_device || h->prof ? 1 : eval_chunks(h->B);
-    if (chunks > 1 && R.eval_conv[s].empty())
-        if (int rc = build_eval_plans(h, replica, s)) return rc;
     while ((int)h->ev_chunk.size() < chunks) {
         cudaEvent_t e;
         CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         h->ev_chunk.push_back(e);
     }
+    ConvProgress done = {};
     for (int c = 0; c < chunks; ++c) {
         const size_t i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
         CK(cudaMemcpyAsync(R.stage[s] + i0 * 196608, images + i0 * 196608, n * 196608, cudaMemcpyDefault, h->ls));
         CK(cudaEventRecord(h->ev_chunk[c], h->ls));
         CK(cudaStreamWaitEvent(h->cs, h->ev_chunk[c], 0));
         op_preprocess(h, replica, s, 0, h->cs, true, lsrc, (int)i0, (int)n);
-        if (chunks > 1) forward_conv_chunk(h, replica, s, c, chunks, h->cs);
+        if (chunks > 1) forward_conv_chunk(h, replica, s, (int)(i0 + n), done, h->cs);
     }
     if (chunks > 1) forward_fc(h, replica, s, h->cs, true);
     else forward(h, replica, s, h->cs, true);

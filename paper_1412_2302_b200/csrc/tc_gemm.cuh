@@ -682,8 +682,10 @@ struct ConvParams {
     int tma_store;
     int m_tiles, n_tiles, groups, splits;   // tile decomposition (m fastest, then n, group, k split)
     int tiles_total;
-    int rot_mod;        // tile t starts its reduction at (filter row, chunk) step (t % rot_mod) % steps of its range: neighbouring tiles
-                        // start at different steps, whatever CTA works on them
+    int m_tile0, m_tiles_all;   // the launch covers the m tiles m_tile0 .. m_tile0 + m_tiles - 1 of a layer of m_tiles_all (all of them, but
+                                // for the chunks of an evaluation)
+    int rot_mod;        // tile t of the layer starts its reduction at (filter row, chunk) step (t % rot_mod) % steps of its range:
+                        // neighbouring tiles start at different steps, whatever CTA and launch works on them
     int b_res;          // 1: all kh*kw weight tiles of the layer fit in one group slot and stay there for the whole CTA (one
                         // n tile, one group, one chunk, no split: conv1), loaded once instead of once per tile
     int cg;             // 1, or 2: CTA pairs (clusters of two) work on tiles of 2 x MH halves with cta_group::2 instructions
@@ -743,6 +745,8 @@ struct ConvCursor {
         g = r % q.groups;
         z = r / q.groups;
     }
+    // number of the tile in the whole layer's list
+    __device__ __forceinline__ int index(const ConvParams& q) const { return q.m_tile0 + m_tile + q.m_tiles_all * rest; }
     int stride;      // tile-list stride: CTAs of the grid, or CTA pairs
     __device__ __forceinline__ void init(const ConvParams& q, int first, int step) {
         stride = step;
@@ -842,13 +846,13 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             int sa = 0; uint32_t pha = 0;
             bool ok = true;
             for (int tile = vb; tile < p.tiles_total && ok; tile += vgrid, tc.next(p)) {
-                const int m0 = tc.m_tile * tile_rows + row0;
+                const int m0 = (p.m_tile0 + tc.m_tile) * tile_rows + row0;
                 const int a_begin = tc.z * per;
                 const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
                 // the reduction order is free: neighbouring tiles start at different (filter row, chunk) steps so that the SMs
                 // do not all ask L2 for the same weight tile at the same moment
                 const int a_end = a_begin + nsteps;
-                int a = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);
+                int a = a_begin + (int)(((unsigned)tc.index(p) % (unsigned)p.rot_mod) % (unsigned)nsteps);
                 int ky = a / p.chunks, ch = a - ky * p.chunks;
                 const int ky0 = a_begin / p.chunks, ch0 = a_begin - ky0 * p.chunks;
                 const int xa = p.a_x0 + tc.g * p.a_gx;
@@ -891,7 +895,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 // the reduction order is free: neighbouring tiles start at different (filter row, chunk) steps so that the SMs
                 // do not all ask L2 for the same weight tile at the same moment
                 const int a_end = a_begin + nsteps;
-                int a = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);
+                int a = a_begin + (int)(((unsigned)tc.index(p) % (unsigned)p.rot_mod) % (unsigned)nsteps);
                 int ky = a / p.chunks, ch = a - ky * p.chunks;
                 const int ky0 = a_begin / p.chunks, ch0 = a_begin - ky0 * p.chunks;
                 const int yb = tc.g * p.b_g_rows + n0;
@@ -936,7 +940,8 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             for (int tile = vb; tile < p.tiles_total && ok; tile += vgrid) {
                 const int a_begin = z * per;
                 const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
-                int ares = a_begin + (int)(((unsigned)tile % (unsigned)p.rot_mod) % (unsigned)nsteps);      // resident filter: the producer's rotation of the filter rows
+                // resident filter (one n tile, one group): the producer's rotation of the filter rows
+                int ares = a_begin + (int)(((unsigned)(p.m_tile0 + tile) % (unsigned)p.rot_mod) % (unsigned)nsteps);
                 TL(const long long cc0 = clock64();)
                 ok = mbar_wait_warp(acce0 + 8u * ab, aph ^ 1u, abort_flag);
                 TL(wC += clock64() - cc0;)
@@ -998,7 +1003,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
         bool ok = true;
         const uint32_t acce_leader = CG == 2 ? mapa_u32(acce0, 0) : acce0;
         for (int tile = vb; tile < p.tiles_total && ok; tile += vgrid, tc.next(p)) {
-            const int m0 = tc.m_tile * tile_rows + row0, n0 = tc.n_tile * BN, g = tc.g;
+            const int m0 = (p.m_tile0 + tc.m_tile) * tile_rows + row0, n0 = tc.n_tile * BN, g = tc.g;
             const int a_begin = tc.z * per;
             const int nsteps = min(p.asteps_total, a_begin + per) - a_begin;
             // with two sets of epilogue warps, the (row half, slab) units of the tile alternate between the sets

@@ -65,10 +65,10 @@ def test_eval_batch_against_oracle(inverted):
 
 @pytest.mark.parametrize("B", [55, 56, 57, 129, 193])
 def test_eval_in_chunks_agrees_with_one_pass(B):
-    """Images in host memory are evaluated in chunks (one up to 55 images, then two, more from 192 on; 57, 129 and 193 do not
-    divide evenly), images on the device in one pass.  Both compute the same sums in fp32, in an order that depends on the tile
-    numbering, and each is within TOL of the oracle by the test above: the logits agree within 2 TOL, the mean loss to the
-    same relative bound, and the counts are exact for the logits of each."""
+    """Images in host memory are evaluated in chunks (one up to 67 images, then two, more from 192 on; 129 and 193 do not
+    divide evenly), images on the device in one pass.  Each is within TOL of the oracle by the test above: the logits agree within
+    2 TOL, the mean loss to the same relative bound (the test below asks for the same bits), and the counts are exact for the
+    logits of each."""
     from paper_1412_2302_b200 import alexnet as A
     seed = synth.BASE_SEED + 32
     net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
@@ -85,4 +85,25 @@ def test_eval_in_chunks_agrees_with_one_pass(B):
         got[where] = z, loss
     assert rel(got["host"][0], got["device"][0]) < 2 * TOL
     assert abs(got["host"][1] - got["device"][1]) < 2 * TOL * max(1.0, abs(got["device"][1]))
+    net.close()
+
+
+@pytest.mark.parametrize("B", [67, 68, 69, 129, 193, 260])
+def test_eval_in_chunks_is_bit_for_bit_the_one_pass(B):
+    """Around the smallest batch in two chunks, and with chunks that do not divide evenly.  The chunks of an evaluation from host memory take the tiles of the whole batch's launches, so where the images come from does
+    not show: logits, counts and loss are those of the one pass over images on the device, bit for bit."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed = synth.BASE_SEED + 33
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    net.set_params(synth.init_params(seed, variance_preserving=True, bias=0.1))
+    gen = torch.Generator().manual_seed(B)
+    lab = torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen)
+    for _ in range(2):                                 # (a second batch: nothing of the first may show)
+        img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen)
+        got = []
+        for im, lb in ((img.pin_memory(), lab.pin_memory()), (img.cuda(), lab.cuda())):
+            torch.cuda.synchronize()
+            got.append((net.eval_batch(0, im, lb), net.get_tensor("P5"), net.get_tensor("Z")))
+        assert got[0][0] == got[1][0]
+        assert np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][2], got[1][2])
     net.close()
