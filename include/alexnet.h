@@ -329,12 +329,16 @@ uint64_t alexnet_launch_count(const alexnet_t* h);
  * kernel class the summed device time (ms) and the number of launches recorded
  * since the last read, and clears the record.  Index 0 = conv_kernel on
  * convolutions (forward and backward-data), 1 = wgrad_kernel (convolution
- * weight gradients), 2 = gemm_kernel (FC backward-data and weight gradients),
+ * weight gradients), 2 = gemm_kernel (FC backward-data and weight gradients)
+ * and fc_update_kernel (FC weight gradients with the update),
  * 3 = the FC forward passes (fc_chain_kernel: one launch for the three layers;
  * or conv_kernel's 1 x 1 case, one launch per layer; HBM-bound at batch 128).
- * Both arrays have four entries. */
+ * Both arrays have four entries.  profile_read_kinds does the same for the
+ * first n of five classes, where index 2 is gemm_kernel alone and 4 is
+ * fc_update_kernel (HBM-bound); both arrays have n entries. */
 int alexnet_profile(alexnet_t* h, int enable);
 int alexnet_profile_read(alexnet_t* h, double* ms4, uint64_t* launches4);
+int alexnet_profile_read_kinds(alexnet_t* h, double* ms, uint64_t* launches, int n);
 
 /* Per-role timeline of the convolution kernel, for the timeline tool.  Only a
  * library built with -DALEXNET_TIMELINE records it (python -m

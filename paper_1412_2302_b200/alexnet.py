@@ -39,7 +39,7 @@ EXPORTS = ["alexnet_param_count", "alexnet_workspace_bytes", "alexnet_create", "
            "alexnet_loader_create", "alexnet_loader_next", "alexnet_loader_release", "alexnet_loader_destroy",
            "alexnet_forward_backward", "alexnet_apply_update", "alexnet_update_and_average", "alexnet_param_regions",
            "alexnet_scale_and_refresh", "alexnet_create_error", "alexnet_debug_expire_wait", "alexnet_set_color_augmentation", "alexnet_average_received", "alexnet_param_layout",
-           "alexnet_stream_wait_fc_gradients", "alexnet_timeline_read"]
+           "alexnet_stream_wait_fc_gradients", "alexnet_timeline_read", "alexnet_profile_read_kinds"]
 
 
 class Config(ctypes.Structure):
@@ -105,6 +105,7 @@ def load_library():
     L.alexnet_launch_count.argtypes = [vp]
     L.alexnet_profile.argtypes = [vp, i32]
     L.alexnet_profile_read.argtypes = [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(u64)]
+    L.alexnet_profile_read_kinds.argtypes = [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(u64), i32]
     L.alexnet_sync.argtypes = [vp]
     L.alexnet_last_error.restype = ctypes.c_char_p
     L.alexnet_last_error.argtypes = [vp]
@@ -303,10 +304,16 @@ class AlexNet:
         self._ck(self.lib.alexnet_profile(self.h, 1 if enable else 0))
 
     def profile_read(self):
-        """Per tensor-core kernel class (conv_kernel on convolutions, wgrad_kernel, gemm_kernel, conv_kernel on FC
-        forward): summed device time in ms and launches since the last read, as two 4-tuples."""
+        """Per tensor-core kernel class (conv_kernel on convolutions, wgrad_kernel, gemm_kernel and fc_update_kernel, conv_kernel
+        on FC forward): summed device time in ms and launches since the last read, as two 4-tuples."""
         ms, n = (ctypes.c_double * 4)(), (ctypes.c_uint64 * 4)()
         self._ck(self.lib.alexnet_profile_read(self.h, ms, n))
+        return tuple(ms), tuple(int(v) for v in n)
+
+    def profile_read_kinds(self):
+        """The same as two 5-tuples, with gemm_kernel alone as the third class and fc_update_kernel as the fifth."""
+        ms, n = (ctypes.c_double * 5)(), (ctypes.c_uint64 * 5)()
+        self._ck(self.lib.alexnet_profile_read_kinds(self.h, ms, n, 5))
         return tuple(ms), tuple(int(v) for v in n)
 
     @property

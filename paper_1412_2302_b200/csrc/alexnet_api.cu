@@ -228,7 +228,7 @@ struct alexnet {
     // optional per-launch timing of the GEMM kernel (event pairs on the launching stream)
     bool prof;
     std::vector<cudaEvent_t> prof_ev;
-    std::vector<int> prof_kind;     // kernel of each recorded pair: 0 conv_kernel (convolutions), 1 wgrad_kernel, 2 gemm_kernel,
+    std::vector<int> prof_kind;     // kernel of each recorded pair: 0 conv_kernel (convolutions), 1 wgrad_kernel, 2 gemm_kernel, 4 fc_update_kernel,
                                     // 3 conv_kernel (FC forward)
     size_t prof_used;
 };
@@ -843,7 +843,7 @@ void launch_gemm(alexnet* h, const Plan& P0, cudaStream_t st, bool early_weights
     else launch_k(tc::gemm_kernel, P.grid, tc::kThreads, P.smem, st, P.p);
     if (h->prof) {
         cudaEventRecord(h->prof_ev[h->prof_used + 1], st);
-        h->prof_kind.push_back(P.conv ? (P.c.kh == 1 && P.c.cpg > 1 ? 3 : 0) : P.wgrad ? 1 : 2);
+        h->prof_kind.push_back(P.conv ? (P.c.kh == 1 && P.c.cpg > 1 ? 3 : 0) : P.wgrad ? 1 : P.upd ? 4 : 2);
         h->prof_used += 2;
     }
     h->launches++;
@@ -1976,20 +1976,32 @@ int alexnet_profile(alexnet_t* h, int enable) {
     return ALEXNET_OK;
 }
 
-int alexnet_profile_read(alexnet_t* h, double* ms3, uint64_t* launches3) {
-    if (!h || !ms3 || !launches3) return ALEXNET_ERR_ARG;
+int alexnet_profile_read_kinds(alexnet_t* h, double* ms, uint64_t* launches, int n) {
+    if (!h || !ms || !launches || n < 1) return ALEXNET_ERR_ARG;
     CK(cudaStreamSynchronize(h->ls));
     CK(cudaStreamSynchronize(h->cs));
-    for (int k = 0; k < 4; ++k) { ms3[k] = 0.0; launches3[k] = 0; }
+    for (int k = 0; k < n; ++k) { ms[k] = 0.0; launches[k] = 0; }
     for (size_t i = 0; i + 1 < h->prof_used; i += 2) {
         float t = 0.f;
         CK(cudaEventElapsedTime(&t, h->prof_ev[i], h->prof_ev[i + 1]));
         const int k = h->prof_kind[i / 2];
-        ms3[k] += t;
-        launches3[k]++;
+        if (k >= n) continue;
+        ms[k] += t;
+        launches[k]++;
     }
     h->prof_used = 0;
     h->prof_kind.clear();
+    return ALEXNET_OK;
+}
+
+int alexnet_profile_read(alexnet_t* h, double* ms4, uint64_t* launches4) {
+    if (!h || !ms4 || !launches4) return ALEXNET_ERR_ARG;
+    double ms[5];
+    uint64_t n[5];
+    if (int rc = alexnet_profile_read_kinds(h, ms, n, 5)) return rc;
+    ms[2] += ms[4]; n[2] += n[4];
+    memcpy(ms4, ms, 4 * sizeof(double));
+    memcpy(launches4, n, 4 * sizeof(uint64_t));
     return ALEXNET_OK;
 }
 

@@ -929,3 +929,20 @@ def test_refused_launch_names_its_kernel():
     net.scale_and_refresh(0, 0.5)
     assert np.array_equal(net.get_params(0, 0), 0.5 * w)
     net.close()
+
+
+def test_profile_kinds_tell_the_fc_updates_from_the_gemms():
+    """One step under per-kernel timing: nine convolution launches, five convolution weight gradients, three FC data gradients
+    (gemm_kernel), three FC forward passes, three FC updates; the four-class form counts the updates with the GEMMs; a step
+    without its update has six GEMMs and no update."""
+    net = make(2, seed=BASE + 16)
+    net.set_params(synth.init_params(BASE + 16))
+    net.profile(True)
+    for step, (call, kinds, four) in enumerate(((net.train_step, (9, 5, 3, 3, 3), (9, 5, 6, 3)),
+                                                (net.forward_backward, (9, 5, 6, 3, 0), (9, 5, 6, 3)))):
+        for read, want in ((net.profile_read_kinds, kinds), (net.profile_read, four)):
+            load(net, 0, BASE + 16, step, 2)
+            call(0)
+            ms, n = read()
+            assert n == want and all((t > 0) == (k > 0) for t, k in zip(ms, n)), (ms, n)
+    net.close()
