@@ -269,15 +269,17 @@ struct Carver {
     }
 };
 
-// k splits of a GEMM with `tiles` output tiles and `steps` k-steps: fill one wave of 148 CTAs, never more (a second,
+constexpr int kSms = 148;    // of a B200: for sizes that must be known without a device (the workspace and what depends on it)
+
+// k splits of a GEMM with `tiles` output tiles and `steps` k-steps: fill one wave of CTAs, never more (a second,
 // nearly empty round costs a whole tile time), and keep at least two k-steps per split
 int pick_splits(int tiles, int steps) {
-    int s = 148 / tiles;
+    int s = kSms / tiles;
     if (s > steps / 2) s = steps / 2;
     if (s < 1) s = 1;
     return s;
 }
-int conv_wg_splits(const ConvL& c, int B, int sm_count = 148) {
+int conv_wg_splits(const ConvL& c, int B, int sm_count = kSms) {
     // one wave: (filter rows x 64-channel input blocks x 128-channel output blocks x groups) units times the row splits
     const long long M = (long long)B * c.gin.Hp * c.gin.Wp;
     const int steps = (int)((M + tc::kWgRows - 1) / tc::kWgRows);
@@ -416,7 +418,7 @@ int make_tm_rows(alexnet* h, CUtensorMap* tm, const void* ptr, bool f32, uint64_
 void finish_plan(const alexnet* h, Plan& P) {
     tc::GemmParams& p = P.p;
     if (p.a_bytes == 0) p.a_bytes = tc::kABytes;
-    const int stage_bytes = p.a_bytes + tc::b_stage_bytes(p.mode, p.BN);
+    const int stage_bytes = p.a_bytes + tc::b_stage_bytes(p.BN);
     int stages = (227 * 1024 - 2048 - 4 * (int)tc::kEpiStageBytes) / stage_bytes;
     if (stages > tc::kMaxStages) stages = tc::kMaxStages;
     p.stages = stages;
@@ -550,7 +552,7 @@ int plan_conv_fwd(alexnet* h, Plan& P, const ConvL& c, const bf16* in, const bf1
     for (int kx = 0; kx < c.k; ++kx) p.tap_off[kx] = kx;
     p.epi = tc::EPI_BF16; p.n_valid = c.cog; p.ldo = c.cout; p.out_gx = c.cog;
     p.Hp = c.gout.Hp; p.Wp = c.gout.Wp; p.H = c.gout.H; p.W = c.gout.W;
-    p.relu = 1; p.mask_scale = 1.f; p.bias = bias; p.mask = nullptr; p.out = out; p.status = h->status;
+    p.relu = 1; p.bias = bias; p.mask = nullptr; p.out = out; p.status = h->status;
     int rc;
     if ((rc = make_tm(h, &p.tmA, in, c.cin, M, (uint64_t)c.cin * 2, p.a_box_rows))) return rc;
     if ((rc = make_tm(h, &p.tmB, wsh, c.cig, (uint64_t)c.taps * c.cout, (uint64_t)c.cig * 2, p.BN / p.cg))) return rc;
@@ -579,7 +581,7 @@ int plan_conv_bwd(alexnet* h, Plan& P, const ConvL& c, const bf16* dy, const bf1
     for (int kx = 0; kx < c.k; ++kx) p.tap_off[kx] = c.k - 1 - kx;
     p.epi = tc::EPI_BF16; p.n_valid = c.cig; p.ldo = c.cin; p.out_gx = c.cig;
     p.Hp = c.gin.Hp; p.Wp = c.gin.Wp; p.H = c.gin.H; p.W = c.gin.W;
-    p.relu = 0; p.mask_scale = 1.f; p.bias = nullptr; p.mask = mask; p.out = dx; p.status = h->status;
+    p.relu = 0; p.bias = nullptr; p.mask = mask; p.out = dx; p.status = h->status;
     int rc;
     if ((rc = make_tm(h, &p.tmA, dy, c.cout, M, (uint64_t)c.cout * 2, p.a_box_rows))) return rc;
     if ((rc = make_tm(h, &p.tmB, wt, c.cog, (uint64_t)c.taps * c.cin, (uint64_t)c.cog * 2, p.BN / p.cg))) return rc;
@@ -593,7 +595,7 @@ int plan_conv_wg(alexnet* h, Plan& P, int l, const ConvL& c, const bf16* dy, con
     const long long M = (long long)h->B * c.gin.Hp * c.gin.Wp;
     p.m_tiles = (c.cog + 127) / 128; p.n_tiles = (c.cig + 63) / 64; p.groups = c.groups; p.kh = c.k; p.kw = c.k;
     p.steps_total = (int)((M + tc::kWgRows - 1) / tc::kWgRows);
-    p.splits = conv_wg_splits(c, h->B, std::min(h->sm_count, 148));   // never more than the workspace was sized for
+    p.splits = conv_wg_splits(c, h->B, std::min(h->sm_count, kSms));   // never more than the workspace was sized for
     p.steps_per_split = (p.steps_total + p.splits - 1) / p.splits;
     p.splits = (p.steps_total + p.steps_per_split - 1) / p.steps_per_split;
     p.tiles_total = p.m_tiles * p.n_tiles * p.groups * p.kh * p.splits;
@@ -604,7 +606,7 @@ int plan_conv_wg(alexnet* h, Plan& P, int l, const ConvL& c, const bf16* dy, con
     for (int ky = 0; ky < c.k; ++ky) p.halo_shift[ky] = (ky - c.pad) * c.gin.Wp - c.pad;
     p.M_total = c.cog; p.n_valid = c.cig; p.ldo = c.cig; p.out_gx = c.cog;
     p.tap_stride = (long long)c.cout * c.cig; p.split_stride = (long long)c.taps * c.cout * c.cig;
-    p.epi = tc::EPI_F32; p.mask_scale = 1.f;
+    p.epi = tc::EPI_F32;
     p.out = h->ws + h->ws_conv_off[l]; p.status = h->status;
     p.bias_partial = h->bias_partial + (size_t)l * kBiasPartial; p.bias_ld = c.cout;
     int rc;
@@ -633,7 +635,7 @@ int plan_fc_fwd(alexnet* h, Plan& P, const FcL& f, const bf16* x, const bf16* ws
     p.a_box_rows = fc_box_rows(B);
     p.halo_shift[0] = 0; p.tap_off[0] = 0; p.tap_off[1] = p.a_box_rows;   // the second chunk's box follows the first in the stage
     p.epi = tc::EPI_F32; p.n_valid = f.N; p.ldo = f.N; p.split_stride = (long long)B * f.N;
-    p.mask_scale = 1.f; p.out = h->ws; p.status = h->status;
+    p.out = h->ws; p.status = h->status;
     int rc;
     if ((rc = make_tm(h, &p.tmA, x, f.K, B, (uint64_t)f.K * 2, p.a_box_rows))) return rc;
     if ((rc = make_tm(h, &p.tmB, wsh, f.K, f.N, (uint64_t)f.K * 2, p.BN))) return rc;
@@ -660,7 +662,7 @@ int plan_fc_bwd(alexnet* h, Plan& P, const FcL& f, const bf16* dy, const bf16* w
     p.mode = tc::MODE_KMN; p.epi = tc::EPI_F32;
     p.M_total = B; p.m_tiles = (B + 127) / 128; p.BN = 256; p.n_tiles = f.K / 256;
     p.groups = 1; p.taps_grid = 1; p.splits = fc_bwd_splits(f, B);
-    p.kk = 4; p.chunks = 1; p.steps_total = (f.N + 63) / 64;
+    p.kk = 4; p.steps_total = (f.N + 63) / 64;
     p.n_valid = f.K; p.ldo = f.K; p.split_stride = (long long)B * f.K;
     p.out = h->ws; p.status = h->status;
     int rc;
@@ -679,7 +681,7 @@ int plan_fc_wg(alexnet* h, Plan& P, const FcL& f, const bf16* dy, const bf16* x,
     const int B = h->B;
     p.mode = tc::MODE_MNMN; p.epi = tc::EPI_F32;
     p.M_total = f.N; p.m_tiles = (f.N + 127) / 128; p.BN = 256; p.n_tiles = f.K / 256;
-    p.groups = 1; p.taps_grid = 1; p.splits = 1; p.kk = 4; p.chunks = 1; p.steps_total = (B + 63) / 64;
+    p.groups = 1; p.taps_grid = 1; p.splits = 1; p.kk = 4; p.steps_total = (B + 63) / 64;
     p.n_valid = f.K; p.ldo = f.K;
     p.out = gout; p.status = h->status;
     int rc;
@@ -1124,7 +1126,7 @@ void op_update(alexnet* h, int r, cudaStream_t st, bool full = false, float gsca
     memset(&none, 0, sizeof(none));
     launch_k(kn::sgd_update_conv_kernel, L.tjobs.tile0[5], 256, 0, st, R.w, R.v, R.g, R.shadow, d,
              h->cfg.lr, h->cfg.momentum, R.wt, L.tjobs, gscale, 0LL, 0LL, 0.f, none);
-    launch_k(kn::sgd_update_kernel, fused ? 148 : 1184, 256, 0, st, R.w, R.v, R.g, R.shadow, (fused ? L.n_weights : L.fc[0].w_off) / 4,
+    launch_k(kn::sgd_update_kernel, fused ? h->sm_count : 1184, 256, 0, st, R.w, R.v, R.g, R.shadow, (fused ? L.n_weights : L.fc[0].w_off) / 4,
              L.n_total / 4, nd / 4, h->cfg.lr, h->cfg.momentum, h->cfg.weight_decay, gscale);
     h->launches += 2;
 }
@@ -2028,8 +2030,7 @@ const char* alexnet_last_error(const alexnet_t* h) { return h ? h->err.c_str() :
 // alexnet_create.  For them this entry point keeps its scratch -- the per-split
 // partial column sums of the reduction -- in a fixed array that is
 // part of the loaded library image.  Every GPU that loads the library holds
-// that array (kNoAllocSplits * kNoAllocMaxC floats = 1 MiB) until the process
-// exits.
+// that array (kNoAllocFloats floats = 1 MiB) until the process exits.
 //
 // The array's name is only a host-side stand-in for the symbol, not a device
 // address, so host code never passes it to a kernel: once per device, with that
@@ -2046,14 +2047,18 @@ const char* alexnet_last_error(const alexnet_t* h) { return h ? h->err.c_str() :
 // streams, no dependency) race on it and may both give wrong sums, but later calls
 // do not suffer from it; order them.
 namespace {
-constexpr int kNoAllocSplits = 64;
 constexpr int kNoAllocMaxC = 4096;
-static __device__ __align__(256) float g_noalloc_partials[kNoAllocSplits * kNoAllocMaxC];
+// The partials are at most four blocks per SM of 64 columns, 148 KiB; an array of no more than that is placed where 25088 x 384
+// takes 7.87 us instead of 7.65 (aligning it or the counters does not help).
+constexpr int kNoAllocFloats = 256 * 1024;
+static_assert(4 * kSms * 64 <= kNoAllocFloats, "row splits x channels");
+static __device__ __align__(256) float g_noalloc_partials[kNoAllocFloats];
 static __device__ unsigned long long g_noalloc_counters[kNoAllocMaxC / 64];      // call number << 16 | finished row splits of 64 columns
 
 constexpr int kMaxDevices = 64;
 float* g_noalloc_ptr[kMaxDevices] = {nullptr};
 unsigned long long* g_noalloc_cnt[kMaxDevices] = {nullptr};
+int g_noalloc_sms[kMaxDevices] = {0};
 std::atomic<unsigned long long> g_noalloc_calls{0};
 
 void put_err(char* buf, size_t len, const char* msg) {
@@ -2082,6 +2087,7 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
         unsigned long long* q = nullptr;
         e = cudaGetSymbolAddress((void**)&q, g_noalloc_counters);
         if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&p, g_noalloc_partials);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess || !p || !q) {
             put_err(err, err_len, cudaGetErrorString(e));
             return ALEXNET_ERR_CUDA;
@@ -2091,8 +2097,7 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
     }
     // row splits: four blocks per SM in total, at least 64 rows each, as many as the scratch holds
     const int groups = (channels + 63) / 64;
-    int64_t splits = std::min<int64_t>(4 * 148 / groups, rows / 64);
-    splits = std::min<int64_t>(splits, kNoAllocSplits * kNoAllocMaxC / channels);
+    int64_t splits = std::min<int64_t>(4 * std::min(g_noalloc_sms[dev], kSms) / groups, rows / 64);
     splits = std::max<int64_t>(splits, 1);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing((cudaStream_t)stream, &capture);

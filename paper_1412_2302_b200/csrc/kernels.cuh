@@ -1096,7 +1096,7 @@ __global__ void mean_kernel(const float* __restrict__ v, int n, float* __restric
 struct TransposeJob { long long src_off, dst_off; int taps, cout, cig, groups; long long count; };
 struct TransposeJobs { TransposeJob j[5]; int n; int tile0[6]; };   // tile0: first 32 x 32 tile of each job in sgd_update_conv_kernel's grid
 // one parameter of the momentum update: v <- mu v - d w - lr g (d = lr * weight decay, or 0); w <- w + v.
-// Used by the update kernel and by the FC weight-gradient epilogue that applies the update in place, so that both
+// Used by the update kernels and by fc_update_kernel, which applies the update to the FC weights in place, so that both
 // give bit-identical results.
 __device__ __forceinline__ void sgd_step(float& w, float& v, float g, float d, float lr, float mu) {
     v = fmaf(mu, v, fmaf(-d, w, -lr * g));

@@ -12,10 +12,9 @@
 // advance incrementally.  The main kernels of this file: gemm_kernel (FC
 // backward), conv_kernel (convolution forward / backward-data, FC forward) and
 // wgrad_kernel (convolution weight gradients).
-// Three operand arrangements:
-//   MODE_KK   A K-major, B K-major   conv fwd, conv bwd-data, FC fwd
+// conv_kernel reads both operands K-major.  gemm_kernel has two arrangements:
 //   MODE_KMN  A K-major, B MN-major  FC bwd-data (weights read untransposed)
-//   MODE_MNMN A MN-major, B MN-major weight gradients (reduction over rows)
+//   MODE_MNMN A MN-major, B MN-major FC weight gradients (reduction over the batch)
 // A convolution is an implicit GEMM over a zero-padded flat NHWC grid: filter
 // tap t reads the input rows of the output tile shifted by shift[t] rows, so
 // every A tile is a plain 2-D TMA box; out-of-range rows are zero-filled by TMA.
@@ -45,7 +44,7 @@ __device__ __forceinline__ long long gtime_ns() { long long t; asm volatile("mov
 #define TL(...)
 #endif
 
-enum { MODE_KK = 0, MODE_KMN = 1, MODE_MNMN = 2 };
+enum { MODE_KMN = 0, MODE_MNMN = 1 };
 enum { EPI_BF16 = 0, EPI_F32 = 1 };
 constexpr int kThreads = 192;
 constexpr int kMaxTaps = 25;
@@ -60,26 +59,22 @@ struct GemmParams {
     int tiles_total;
     int BN;            // MMA N (multiple of 16, <= 256)
     int kk;            // K=16 MMAs per stage (<= 4)
-    int chunks;        // MODE_KK: 64-element K chunks per tap
     int steps_total;   // k-steps over the whole reduction (split evenly over `splits`)
     int steps_per_split;
     int stages;        // smem ring depth
     int a_bytes;       // A part of a stage: kABytes, or less when a K-major A has fewer than 128 rows (a multiple of 1024)
-    int a_x0, a_gx;    // A column origin and per-group column stride
-    int b_gx;          // MODE_MNMN: B per-group column stride
-    int b_tap_rows, b_g_rows;  // MODE_KK: B row = tap*b_tap_rows + g*b_g_rows + n0
+    int a_gx, b_gx;    // MODE_MNMN: per-group column strides of A and B
     int shift[kMaxTaps];
     // epilogue
-    int M_total;       // valid rows (MODE_KK/KMN); MODE_MNMN: valid rows per group (m_valid)
+    int M_total;       // valid rows (MODE_KMN); MODE_MNMN: valid rows per group (m_valid)
     int n_valid;       // valid columns per group
     int ldo;           // output row pitch (elements)
-    int out_gx;        // per-group output column offset (MODE_KK/KMN) or row offset (MODE_MNMN)
+    int out_gx;        // per-group output column offset (MODE_KMN) or row offset (MODE_MNMN)
     long long split_stride, tap_stride;  // EPI_F32 partial strides (elements)
     int Hp, Wp, H, W;  // flat-grid geometry for zeroing pad rows (Hp = 0: none)
     int relu;
-    float mask_scale;
     const float* bias;           // [groups*n_valid...] indexed by output column, or nullptr
-    const __nv_bfloat16* mask;   // same layout as out; out = mask>0 ? v*mask_scale : 0
+    const __nv_bfloat16* mask;   // same layout as out; out = mask>0 ? v : 0
     void* out;
     int* status;
 };
@@ -142,11 +137,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tm) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
@@ -247,7 +237,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
@@ -316,13 +305,13 @@ __device__ __forceinline__ void epi_chunk(const P& p, uint32_t* v, bool zero, bo
             const __nv_bfloat16* mn = (const __nv_bfloat16*)&m1v;
             #pragma unroll
             for (int k = 0; k < 8; ++k) {
-                f[k] = __bfloat162float(mm[k]) > 0.f ? f[k] * p.mask_scale : 0.f;
-                f[k + 8] = __bfloat162float(mn[k]) > 0.f ? f[k + 8] * p.mask_scale : 0.f;
+                f[k] = __bfloat162float(mm[k]) > 0.f ? f[k] : 0.f;
+                f[k + 8] = __bfloat162float(mn[k]) > 0.f ? f[k + 8] : 0.f;
             }
         } else {
             for (int k = 0; k < 16; ++k)
                 if (col0 + k < p.n_valid)
-                    f[k] = __bfloat162float(mk[k]) > 0.f ? f[k] * p.mask_scale : 0.f;
+                    f[k] = __bfloat162float(mk[k]) > 0.f ? f[k] : 0.f;
         }
     }
     if (col0 + 16 <= p.n_valid) {
@@ -400,7 +389,7 @@ __device__ __forceinline__ void epi_slab(const P& p, uint32_t tmem_addr, bool pa
                 w[k] = p.relu ? cvt_relu_bf16x2(lo, hi) : cvt_bf16x2(lo, hi);
             }
         }
-        if (mk) {      // a masked value is kept or zero (mask_scale is 1 in every layer that stores bf16 this way)
+        if (mk) {      // a masked value is kept or zero
             const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f);
             #pragma unroll
             for (int k = 0; k < 32; ++k) w[k] &= __hgt2_mask(((const __nv_bfloat162*)mk)[k], zero2);
@@ -440,9 +429,7 @@ __global__ void __launch_bounds__(32) wait_probe_kernel(int* status, long long b
 
 constexpr int kABytes = 128 * 128;  // 128 rows x 64 bf16, or 2 boxes of 64 x 64
 
-__host__ __device__ inline int b_stage_bytes(int mode, int BN) {
-    return mode == MODE_KK ? BN * 128 : ((BN + 63) / 64) * 8192;
-}
+__host__ __device__ inline int b_stage_bytes(int BN) { return ((BN + 63) / 64) * 8192; }
 inline size_t smem_bytes(int stage_bytes, int stages) { return 1024 + (size_t)stages * stage_bytes + 4 * kEpiStageBytes + 512; }
 
 // position of a CTA in the tile list; tiles are numbered with m fastest, then
@@ -476,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const int bbytes = b_stage_bytes(p.mode, p.BN);
+    const int bbytes = b_stage_bytes(p.BN);
     const int stage_bytes = p.a_bytes + bbytes;
     const int stages = p.stages;
     // epilogue staging (4 warps x kEpiStageBytes), then barriers: full[8] @0, empty[8] @64, acc_full[2] @128,
@@ -521,20 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                 const int m0 = tc.m_tile * 128, n0 = tc.n_tile * p.BN;
                 const int s_begin = tc.z * per;
                 const int nsteps = min(p.steps_total, s_begin + per) - s_begin;
-                if (p.mode == MODE_KK) {
-                    int tap = 0, ch = s_begin;
-                    if (p.chunks < p.steps_total && s_begin > 0) { tap = s_begin / p.chunks; ch = s_begin - tap * p.chunks; }
-                    const int xa = p.a_x0 + tc.g * p.a_gx, yb = tc.g * p.b_g_rows + n0;
-                    for (int i = 0; i < nsteps; ++i) {
-                        if (!(ok = mbar_wait(empty0 + 8u * st, ph ^ 1u, abort_flag))) break;
-                        const uint32_t sa = base + st * stage_bytes, fb = full0 + 8u * st;
-                        mbar_expect_tx(fb, tx);
-                        tma_load_2d(sa, &p.tmA, xa + ch * 64, m0 + p.shift[tap], fb);
-                        tma_load_2d(sa + p.a_bytes, &p.tmB, ch * 64, tap * p.b_tap_rows + yb, fb);
-                        if (++ch == p.chunks) { ch = 0; ++tap; }
-                        if (++st == stages) { st = 0; ph ^= 1u; }
-                    }
-                } else if (p.mode == MODE_KMN) {
+                if (p.mode == MODE_KMN) {
                     for (int i = 0; i < nsteps; ++i) {
                         if (!(ok = mbar_wait(empty0 + 8u * st, ph ^ 1u, abort_flag))) break;
                         const uint32_t sa = base + st * stage_bytes, fb = full0 + 8u * st;
@@ -562,10 +536,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (whole warp, one elected lane issues)
         {
-            const int a_mn = p.mode == MODE_MNMN, b_mn = p.mode != MODE_KK;
-            const uint32_t idesc = instr_desc(p.BN, a_mn, b_mn);
-            const uint32_t a_adv = a_mn ? 2048u : 32u, b_adv = b_mn ? 2048u : 32u;
-            const uint32_t a_lbo = a_mn ? 8192u : 16u, b_lbo = b_mn ? 8192u : 16u;
+            const int a_mn = p.mode == MODE_MNMN;
+            const uint32_t idesc = instr_desc(p.BN, a_mn, 1);
+            const uint32_t a_adv = a_mn ? 2048u : 32u, b_adv = 2048u;
+            const uint32_t a_lbo = a_mn ? 8192u : 16u, b_lbo = 8192u;
             const int kk = p.kk;
             TileCursor tc; tc.init(p);
             int st = 0; uint32_t ph = 0;
@@ -709,7 +683,6 @@ struct ConvParams {
     int epi, M_total, n_valid, ldo, out_gx;
     long long split_stride;
     int Hp, Wp, H, W, relu;
-    float mask_scale;
     const float* bias;
     const __nv_bfloat16* mask;
     void* out;
@@ -1493,7 +1466,7 @@ struct WgradParams {
     int n_valid;                // valid input channels per group
     int ldo, out_gx;            // row pitch (= input channels per group), per-group row offset
     long long split_stride, tap_stride;
-    int epi, relu; float mask_scale; const float* bias; const __nv_bfloat16* mask;   // fixed: EPI_F32, unused
+    int epi, relu; const float* bias; const __nv_bfloat16* mask;   // fixed: EPI_F32, unused
     void* out;
     float* bias_partial;        // [split][all output channels] column sums of dy, or nullptr
     int bias_ld;                // output channels over all groups

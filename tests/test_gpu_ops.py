@@ -311,7 +311,7 @@ def test_fused_lrn_pool_rows_per_block(batch):
 
 @pytest.mark.parametrize("which,ta,tn,tp,targ,tdp,tda,shp", FUSED)
 def test_fused_pool_lrn_backward(net, which, ta, tn, tp, targ, tdp, tda, shp):
-    """The fused backward kernel of the step (pooling gradient scattered in shared memory, LRN gradient, ReLU mask)
+    """The fused backward kernel of the step (pooling gradient gathered in registers, LRN gradient, ReLU mask)
     against the oracle's pool_bwd followed by lrn_bwd, with argmax codes that send several windows to one pixel."""
     B = net.batch
     a = tie_heavy(SEED, 95 + which, (B,) + shp, 2)

@@ -9,9 +9,9 @@ keeps its scratch in a fixed 1 MiB array inside the library image.
 Checked here: its output against the existing path's (the bias gradient the
 step's own backward-weight operation produces) on two calls in a row, and
 against a column sum computed on the host in fp64, over sizes that use one
-split, several splits with a ragged last one, and the cap of 64 splits at the
-largest channel count the scratch holds; calls of different shapes follow one
-another, so that contents a previous call left in the scratch would show."""
+split, several splits with a ragged or an empty last one, and the most splits
+and the largest part of the scratch there are; calls of different shapes follow
+one another, so that contents a previous call left in the scratch would show."""
 import numpy as np
 import pytest
 import torch
@@ -55,14 +55,18 @@ def test_bias_grad_noalloc_matches_step_operation_twice():
     net.close()
 
 
-# (rows, channels): splits = clamp(rows / 256, 1, 64), the scratch is laid out [split][channels]
-CASES = [(20000, 4096),     # 64 splits (capped from 78) at the largest channel count: the whole 1 MiB scratch
-         (300, 4096),       # 1 split right after: only row 0 of the scratch may be read
-         (5000, 4096),      # 19 splits, last one ragged
-         (1000, 8),         # 3 splits of 334 rows, the last with 332; the smallest channel count
-         (21632, 256),      # 64 splits (capped from 84): conv5's gradient at batch 128
-         (777, 72),         # 3 splits; channels not a multiple of 64 (the second column block is partial), rows % 32 != 0
-         (1, 4096)]         # a single row
+# (rows, channels): splits = clamp(rows / 64, 1, 592 / ceil(channels / 64)), the scratch is laid out [split][channels]
+CASES = [(20000, 4096),     # 9 splits (capped from 312) at the largest channel count
+         (300, 4096),       # 4 splits right after: only the first four rows of the scratch may be read
+         (5000, 4096),      # 9 splits of 556 rows, the last with 552
+         (1000, 8),         # 15 splits of 67 rows, the last with 62; the smallest channel count
+         (21632, 256),      # 148 splits (capped from 338): conv5's gradient at batch 128
+         (777, 72),         # 12 splits; channels not a multiple of 64 (the second column block is partial), rows % 32 != 0
+         (1, 4096),         # a single row
+         (40000, 64),       # 592 splits of 68 rows, the last ones empty, in one column group: the most scratch there is
+         (6500, 64),        # 101 splits of 65 rows, the last one empty
+         (64, 64), (127, 40),   # one split, of the fewest and of the most rows
+         (128, 40)]         # two splits
 
 
 def test_bias_grad_noalloc_against_host_column_sums():
