@@ -322,8 +322,9 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 }
 // Both kernels work on PIXEL PAIRS: a thread owns eight channels of the pixels (2i, 2i+1) of a row and keeps every fp32 value of
 // the pair in one 64-bit register, so that sums and products are the packed instructions of sm_100 (add / mul / fma.rn.f32x2):
-// the kernels are bound by instruction issue and by the special-function unit (two instructions per element, 16 lanes per
-// SM and cycle), not by HBM, and packing halves the arithmetic instructions.  Window sums take pair sums shared by
+// the forward kernel is bound by the special-function unit (two instructions per element, 16 lanes per SM and cycle: 63% busy),
+// the backward one by instruction issue (64% of the slots; special functions 37%), neither by HBM (26% and 32%), and packing
+// halves the arithmetic instructions.  Window sums take pair sums shared by
 // neighbouring channels.  Measured at batch 128 (back to back), this form against one thread per pixel vector with the
 // pooling gradient scattered through shared memory: forward 40.4 -> 36.6 us (LRN1) and 27.6 -> 24.8 (LRN2), backward 79.1 ->
 // 53.5 and 48.9 -> 34; at batch 512 forward 141 -> 128 and 97 -> 83.  Same arithmetic in the same order as the single-operation kernels.
