@@ -891,7 +891,7 @@ void op_conv_wg(alexnet* h, int r, int l, int slot, cudaStream_t st, bool reduce
     launch_gemm(h, P, st);     // weight-gradient partials per row split, and the bias-gradient partials
     if (!reduce) return;
     const long long total = (long long)c.taps * c.cout * c.cig;
-    launch_k(kn::wgrad_reduce_kernel, nblk(total / 4, 256), 256, 0, st, h->ws + h->ws_conv_off[l], P.w.splits, P.w.split_stride, total,
+    launch_k(kn::wgrad_reduce_kernel, nblk(total, 256), 256, 0, st, h->ws + h->ws_conv_off[l], P.w.splits, P.w.split_stride, total,
              R.g + c.w_off, l == 0, h->bias_partial + (size_t)l * kBiasPartial, c.cout, R.g + c.b_off);
     h->launches++;
 }

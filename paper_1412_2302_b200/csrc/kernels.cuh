@@ -770,26 +770,30 @@ __global__ void __launch_bounds__(256) fc_reduce_bwd_kernel(const float* __restr
         db[blockIdx.x * 32 + threadIdx.x] = s;
     }
 }
-// g[i] = sum_z ws[z][i]; conv1: entries of the 12x12 zero-padded filter outside 11x11 stay zero.  One thread = four consecutive entries.
-// The first `cout / 4` threads also add the per-split bias-gradient partials: db[c] = sum_z bias_partial[z][c].
+// g[i] = sum_z ws[z][i]; conv1: entries of the 12x12 zero-padded filter outside 11x11 stay zero.
+// The first `cout` threads also add the per-split bias-gradient partials: db[c] = sum_z bias_partial[z][c].
+// One entry per thread: with four entries per thread and 8 or 16 vectors in flight conv1, whose 41472 entries have up to 49 splits,
+// has a quarter of the threads and takes 10 us more (weight gradient and reduction 51.5 -> 61.8 us at batch 128, 14.6 -> 22.8 at 8;
+// conv2 59.1 -> 60.7; conv3 and conv4, hidden beside the data gradients, 41 -> 40).
 __global__ void wgrad_reduce_kernel(const float* __restrict__ ws, int splits, long long split_stride,
                                     long long total, float* __restrict__ g, int conv1_pad_mask,
                                     const float* __restrict__ bias_partial, int cout, float* __restrict__ db) {
     pdl_sync();
-    const long long t = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
-    if (t >= total) return;                      // total, the split stride and cout are multiples of 4
-    float4 v = sum_splits<8>(ws + t, split_stride, splits);
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= total) return;
+    float v = 0.f;
+    for (int z = 0; z < splits; ++z) v += ws[z * split_stride + t];
     if (conv1_pad_mask) {
-        float* gp = &v.x;
-        #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int ch = (int)((t + k) % 48), tap = (int)((t + k) / (48 * 96));
-            const int ky = (tap / 3) * 4 + (ch / 3) / 4, kx = (tap % 3) * 4 + (ch / 3) % 4;
-            if (ky > 10 || kx > 10) gp[k] = 0.f;
-        }
+        const int ch = (int)(t % 48), tap = (int)(t / (48 * 96));
+        const int ky = (tap / 3) * 4 + (ch / 3) / 4, kx = (tap % 3) * 4 + (ch / 3) % 4;
+        if (ky > 10 || kx > 10) v = 0.f;
     }
-    *(float4*)(g + t) = v;
-    if (bias_partial && t < cout) *(float4*)(db + t) = sum_splits<8>(bias_partial + t, cout, splits);
+    g[t] = v;
+    if (bias_partial && t < cout) {
+        float b = 0.f;
+        for (int z = 0; z < splits; ++z) b += bias_partial[(size_t)z * cout + t];
+        db[t] = b;
+    }
 }
 
 // db[c] = sum over rows of dy[row][c] (bf16 in, fp32 out), two stages: grid (ceil(C/64), row_splits)
