@@ -153,7 +153,7 @@ struct Plan { tc::GemmParams p; tc::ConvParams c; tc::WgradParams w; tc::FcUpdPa
 // CTAs (one per SM) of the FC weight-gradient + update kernels; the SMs left over are those of the data gradients of conv5..conv3
 // that run beside them: fc_update_kernel reaches most of the HBM rate on this many SMs (see there), and a chain
 // kernel whose grid fits beside it neither waits for it nor leaves CTAs of a second wave behind.
-// Measured at batch 128 only (fc6 161 us on 64 SMs, 134 on 80, the step no faster); at smaller batches, where the chain beside the
+// Measured at batch 128 only (fc6 161 us on 64 SMs, 134 on 80); at smaller batches, where the chain beside the
 // updates is short, more SMs may pay.
 constexpr int kFcUpdCtas = 64;
 
