@@ -148,7 +148,7 @@ Layout make_layout() {
 const long long kCanonCount = 60965224;
 
 // ------------------------------------------------------------------- handle
-constexpr size_t kBiasPartial = 65536;    // floats per conv layer: row splits (<= 148) x output channels (<= 384)
+constexpr size_t kBiasPartial = 65536;    // floats per conv layer: (row splits x sharers of a dy tile <= 148) x output channels (<= 384)
 struct Plan { tc::GemmParams p; tc::ConvParams c; tc::WgradParams w; tc::FcUpdParams u; bool conv, wgrad, upd; int upd_K; int grid; size_t smem; bool valid; };
 // CTAs (one per SM) of the FC weight-gradient + update kernels; the SMs left over are those of the data gradients of conv5..conv3
 // that run beside them: fc_update_kernel reaches most of the HBM rate on this many SMs (see there), and a chain
@@ -156,6 +156,14 @@ struct Plan { tc::GemmParams p; tc::ConvParams c; tc::WgradParams w; tc::FcUpdPa
 // Measured at batch 128 only (fc6 161 us on 64 SMs, 134 on 80); at smaller batches, where the chain beside the
 // updates is short, more SMs may pay.
 constexpr int kFcUpdCtas = 64;
+// Conv weight gradients of at most this many 128-row steps run with one CTA per tile, which takes all row splits in turn
+// (WgradParams::solo).  Below about batch 64 these kernels are not the longest branch, and a wave of CTAs of a few steps each costs
+// more than it saves: each takes a whole SM from the data gradients and the FC updates beside it for its set-up and epilogue,
+// and the update adds its partials (64 MB of them at batch 8).  Steps with three handles taking turns, no solo / 30 / 64 / 110 / 220
+// steps: batch 4 390 / 353 / 353 / 351 / 351 us, 8 414 / 386 / 381 / 381 / 375, 16 441 / 416 / 417 / 416 / 415, 32 512 / 512 / 490 / 489 /
+// 487, 64 687 / 693 / 692 / 677 / 677; one handle alone 457 / 476 / 477 / 472 / 473, 466 / 467 / 467 / 468 / 521, 495 / 494 / 495 / 496 /
+// 496, 552 / 553 / 545 / 545 / 564, 720 / 719 / 719 / 715 / 715: at 220 steps conv1, the last kernel of the pass, takes too long.
+constexpr int kWgSoloSteps = 110;
 
 struct Tensor {  // description of one exportable device tensor
     void* ptr; int kind; int C, Hp, Wp, H, W; long long N;
@@ -600,17 +608,23 @@ int plan_conv_wg(alexnet* h, Plan& P, int l, const ConvL& c, const bf16* dy, con
     p.splits = conv_wg_splits(c, h->B, std::min(h->sm_count, kSms));   // never more than the workspace was sized for
     p.steps_per_split = (p.steps_total + p.splits - 1) / p.splits;
     p.splits = (p.steps_total + p.steps_per_split - 1) / p.steps_per_split;
-    p.tiles_total = p.m_tiles * p.n_tiles * p.groups * p.kh * p.splits;
-    if (c.k <= 4) { p.NI = 1; p.acc_kx0[0] = 0; p.acc_taps[0] = c.k; }
-    else { p.NI = 2; p.acc_kx0[0] = 0; p.acc_taps[0] = 3; p.acc_kx0[1] = 3; p.acc_taps[1] = c.k - 3; }
+    p.solo = p.splits > 1 && p.steps_total <= kWgSoloSteps;
+    p.parts = p.solo ? 1 : p.splits;
+    p.NI = c.k <= 4 ? 1 : 2;
+    p.acc_kx0[0] = 0; p.acc_taps[0] = std::min(c.k, 3); p.acc_kx0[1] = 3; p.acc_taps[1] = c.k - 3;
+    p.kw_parts = p.solo && 2 * 64 * c.k > 512 ? 2 : 1;
+    if (p.kw_parts == 2) p.NI = 1;
+    p.tiles_total = p.m_tiles * p.n_tiles * p.groups * p.kh * p.kw_parts * p.parts;
     p.stages = std::min(8, (int)((227 * 1024 - 2048) / (tc::kWgABytes + tc::kWgBBytes)));
     p.a_gx = c.cog; p.b_gx = c.cig;
     for (int ky = 0; ky < c.k; ++ky) p.halo_shift[ky] = (ky - c.pad) * c.gin.Wp - c.pad;
     p.M_total = c.cog; p.n_valid = c.cig; p.ldo = c.cig; p.out_gx = c.cog;
     p.tap_stride = (long long)c.cout * c.cig; p.split_stride = (long long)c.taps * c.cout * c.cig;
-    p.epi = tc::EPI_F32;
     p.out = h->ws + h->ws_conv_off[l]; p.status = h->status;
     p.bias_partial = h->bias_partial + (size_t)l * kBiasPartial; p.bias_ld = c.cout;
+    const int sharers = p.kh * p.n_tiles * p.kw_parts;
+    p.bias_sharers = p.steps_per_split * (p.solo ? p.splits : 1) >= 2 * sharers ? sharers : 1;      // (few steps: not worth more partials)
+    p.bias_parts = p.parts * p.bias_sharers;
     int rc;
     if ((rc = make_tm(h, &p.tmA, dy, c.cout, M, (uint64_t)c.cout * 2, tc::kWgRows))) return rc;
     if ((rc = make_tm(h, &p.tmB, xin, c.cin, M, (uint64_t)c.cin * 2, tc::kWgRows + 8))) return rc;
@@ -893,8 +907,9 @@ void op_conv_wg(alexnet* h, int r, int l, int slot, cudaStream_t st, bool reduce
     launch_gemm(h, P, st);     // weight-gradient partials per row split, and the bias-gradient partials
     if (!reduce) return;
     const long long total = (long long)c.taps * c.cout * c.cig;
-    launch_k(kn::wgrad_reduce_kernel, nblk(total, 256), 256, 0, st, h->ws + h->ws_conv_off[l], P.w.splits, P.w.split_stride, total,
-             R.g + c.w_off, l == 0, h->bias_partial + (size_t)l * kBiasPartial, c.cout, R.g + c.b_off);
+    launch_k(kn::wgrad_reduce_kernel, nblk(total, 256) + nblk(c.cout / 4, 32), 256, 0, st, h->ws + h->ws_conv_off[l], P.w.parts, P.w.split_stride, total,
+             R.g + c.w_off, l == 0, h->bias_partial + (size_t)l * kBiasPartial, P.w.bias_parts, c.cout, R.g + c.b_off,
+             nblk(total, 256));
     h->launches++;
 }
 void op_fc_fwd(alexnet* h, int r, int l, uint64_t step, cudaStream_t st, bool eval = false, bool gemm_only = false,
@@ -1114,20 +1129,21 @@ void op_update(alexnet* h, int r, cudaStream_t st, bool full = false, float gsca
             src.on = 1;
             for (int l = 0; l < 5; ++l) {
                 const tc::WgradParams& wp = R.conv_wg[l][reduce_slot].w;
-                src.splits[l] = wp.splits; src.cout[l] = L.conv[l].cout;
+                src.splits[l] = wp.parts; src.bparts[l] = wp.bias_parts; src.cout[l] = L.conv[l].cout;
                 src.ws[l] = h->ws + h->ws_conv_off[l]; src.stride[l] = wp.split_stride;
                 src.bpart[l] = h->bias_partial + (size_t)l * kBiasPartial; src.b_off4[l] = L.conv[l].b_off / 4;
             }
         }
-        launch_k(kn::sgd_update_conv_kernel, L.tjobs.tile0[5] + nblk(e4 - b4, 256), 256, 0, st, R.w, R.v, R.g, R.shadow, d,
-                 h->cfg.lr, h->cfg.momentum, R.wt, L.tjobs, gscale, b4, e4, 0.f, src);
+        const int bias_blocks = nblk(e4 - b4, 32);
+        launch_k(kn::sgd_update_conv_kernel, bias_blocks + L.tjobs.tile0[5], 256, 0, st, R.w, R.v, R.g, R.shadow, d,
+                 h->cfg.lr, h->cfg.momentum, R.wt, L.tjobs, gscale, bias_blocks, b4, e4, 0.f, src);
         h->launches++;
         return;
     }
     kn::ConvSplitSrc none;
     memset(&none, 0, sizeof(none));
     launch_k(kn::sgd_update_conv_kernel, L.tjobs.tile0[5], 256, 0, st, R.w, R.v, R.g, R.shadow, d,
-             h->cfg.lr, h->cfg.momentum, R.wt, L.tjobs, gscale, 0LL, 0LL, 0.f, none);
+             h->cfg.lr, h->cfg.momentum, R.wt, L.tjobs, gscale, 0, 0LL, 0LL, 0.f, none);
     launch_k(kn::sgd_update_kernel, fused ? h->sm_count : 1184, 256, 0, st, R.w, R.v, R.g, R.shadow, (fused ? L.n_weights : L.fc[0].w_off) / 4,
              L.n_total / 4, nd / 4, h->cfg.lr, h->cfg.momentum, h->cfg.weight_decay, gscale);
     h->launches += 2;

@@ -63,6 +63,19 @@ __device__ __forceinline__ float4 sum_splits(const float* __restrict__ src, long
     return s;
 }
 
+// Four consecutive channels of a conv layer's bias gradient from its partials [parts][cout], by eight consecutive lanes of a
+// warp: lane k (0..7) adds the partials k, k + 8, ..., then the lanes add up in pairs, so the order is fixed; every lane of
+// the eight has the result.  There are up to 148 partials (conv1): one thread per channel group with 16 loads in flight took 8 us.
+__device__ __forceinline__ float4 bias_sum8(const float* __restrict__ bp, int cout, int parts, int k) {
+    float4 s = k < parts ? sum_splits<10>(bp + (long long)k * cout, 8LL * cout, (parts - k + 7) / 8) : make_float4(0.f, 0.f, 0.f, 0.f);
+    #pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        s.x += __shfl_xor_sync(~0u, s.x, o); s.y += __shfl_xor_sync(~0u, s.y, o);
+        s.z += __shfl_xor_sync(~0u, s.z, o); s.w += __shfl_xor_sync(~0u, s.w, o);
+    }
+    return s;
+}
+
 // ------------------------------------------------------------- preprocessing
 // Per image: crop offset (ox, oy) in [0,29]^2 and flip bit from the hash
 // (stream 1, idx = image).  out = u8[sy][sx][c] - mean[sy][sx][c] with
@@ -771,14 +784,22 @@ __global__ void __launch_bounds__(256) fc_reduce_bwd_kernel(const float* __restr
     }
 }
 // g[i] = sum_z ws[z][i]; conv1: entries of the 12x12 zero-padded filter outside 11x11 stay zero.
-// The first `cout` threads also add the per-split bias-gradient partials: db[c] = sum_z bias_partial[z][c].
+// The blocks from bias_block0 on add the bias-gradient partials, 32 groups of four channels each (cout is a multiple of 4).
 // One entry per thread: with four entries per thread and 8 or 16 vectors in flight conv1, whose 41472 entries have up to 49 splits,
 // has a quarter of the threads and takes 10 us more (weight gradient and reduction 51.5 -> 61.8 us at batch 128, 14.6 -> 22.8 at 8;
 // conv2 59.1 -> 60.7; conv3 and conv4, hidden beside the data gradients, 41 -> 40).
 __global__ void wgrad_reduce_kernel(const float* __restrict__ ws, int splits, long long split_stride,
                                     long long total, float* __restrict__ g, int conv1_pad_mask,
-                                    const float* __restrict__ bias_partial, int cout, float* __restrict__ db) {
+                                    const float* __restrict__ bias_partial, int bias_parts, int cout, float* __restrict__ db,
+                                    int bias_block0) {
     pdl_sync();
+    if ((int)blockIdx.x >= bias_block0) {
+        const int c4 = ((int)blockIdx.x - bias_block0) * 32 + (threadIdx.x >> 3), k = threadIdx.x & 7;
+        const bool in = 4 * c4 < cout;
+        const float4 b = bias_sum8(bias_partial + (in ? 4 * c4 : 0), cout, bias_parts, k);
+        if (in && k == 0) *(float4*)(db + 4 * c4) = b;
+        return;
+    }
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     float v = 0.f;
@@ -789,11 +810,6 @@ __global__ void wgrad_reduce_kernel(const float* __restrict__ ws, int splits, lo
         if (ky > 10 || kx > 10) v = 0.f;
     }
     g[t] = v;
-    if (bias_partial && t < cout) {
-        float b = 0.f;
-        for (int z = 0; z < splits; ++z) b += bias_partial[(size_t)z * cout + t];
-        db[t] = b;
-    }
 }
 
 // db[c] = sum over rows of dy[row][c] (bf16 in, fp32 out), two stages: grid (ceil(C/64), row_splits)
@@ -1140,37 +1156,40 @@ __global__ void sgd_update_kernel(float* __restrict__ w, float* __restrict__ v, 
 // order and with conv1's pad entries zeroed - wgrad_reduce_kernel's arithmetic - and stores the sums to g as that kernel does.
 struct ConvSplitSrc {
     int on;
-    int splits[5], cout[5];
+    int splits[5], bparts[5], cout[5];
     const float* ws[5]; long long stride[5];       // layer l: ws[l][z * stride[l] + index within the layer's filters]
-    const float* bpart[5]; long long b_off4[5];    // bias partials [z][cout]; first 16-byte vector of the layer's biases
+    const float* bpart[5]; long long b_off4[5];    // bias partials [bparts][cout]; first 16-byte vector of the layer's biases
 };
 __global__ void __launch_bounds__(256) sgd_update_conv_kernel(float* __restrict__ w, float* __restrict__ v, float* __restrict__ g,
                                                               __nv_bfloat16* __restrict__ shadow, float d, float lr, float mu,
                                                               __nv_bfloat16* __restrict__ wt, const TransposeJobs jobs, float gscale,
-                                                              long long tail_begin4, long long tail_end4, float tail_d,
-                                                              const ConvSplitSrc src) {
+                                                              int bias_blocks, long long tail_begin4, long long tail_end4,
+                                                              float tail_d, const ConvSplitSrc src) {
     pdl_sync();
     __shared__ __nv_bfloat16 tile[32][36];       // [input channel][output channel], padded
-    if ((int)blockIdx.x >= jobs.tile0[jobs.n]) {
-        // blocks past the filter tiles: the plain update of the 16-byte vectors [tail_begin4, tail_end4) (the biases, when the
-        // FC weights have been updated by their weight-gradient kernels), sgd_update_kernel's arithmetic, one launch less
-        const long long i = tail_begin4 + (long long)((int)blockIdx.x - jobs.tile0[jobs.n]) * 256 + threadIdx.x;
-        if (i < tail_end4) {
+    const int tile_block = (int)blockIdx.x - bias_blocks;
+    if (tile_block < 0) {
+        // blocks before the filter tiles (they have the longest sums): the plain update of the 16-byte vectors
+        // [tail_begin4, tail_end4) (the biases, when the FC weights have been updated by their weight-gradient kernels),
+        // sgd_update_kernel's arithmetic, one launch less.  Eight lanes per vector, for the conv layers' sums.
+        const long long i = tail_begin4 + (long long)blockIdx.x * 32 + (threadIdx.x >> 3);
+        const int k = threadIdx.x & 7;
+        int lb = -1;
+        if (src.on) {
+            #pragma unroll
+            for (int l = 0; l < 5; ++l)
+                if (i >= src.b_off4[l] && i < src.b_off4[l] + src.cout[l] / 4) lb = l;
+        }
+        // a conv layer's bias gradient from its partials (the lanes of a warp may belong to different layers: all of them add)
+        float4 gv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (src.on) {
+            const float* bp = lb >= 0 ? src.bpart[lb] + 4 * (i - src.b_off4[lb]) : src.bpart[0];
+            gv = bias_sum8(bp, lb >= 0 ? src.cout[lb] : 0, lb >= 0 ? src.bparts[lb] : 0, k);
+        }
+        if (i < tail_end4 && k == 0) {
             float4 wv = ((float4*)w)[i], vv = ((float4*)v)[i];
-            float4 gv;
-            int lb = -1;
-            if (src.on) {
-                #pragma unroll
-                for (int l = 0; l < 5; ++l)
-                    if (i >= src.b_off4[l] && i < src.b_off4[l] + src.cout[l] / 4) lb = l;
-            }
-            if (lb >= 0) {                       // a conv layer's bias gradient from its partials
-                const float* bp = src.bpart[lb] + 4 * (i - src.b_off4[lb]);
-                gv = sum_splits<8>(bp, src.cout[lb], src.splits[lb]);
-                ((float4*)g)[i] = gv;
-            } else {
-                gv = ((const float4*)g)[i];
-            }
+            if (lb >= 0) ((float4*)g)[i] = gv;
+            else gv = ((const float4*)g)[i];
             sgd_step(wv.x, vv.x, gscale * gv.x, tail_d, lr, mu);
             sgd_step(wv.y, vv.y, gscale * gv.y, tail_d, lr, mu);
             sgd_step(wv.z, vv.z, gscale * gv.z, tail_d, lr, mu);
@@ -1183,11 +1202,11 @@ __global__ void __launch_bounds__(256) sgd_update_conv_kernel(float* __restrict_
         return;
     }
     int q = 0;
-    while (q + 1 < jobs.n && (int)blockIdx.x >= jobs.tile0[q + 1]) ++q;
+    while (q + 1 < jobs.n && tile_block >= jobs.tile0[q + 1]) ++q;
     const TransposeJob J = jobs.j[q];
     const int cog = J.cout / J.groups;
     const int ci_blocks = (J.cig + 31) / 32, co_blocks = J.cout / 32;     // cout is a multiple of 32 in every layer
-    int t = (int)blockIdx.x - jobs.tile0[q];
+    int t = tile_block - jobs.tile0[q];
     const int cib = t % ci_blocks; t /= ci_blocks;
     const int cob = t % co_blocks, tap = t / co_blocks;
     const int r = threadIdx.x >> 3, c4 = threadIdx.x & 7;

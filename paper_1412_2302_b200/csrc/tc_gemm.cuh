@@ -128,6 +128,20 @@ __device__ __forceinline__ bool mbar_wait_budget(uint32_t bar, uint32_t parity, 
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     return mbar_wait_budget(bar, parity, abort_flag, kWaitBudgetCycles);
 }
+// For whole warps that wait for a main loop (the epilogues) or have slack (the bias sums): suspended from the start, one result for the
+// warp.  Polling costs power, and at batch 100 and above a step runs at the board's power limit: four to eight warps of every SM
+// polling through the main loops cost 0.5% of a step at batch 128 and 0.3% at 512.
+__device__ __forceinline__ bool mbar_wait_idle(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    const long long t0 = clock64();
+    bool ok = false;
+    while (!ok) {
+        #pragma unroll 1
+        for (int i = 0; i < 256 && !ok; ++i) ok = mbar_try_wait(bar, parity);
+        if (ok || *abort_flag) break;
+        if (clock64() - t0 > kWaitBudgetCycles) { *abort_flag = 1; break; }
+    }
+    return __all_sync(0xffffffffu, ok);
+}
 // the same for a whole warp that must take one decision (all lanes wait; any failure fails all)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                                long long budget = kWaitBudgetCycles) {
@@ -227,6 +241,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31};"
+        :: "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+           "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+           "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // TMA store of one box from shared memory (bulk async-group completion)
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, uint32_t src, int x, int y, int z) {
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
@@ -593,7 +617,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const __grid_constant
                 }
                 row_off = (long long)tc.z * p.split_stride + (long long)row * p.ldo + g * p.out_gx;
             }
-            if (!(ok = mbar_wait(accf0 + 8u * ab, aph, abort_flag))) break;
+            if (!(ok = mbar_wait_idle(accf0 + 8u * ab, aph, abort_flag))) break;
             tc_fence_after();
             const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * p.BN);
             if (p.tma_store) {
@@ -988,7 +1012,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 epi_mask_load(row < p.M_total ? (const uint4*)(p.mask + (long long)row * p.ldo + g * p.out_gx + n0 + (first % nslab) * slab) : nullptr, mk);
             }
             TL(const long long ce0 = clock64();)
-            ok = mbar_wait(accf0 + 8u * ab, aph, abort_flag);
+            ok = mbar_wait_idle(accf0 + 8u * ab, aph, abort_flag);
             TL(if (ew == 0 && lane == 0) tl[8] += clock64() - ce0;)
             if (!ok) break;
             tc_fence_after();
@@ -1306,7 +1330,7 @@ __global__ void __launch_bounds__(kChainThreads, 1) fc_chain_kernel(const __grid
         for (int l = 0; l < p.nlayers && ok; ++l) {
             const FcChainLayer& L = p.L[l];
             CHAIN_UNIT(L)
-            ok = mbar_wait(accf0 + 8u * ab, aph, abort_flag);
+            ok = mbar_wait_idle(accf0 + 8u * ab, aph, abort_flag);
             if (!ok) break;
             TL(if (et == 0 && l < 2) tl[9 + 3 * l] = gtime_ns();)
             tc_fence_after();
@@ -1448,13 +1472,18 @@ __global__ void __launch_bounds__(kChainThreads, 1) fc_chain_kernel(const __grid
 // (128 bytes), which makes N block j read the halo from row j on.  One
 // instruction therefore covers up to four taps (N = 64 * taps <= 256); a
 // five-tap row takes two accumulators with an issuer warp each.
-// Each CTA writes fp32 partial sums [split][tap][co][ci]; a reduction kernel
-// adds the splits in a fixed order.
+// Each CTA writes fp32 partial sums [split][tap][co][ci]; a reduction kernel or the update adds the splits in a fixed order.
+// Short reductions (plan_conv_wg) run with ONE CTA per tile that takes all splits, one after another: the first accumulates in
+// the first columns of the tensor memory, the later ones beside it, and the epilogue warps add each of these to the first in
+// tensor memory: the same sums in the same order, so the same bits, and one partial per tile.
 // Warps: 0 = TMA producer, 1..NI = MMA issuers, NI+1..NI+4 = epilogue.
 struct WgradParams {
     CUtensorMap tmA, tmB;       // dy [M][cout] box {64, kWgRows}; x [M][cin] box {64, kWgRows + 8}
-    int m_tiles, n_tiles, groups, kh, splits;   // tile decomposition (m fastest, then n, group, ky, split)
+    int m_tiles, n_tiles, groups, kh, splits;   // tile decomposition (m fastest, then n, group, ky, part of the filter row, split)
     int tiles_total;
+    int solo;                   // 1: a CTA takes all splits of its tile and leaves one sum
+    int kw_parts;               // 2: the accumulators of a five-tap row go to two CTAs (solo, where twice their columns would not fit)
+    int parts;                  // slots of partial sums: splits, or 1 (solo)
     int kw;                     // taps per filter row
     int NI;                     // accumulators = issuers (1 or 2)
     int acc_kx0[2], acc_taps[2];  // first tap and tap count of each accumulator
@@ -1466,10 +1495,11 @@ struct WgradParams {
     int n_valid;                // valid input channels per group
     int ldo, out_gx;            // row pitch (= input channels per group), per-group row offset
     long long split_stride, tap_stride;
-    int epi, relu; const float* bias; const __nv_bfloat16* mask;   // fixed: EPI_F32, unused
-    void* out;
-    float* bias_partial;        // [split][all output channels] column sums of dy, or nullptr
+    float* out;
+    float* bias_partial;        // [split, or 1 when solo][sharer][all output channels] column sums of dy, or nullptr
     int bias_ld;                // output channels over all groups
+    int bias_sharers;           // of the kh * n_tiles * kw_parts CTAs that load the same dy tiles, how many share its sums
+    int bias_parts;             // partials: splits (1 when solo) x sharers
     int* status;
 };
 constexpr int kWgRows = 128;                           // rows of the flat grid per step: 8 MMAs (K = 16 each) per barrier wait
@@ -1484,37 +1514,47 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
     const uint32_t base = (raw + 1023u) & ~1023u;
     const int stages = p.stages, NI = p.NI;
     constexpr uint32_t stage_bytes = kWgABytes + kWgBBytes;
-    // 4 KB for the bias-gradient reduction, then barriers: full[8] @0, empty[8] @64, acc_full @128, tmem slot @136,
-    // abort flag @144
+    // 4 KB for the bias-gradient reduction, then barriers: full[8] @0, empty[8] @64, acc_full[2] @128, acc_added @144,
+    // tmem slot @160, abort flag @168
     const uint32_t red_base = base + stages * stage_bytes;
     const uint32_t bar_base = red_base + 4096u;
     uint8_t* gen = smem_raw + (bar_base - raw);
-    volatile int* abort_flag = (volatile int*)(gen + 144);
-    volatile uint32_t* tmem_slot = (volatile uint32_t*)(gen + 136);
-    const uint32_t full0 = bar_base, empty0 = bar_base + 64u, accf = bar_base + 128u;
+    volatile int* abort_flag = (volatile int*)(gen + 168);
+    volatile uint32_t* tmem_slot = (volatile uint32_t*)(gen + 160);
+    const uint32_t full0 = bar_base, empty0 = bar_base + 64u, accf0 = bar_base + 128u, acca = bar_base + 144u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int acc_cols = 64 * p.kw;
-    uint32_t ncols = 32;
-    while ((int)ncols < acc_cols) ncols <<= 1;
 
     // this CTA's tile (one per CTA: the grid equals the tile count)
     int r = blockIdx.x;
     const int m_tile = r % p.m_tiles; r /= p.m_tiles;
     const int n_tile = r % p.n_tiles; r /= p.n_tiles;
     const int g = r % p.groups; r /= p.groups;
-    const int ky = r % p.kh;
-    const int z = r / p.kh;
-    const int s_begin = z * p.steps_per_split;
-    const int nsteps = min(p.steps_total, s_begin + p.steps_per_split) - s_begin;
+    const int ky = r % p.kh; r /= p.kh;
+    const int part = r % p.kw_parts, z = r / p.kw_parts;       // solo: z = 0
+    const int per = p.steps_per_split, nz = p.solo ? p.splits : 1;
+    const int s_begin = z * per;
+    const int nsteps = min(p.steps_total, s_begin + nz * per) - s_begin;       // every split has at least one step
+    // the taps of this CTA: a whole filter row, or one accumulator's
+    const int kx_lo = p.kw_parts == 2 ? p.acc_kx0[part] : 0, kx_n = p.kw_parts == 2 ? p.acc_taps[part] : p.kw;
+    const int acc_cols = 64 * kx_n;
+    uint32_t ncols = 32;
+    while ((int)ncols < (nz > 1 ? 2 : 1) * acc_cols) ncols <<= 1;
 
-    // the CTAs of filter row 0 and input block 0 also sum the dy tile over the rows (the bias gradient): their four
-    // epilogue warps read every A stage and release it together with the issuers
-    const bool do_bias = p.bias_partial != nullptr && ky == 0 && n_tile == 0;
+    // The CTAs also sum the dy tiles over the rows (the bias gradient), in their otherwise idle epilogue warps, which release
+    // every stage together with the issuers.  A dy tile is loaded by kh * n_tiles CTAs (the filter rows and input blocks of one
+    // output block and row range); bias_sharers of them share its sums: step i is summed by sharer i % bias_sharers.  A sum
+    // reads 32 KB of shared memory, whose bandwidth bounds this kernel (about 160 KB of operand reads and TMA writes per
+    // step), so a CTA that summed every step took a quarter longer than the others and the launch waited for it.  One CTA
+    // summing everything / shared, kernel and reduction in bursts: conv1 51.6 / 47.1, conv3 41.4 / 36.2, conv4 42.1 / 36.7 us
+    // at batch 128 (conv2 and conv5 alike); conv1..conv5 183, 203, 138, 141, 77 / 158, 193, 105, 108, 68 us at 512.
+    const int bias_me = (part * p.kh + ky) * p.n_tiles + n_tile;
+    const bool do_bias = p.bias_partial != nullptr && bias_me < p.bias_sharers;
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         for (int s = 0; s < stages; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, NI + (do_bias ? 4 : 0)); }
-        mbar_init(accf, NI);
+        mbar_init(accf0, NI); mbar_init(accf0 + 8u, NI);       // even and odd splits
+        mbar_init(acca, 4);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         tma_prefetch_desc(&p.tmA);
         tma_prefetch_desc(&p.tmB);
@@ -1543,15 +1583,17 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
         }
     } else if (warp <= NI) {
         {
-            const int a = warp - 1;
+            const int a = warp - 1 + part;
             const int taps = p.acc_taps[a], kx0 = p.acc_kx0[a];
             const uint32_t idesc = instr_desc(64 * taps, 1, 1);
             const uint64_t adesc0 = smem_desc(0, kWgRows * 128, 1024), bdesc0 = smem_desc(0, 128, 1024);
-            const uint32_t d = tmem + (uint32_t)(kx0 * 64);
             int st = 0; uint32_t ph = 0;
-            bool ok = true;
+            uint32_t d = tmem + (uint32_t)((kx0 - kx_lo) * 64);
+            int in_split = 0, zi = 0;
             for (int i = 0; i < nsteps; ++i) {
-                if (!(ok = mbar_wait_warp(full0 + 8u * st, ph, abort_flag))) break;
+                // (the columns of split 2 on are those of split 1: free once the split before has been added)
+                if (in_split == 0 && zi >= 2 && !mbar_wait_warp(acca, (uint32_t)zi & 1u, abort_flag)) break;
+                if (!(mbar_wait_warp(full0 + 8u * st, ph, abort_flag))) break;
                 tc_fence_after();
                 // (masked: in a cluster launch the address of a CTA's shared memory carries its rank above these bits, which
                 // would reach into the descriptor's leading-dimension field)
@@ -1560,42 +1602,90 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
                 const uint64_t bd = bdesc0 + (uint64_t)((sa + kWgABytes + (uint32_t)kx0 * 128u) >> 4);
                 #pragma unroll
                 for (int j = 0; j < kWgRows / 16; ++j)
-                    umma(d, ad + (uint64_t)(128 * j), bd + (uint64_t)(128 * j), idesc, (i > 0 || j > 0) ? 1u : 0u);
+                    umma(d, ad + (uint64_t)(128 * j), bd + (uint64_t)(128 * j), idesc, (in_split > 0 || j > 0) ? 1u : 0u);
                 umma_commit(empty0 + 8u * st);
                 if (++st == stages) { st = 0; ph ^= 1u; }
+                if (++in_split == per || i == nsteps - 1) {
+                    umma_commit(accf0 + 8u * (zi & 1));
+                    in_split = 0;
+                    if (zi++ == 0) d += (uint32_t)acc_cols;
+                }
             }
-            if (ok) umma_commit(accf);
         }
     } else {
         const int quad = warp & 3;
         const int row = m_tile * 128 + quad * 32 + lane;     // output channel within the group
         const bool row_ok = row < p.M_total;
-        if (do_bias) {
-            // thread te: eight output channels (16-byte chunk cc of the 128-channel tile) of rows rg*16 .. rg*16+15 of a stage
-            const int te = (warp - NI - 1) * 32 + lane, cc = te & 15, rg = te >> 4;
-            float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            int st = 0; uint32_t ph = 0;
-            bool ok = true;
-            for (int i = 0; i < nsteps; ++i) {
-                if (!(ok = mbar_wait(full0 + 8u * st, ph, abort_flag))) break;
-                const uint32_t a0 = base + st * stage_bytes + (uint32_t)(cc >> 3) * (kWgRows * 128u) + (uint32_t)rg * (kWgRows / 8 * 128u);
-                #pragma unroll
-                for (int rr = 0; rr < kWgRows / 8; ++rr) {
-                    uint4 u;
-                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w)
-                                 : "r"(a0 + (uint32_t)rr * 128u + (uint32_t)(((cc & 7) ^ (rr & 7)) << 4)));
-                    const __nv_bfloat162* hh = (const __nv_bfloat162*)&u;
+        // thread te: eight output channels (16-byte chunk cc of the 128-channel tile) of rows rg*16 .. rg*16+15 of a stage
+        const int te = (warp - NI - 1) * 32 + lane, cc = te & 15, rg = te >> 4;
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        int st = 0, turn = 0; uint32_t ph = 0;      // turn: step % bias_sharers
+        const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16);
+        bool ok = true;
+        for (int zi = 0; zi < nz && ok; ++zi) {
+            const int zsteps = do_bias ? min(per, nsteps - zi * per) : 0;
+            for (int i = 0; i < zsteps; ++i) {
+                if (!(ok = mbar_wait_idle(full0 + 8u * st, ph, abort_flag))) break;
+                const bool mine = turn == bias_me;
+                if (++turn == p.bias_sharers) turn = 0;
+                if (mine) {
+                    const uint32_t a0 = base + st * stage_bytes + (uint32_t)(cc >> 3) * (kWgRows * 128u) + (uint32_t)rg * (kWgRows / 8 * 128u);
                     #pragma unroll
-                    for (int k = 0; k < 4; ++k) { const float2 f = __bfloat1622float2(hh[k]); acc[2 * k] += f.x; acc[2 * k + 1] += f.y; }
+                    for (int rr = 0; rr < kWgRows / 8; ++rr) {
+                        uint4 u;
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w)
+                                     : "r"(a0 + (uint32_t)rr * 128u + (uint32_t)(((cc & 7) ^ (rr & 7)) << 4)));
+                        const __nv_bfloat162* hh = (const __nv_bfloat162*)&u;
+                        #pragma unroll
+                        for (int k = 0; k < 4; ++k) { const float2 f = __bfloat1622float2(hh[k]); acc[2 * k] += f.x; acc[2 * k + 1] += f.y; }
+                    }
+                    // these were generic-proxy reads of a stage that TMA (the async proxy) overwrites once it is released: without
+                    // a proxy fence between the reads and the release the refill may overtake reads still in flight (seen as a
+                    // wrong bias partial in a few per cent of the steps, only when other kernels shared the GPU)
+                    fence_async_smem();
                 }
-                // these were generic-proxy reads of a stage that TMA (the async proxy) overwrites once it is released: without
-                // a proxy fence between the reads and the release the refill may overtake reads still in flight (seen as a
-                // wrong bias partial in a few per cent of the steps, only when other kernels shared the GPU)
-                fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty0 + 8u * st);
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
+            if (!ok || !(ok = mbar_wait_idle(accf0 + 8u * (zi & 1), (uint32_t)(zi >> 1) & 1u, abort_flag))) break;
+            tc_fence_after();
+            if (zi > 0) {          // this split's sums onto those of the splits before
+                #pragma unroll 1
+                for (int c = 0; c < acc_cols; c += 32) {
+                    uint32_t u[32], v[32];
+                    tmem_ld32(t0 + (uint32_t)c, u);
+                    tmem_ld32(t0 + (uint32_t)(acc_cols + c), v);
+                    tmem_ld_wait();
+                    #pragma unroll
+                    for (int q = 0; q < 32; ++q) u[q] = __float_as_uint(__uint_as_float(u[q]) + __uint_as_float(v[q]));
+                    tmem_st32(t0 + (uint32_t)c, u);
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acca);
+            }
+        }
+        if (ok) {
+            float* out = p.out + (long long)z * p.split_stride + (long long)(ky * p.kw + kx_lo) * p.tap_stride + (long long)(g * p.out_gx + row) * p.ldo + n_tile * 64;
+            const int nch = row_ok ? min(4, (p.n_valid - n_tile * 64) / 16) : 0;        // 16-column chunks that exist (n_valid is a multiple of 16)
+            #pragma unroll 1
+            for (int kx = 0; kx < kx_n; ++kx, out += p.tap_stride) {
+                uint32_t v[64];
+                tmem_ld32(t0 + (uint32_t)(kx * 64), v);
+                tmem_ld32(t0 + (uint32_t)(kx * 64 + 32), v + 32);
+                tmem_ld_wait();
+                #pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (c < nch) {
+                        #pragma unroll
+                        for (int q = 4 * c; q < 4 * c + 4; ++q)
+                            *(float4*)(out + 4 * q) = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+                    }
+            }
+        }
+        if (do_bias) {
             float* red = (float*)(smem_raw + (red_base - raw));     // [8 row groups][128 channels]
             #pragma unroll
             for (int k = 0; k < 8; ++k) red[rg * 128 + cc * 8 + k] = acc[k];
@@ -1604,22 +1694,7 @@ __global__ void __launch_bounds__(32 * 7, 1) wgrad_kernel(const __grid_constant_
                 float sum = 0.f;
                 #pragma unroll
                 for (int q = 0; q < 8; ++q) sum += red[q * 128 + te];
-                p.bias_partial[(size_t)z * p.bias_ld + g * p.out_gx + m_tile * 128 + te] = sum;
-            }
-        }
-        if (mbar_wait(accf, 0, abort_flag)) {
-            tc_fence_after();
-            const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16);
-            for (int kx = 0; kx < p.kw; ++kx) {
-                const long long row_off = (long long)z * p.split_stride + (long long)(ky * p.kw + kx) * p.tap_stride +
-                                          (long long)(g * p.out_gx + row) * p.ldo;
-                for (int c = 0; c < 64; c += 16) {
-                    uint32_t v[16];
-                    tmem_ld16(t0 + (uint32_t)(kx * 64 + c), v);
-                    tmem_ld_wait();
-                    if (!row_ok) continue;
-                    epi_chunk(p, v, nsteps <= 0, false, row_off, n_tile * 64 + c, g);
-                }
+                p.bias_partial[(size_t)(z * p.bias_sharers + bias_me) * p.bias_ld + g * p.out_gx + m_tile * 128 + te] = sum;
             }
         }
     }

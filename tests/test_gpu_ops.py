@@ -115,6 +115,35 @@ def test_conv_backward_weight_and_bias(net, params, name, tin, tdy, shp, ho):
     assert rel(g[o:o + n], db) < 1e-3
 
 
+# one CTA per tile for all row splits / a CTA per split: the line lies between batch 71 and 72 for the 13 x 13 layers, between 16
+# and 17 for conv2 (whose filter rows are then cut in two) and between 4 and 5 for conv1
+@pytest.mark.parametrize("batch", [1, 4, 5, 17, 71, 72])
+def test_conv_backward_weight_over_batches(batch):
+    import torch
+    from paper_1412_2302_b200.alexnet import AlexNet
+    n = AlexNet(batch=batch, seed=SEED, mean_image=synth.mean_image(SEED))
+    off, _ = O.param_offsets()
+    for name, tin, tdy, shp, ho in WG:
+        if batch > 20 and name in ("conv1", "conv2"):
+            continue
+        c = O.CONV[name]
+        x = synth.bf16_grid(SEED, 51 + tag(name), (batch,) + shp, -1, 1)
+        dy = synth.bf16_grid(SEED, 52 + tag(name), (batch, c["cout"], ho, ho), -1, 1)
+        n.set_tensor(tin, x)
+        n.set_tensor(tdy, dy)
+        n.run_op(name.upper() + "_BWD_WEIGHT")
+        n.sync()
+        o, cnt, shape = off[name + ".W"]
+        xt, dt = torch.from_numpy(np.ascontiguousarray(x)).cuda().double(), torch.from_numpy(np.ascontiguousarray(dy)).cuda().double()
+        dw = torch.nn.grad.conv2d_weight(xt, shape, dt, stride=c["s"], padding=c["p"], groups=c["g"]).cpu().numpy().ravel()
+        db = dt.sum((0, 2, 3)).cpu().numpy()
+        g = n.get_params(0, 2)
+        # exact products and 32-bit sums of at most 72 * 13 * 13 or 17 * 27 * 27 terms: 2^-24 sqrt(12393) = 7e-6
+        assert rel(g[o:o + cnt], dw) < 2e-5, (name, rel(g[o:o + cnt], dw))
+        o, cnt, _ = off[name + ".b"]
+        assert rel(g[o:o + cnt], db) < 2e-5, (name, rel(g[o:o + cnt], db))
+
+
 FCS = [("fc6", "P5", "F6", "M6", 2), ("fc7", "F6", "F7", "M7", 3), ("fc8", "F7", "Z", None, None)]
 
 
