@@ -1001,7 +1001,12 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
                                                                int* __restrict__ done_counter, int B, int N,
                                                                int32_t* __restrict__ counts, const int* __restrict__ status,
                                                                HostResult* host_out, uint32_t seq) {
-    pdl_sync();
+    pdl_trigger();
+    // the bias and the labels were written before the pass began: fetched while the predecessor runs
+    const int lab = labels[blockIdx.x];
+    float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((N & 3) == 0 && 4 * (int)threadIdx.x < N) b4 = __ldg((const float4*)bias + threadIdx.x);
+    pdl_wait();
     __shared__ float red[32];
     __shared__ __align__(16) float zs[1024];
     __shared__ int last;
@@ -1012,7 +1017,7 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
         // sees which column; the sums below keep the column -> thread mapping of softmax_xent_kernel)
         for (int j = 4 * tid; j < N; j += 1024) {
             const long long t = (long long)n * N + j;
-            const float4 b4 = __ldg((const float4*)(bias + j));
+            if (j >= 1024) b4 = __ldg((const float4*)(bias + j));
             float4 v = sum_splits<16>(ws + t, split_stride, splits);
             v.x += b4.x; v.y += b4.y; v.z += b4.z; v.w += b4.w;
             *(float4*)(z + t) = v;
@@ -1043,12 +1048,12 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
     __syncthreads();
     sum = 0.f;
     for (int w = 0; w < 8; ++w) sum += red[w];
-    const int lab = labels[n];
     const float inv = 1.f / sum, invB = 1.f / (float)B;
     for (int j = tid; j < N; j += 256) {
         const float pj = expf(zs[j] - mx) * inv;
         dz[(size_t)n * N + j] = __float2bfloat16_rn((pj - (j == lab ? 1.f : 0.f)) * invB);
     }
+    int top1 = 0, top5 = 0;
     if (EVAL) {
         const float zl = zs[lab];
         int c = 0;
@@ -1060,9 +1065,22 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
         if (tid == 0) {
             int k = 0;
             for (int w = 0; w < 8; ++w) k += __float_as_int(red[w]);
-            if (k < 1) atomicAdd(counts, 1);
-            if (k < 5) atomicAdd(counts + 1, 1);
+            if (B == 1) {         // nobody to wait for: no counters
+                top1 = k < 1; top5 = k < 5;
+            } else {
+                if (k < 1) atomicAdd(counts, 1);
+                if (k < 5) atomicAdd(counts + 1, 1);
+            }
         }
+    }
+    if (B == 1) {
+        if (tid == 0) {
+            const float t = -(zs[lab] - mx - logf(sum));
+            loss_n[0] = t;
+            *loss_mean = t;
+            if (EVAL) publish_result(host_out, top1, top5, t, *(volatile const int*)status, seq);
+        }
+        return;
     }
     if (tid == 0) {
         loss_n[n] = -(zs[lab] - mx - logf(sum));

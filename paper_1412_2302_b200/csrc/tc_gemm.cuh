@@ -713,7 +713,7 @@ struct ConvParams {
     int* status;
     // FC forward with the split-K reduction inside the kernel: the `zcluster` CTAs of a thread-block cluster are the k splits
     // of one 128-row x BN tile (one tile per CTA, m_tiles == 1).  Each leaves its fp32 partial tile in its own shared
-    // memory; after a cluster barrier CTA z adds rows [z * 128 / zcluster, ...) of all partials in split order through
+    // memory; after a cluster barrier every CTA adds its share of the batch's rows over all partials in split order through
     // distributed shared memory and applies bias, ReLU and dropout (the arithmetic of fc_reduce_fwd_kernel, so the result
     // is bit-identical to the two-launch form), writing the layer's bf16 output and its keep mask.  0: off.
     int zcluster;
@@ -1049,7 +1049,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * acc_cols + h * BN);
                 if (zc) {
                     // the partial tile stays on chip: row r of the tile to the (idle) operand ring, 32 columns per unit
-                    for (int c = 0; c < BN; c += 32, ++unit) {
+                    for (int c = 0; c < BN && quad * 32 < p.M_total; c += 32, ++unit) {       // (quadrants past the batch are not read)
                         if (E == 2 && (unit & 1) != eset) continue;
                         uint32_t v[32];
                         tmem_ld32(t0 + (uint32_t)c, v);
@@ -1084,17 +1084,22 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
         cluster_sync_all();
         if (warp > MH + 1) {
             const int T = 128 * p.epi_sets, t = (warp - (MH + 2)) * 32 + lane;
-            const int rows_per = 128 / zdiv, n0 = ((int)blockIdx.x / zdiv) * BN;
-            for (int idx = t; idx < rows_per * 32; idx += T) {
-                const int row = zrank * rows_per + (idx >> 5), c4 = idx & 31;
+            // The batch's rows of the tile are dealt out evenly, in quarters of rows, and all remote loads of a thread are in flight
+            // together.  With a fixed 32 rows per CTA at any batch and one load at a time: fc6 22.7 -> 21.2 us at batch 1 and 8,
+            // 23.7 -> 21.6 at 32, 24.4 -> 24.2 at 128 (bound by distributed shared memory: about 8 B/clk per SM); fc7 alike.
+            const int n0 = ((int)blockIdx.x / zdiv) * BN, total = p.M_total * 32, each = (total + zdiv - 1) / zdiv;
+            for (int idx = zrank * each + t; idx < min(total, (zrank + 1) * each); idx += T) {
+                const int row = idx >> 5, c4 = idx & 31;
                 const uint32_t local = ring_a + (uint32_t)(row * kZcPitch + 4 * c4) * 4u;
+                float4 v[8];
+                #pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q < zc)
+                        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[q].x), "=f"(v[q].y), "=f"(v[q].z), "=f"(v[q].w) : "r"(mapa_u32(local, (uint32_t)q)) : "memory");
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int q = 0; q < zc; ++q) {
-                    float4 v;
-                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(mapa_u32(local, (uint32_t)q)) : "memory");
-                    acc[0] += v.x; acc[1] += v.y; acc[2] += v.z; acc[3] += v.w;
-                }
-                if (row >= p.M_total) continue;
+                #pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q < zc) { acc[0] += v[q].x; acc[1] += v[q].y; acc[2] += v[q].z; acc[3] += v[q].w; }
                 const int n = n0 + 4 * c4;
                 if (n >= p.n_valid) continue;                      // n_valid is a multiple of 4 in the layers that run this way
                 const long long tt = (long long)row * p.n_valid + n;
