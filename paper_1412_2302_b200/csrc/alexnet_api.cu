@@ -805,14 +805,19 @@ int build_plans(alexnet* h, int r) {
 }
 
 // An evaluation whose images come over PCIe works in chunks of images: the convolution layers of one chunk run while the next is
-// copied (3.6 us per image); what is left behind the last copy is one chunk's time and the FC layers.  A chunk's dependent launches
-// cost a fixed time and small grids fill the machine badly, so chunks below about 50 images take longer than the copy they should
-// hide behind and the delay adds up from chunk to chunk, while two chunks can be smaller, since only the first has to keep up.
-// Measured, 3 / 4 / 5 chunks: 256 images 1238 / 1217 / 1310 us; 4 / 5 / 6: 320 images 1495 / 1483 / 1574; 7 / 8 / 9: 512 images 2201 / 2195 /
-// 2259; one / two: 56 images 450 / 473, 64 487 / 503, 72 538 / 524, 80 572 / 545.
-constexpr int kEvalChunk = 64, kEvalTwoChunks = 68;
-int eval_chunks(int B) { return std::max(B >= kEvalTwoChunks ? 2 : 1, B / kEvalChunk); }
-inline int chunk_begin(int B, int chunks, int c) { return (int)((long long)B * c / chunks); }
+// copied (3.2 us per image: the 227 rows of the crop).  What is left behind the last copy is one chunk's time and the FC layers.  A
+// chunk's dependent launches cost a fixed time and small grids fill the machine badly, so chunks below about 70 images take
+// longer than the copy they should hide behind and the delay adds up from chunk to chunk, while two chunks can be smaller:
+// only the first has to keep up, and it is the smaller one, so that it ends when the second has arrived.
+// Measured, 1 / 2 chunks: 64 images 464 / 484 us, 72 512 / 490, 100 656 / 593 (two equal ones: 616); 2 / 3: 192 961 / 949, 240 1150 / 1089;
+// 3 / 4: 256 1141 / 1186, 300 1344 / 1337, 320 - / 1376; 5 / 6 / 7: 512 2061 / 2015 / 2100.
+constexpr int kEvalTwoChunks = 68, kEvalThreeChunks = 192, kEvalChunk = 75;
+constexpr size_t kEvalRow0 = 14;      // first source row of the centre crop (preprocess_kernel)
+int eval_chunks(int B) { return B < kEvalTwoChunks ? 1 : B < kEvalThreeChunks ? 2 : std::max(3, B / kEvalChunk); }
+inline int chunk_begin(int B, int chunks, int c) {
+    if (chunks == 2 && c == 1) return (56 * B - 1050) / 100;
+    return (int)((long long)B * c / chunks);
+}
 
 // ---------------------------------------------------------------- launches
 inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
@@ -1178,17 +1183,22 @@ void op_average(alexnet* h, cudaStream_t st) {
     h->launches++;
     refresh_transposed_both(h, st);
 }
-// labels != nullptr: taken along by the kernel (see label_source)
+// labels != nullptr: taken along by the kernel (see label_source); src: the images, where they are not in the slot's staging buffer
 void op_preprocess(alexnet* h, int r, int slot, uint64_t step, cudaStream_t st, bool eval = false, const int32_t* labels = nullptr, int i0 = 0,
-                   int images = 0) {
+                   int images = 0, const uint8_t* src = nullptr) {
     Replica& R = h->rep[r];
     if (!images) images = h->B;
     kn::ColorAug aug = h->color;
     aug.key = kn::stream_key(h->cfg.seed, 10, r, step);
     const bool augment = aug.sigma != 0.f && !eval;
-    launch_k(augment ? kn::preprocess_kernel<true> : kn::preprocess_kernel<false>, dim3(images, 57), 256, 0, st, R.stage[slot], h->mean, R.x0[slot],
+    launch_k(augment ? kn::preprocess_kernel<true> : kn::preprocess_kernel<false>, dim3(images, 57), 256, 0, st, src ? src : R.stage[slot], h->mean, R.x0[slot],
              R.cf[slot], labels, R.labels[slot], i0, kn::stream_key(h->cfg.seed, 1, r, step), eval ? 1 : 0, aug);
     h->launches++;
+}
+int current_device() {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    return dev;
 }
 // the address under which a kernel on this device can read the caller's labels, or nullptr (then they are copied)
 const int32_t* label_source(const int32_t* labels) {
@@ -1772,8 +1782,13 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     ++h->result_seq;
     // the copies run on the copy stream, everything else (preprocessing too) on the compute stream
     cudaPointerAttributes at{};
-    const bool on_device = cudaPointerGetAttributes(&at, images) == cudaSuccess && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
-    cudaGetLastError();
+    if (cudaPointerGetAttributes(&at, images) != cudaSuccess) { cudaGetLastError(); at = cudaPointerAttributes{}; }
+    const bool on_device = at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged, pinned = at.type == cudaMemoryTypeHost;
+    // The call ends when the batch has been evaluated, so preprocessing may read images in device memory where they are (16-byte
+    // vectors): 1 image 145 -> 134 us, 256 images 632 -> 615.  (Images in pinned host memory read that way: 1 image 145
+    // us against 143 with the copy, 8 221 against 184.)
+    const uint8_t* src = nullptr;
+    if (at.type == cudaMemoryTypeDevice && at.device == current_device() && ((uintptr_t)at.devicePointer & 15) == 0) src = (const uint8_t*)at.devicePointer;
     const int chunks = on_device || h->prof ? 1 : eval_chunks(h->B);
     while ((int)h->ev_chunk.size() < chunks) {
         cudaEvent_t e;
@@ -1783,10 +1798,13 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     ConvProgress done = {};
     for (int c = 0; c < chunks; ++c) {
         const size_t i0 = chunk_begin(h->B, chunks, c), n = chunk_begin(h->B, chunks, c + 1) - i0;
-        CK(cudaMemcpyAsync(R.stage[s] + i0 * 196608, images + i0 * 196608, n * 196608, cudaMemcpyDefault, h->ls));
+        // of an image in pinned memory only the rows of the centre crop are copied
+        const size_t at0 = i0 * 196608 + kEvalRow0 * 768;
+        if (!src && pinned) CK(cudaMemcpy2DAsync(R.stage[s] + at0, 196608, images + at0, 196608, 227 * 768, n, cudaMemcpyDefault, h->ls));
+        else if (!src) CK(cudaMemcpyAsync(R.stage[s] + i0 * 196608, images + i0 * 196608, n * 196608, cudaMemcpyDefault, h->ls));
         CK(cudaEventRecord(h->ev_chunk[c], h->ls));
         CK(cudaStreamWaitEvent(h->cs, h->ev_chunk[c], 0));
-        op_preprocess(h, replica, s, 0, h->cs, true, lsrc, (int)i0, (int)n);
+        op_preprocess(h, replica, s, 0, h->cs, true, lsrc, (int)i0, (int)n, src);
         if (chunks > 1) forward_conv_chunk(h, replica, s, (int)(i0 + n), done, h->cs);
     }
     if (chunks > 1) forward_fc(h, replica, s, h->cs, true);

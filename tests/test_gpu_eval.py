@@ -107,3 +107,22 @@ def test_eval_in_chunks_is_bit_for_bit_the_one_pass(B):
         assert got[0][0] == got[1][0]
         assert np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][2], got[1][2])
     net.close()
+
+
+def test_eval_images_where_they_are():
+    """Aligned images on the device are read in place, others are copied first, and of pinned images only the crop's rows travel: one result."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed, B = synth.BASE_SEED + 34, 3
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    net.set_params(synth.init_params(seed, variance_preserving=True, bias=0.1))
+    gen = torch.Generator().manual_seed(B)
+    lab = torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen)
+    img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen)
+    shifted = torch.zeros(img.numel() + 16, dtype=torch.uint8, device="cuda")
+    odd = shifted[5:5 + img.numel()].view(img.shape)
+    odd.copy_(img)
+    torch.cuda.synchronize()
+    got = [(net.eval_batch(0, im, lab.pin_memory()), net.get_tensor("X0"), net.get_tensor("Z")) for im in (img.cuda(), odd, img.pin_memory(), img)]
+    for g in got[1:]:
+        assert g[0] == got[0][0] and np.array_equal(g[1], got[0][1]) and np.array_equal(g[2], got[0][2])
+    net.close()
