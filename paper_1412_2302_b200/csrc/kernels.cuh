@@ -865,13 +865,19 @@ __global__ void colsum_scalar_kernel(const __nv_bfloat16* __restrict__ dy, int r
 // blocks in the low 16 bits of a word whose upper bits are the number of the launch: the first block of a launch sets the
 // word to its number and a count of zero (a maximum: every later block of the launch leaves the count alone), so a launch
 // owes nothing to what an earlier one left there, be it one that overlapped another or one that died.  HBM-bound (L2-bound
-// where dy fits); 25088 x 384 took 12.2 us per call as two launches with one load in flight per thread, 7.6 us in this form,
-// about half of it the launch.
-__global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
-                                                        unsigned long long* __restrict__ counters, unsigned long long launch,
-                                                        float* __restrict__ db) {
+// where dy fits); what it spends beside that is the launch and the tail of the last block.  Hence one block of 1024 threads per SM
+// and not four of 256: a quarter of the partials and of the atomics on a group's word, and one round of loads in the tail.
+// Per call, four blocks of 256 / one of 1024: 25088 x 384 7.33 / 6.26 us, 60000 x 2048 47.4 / 41.1, 8000 x 104 7.0 / 5.5, 3000 x 384 6.3 /
+// 5.6, 3000 x 104 5.05 / 4.95.  Below that the larger block only takes longer to start (1500 x 104 4.3 / 4.9, 700 x 384 4.1 to 4.4 / 4.9),
+// so calls of fewer than 300 thousand elements keep blocks of 256.
+constexpr long long kBgSmall = 300000;
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
+                                                               unsigned long long* __restrict__ counters, unsigned long long launch,
+                                                               float* __restrict__ db) {
     pdl_sync();
-    __shared__ __align__(16) float red[16][68];
+    constexpr int RL = THREADS / 8, WARPS = THREADS / 32, ZL = THREADS / 16;       // lanes over the rows; over the splits in the tail
+    __shared__ __align__(16) float red[WARPS][68];
     __shared__ bool last;
     const int tid = threadIdx.x, cc = tid & 7, rl = tid >> 3;
     const int c0 = blockIdx.x * 64 + cc * 8;
@@ -879,12 +885,12 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
     const long long r0 = (long long)blockIdx.y * per, r1 = min(rows, r0 + per);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (c0 < C) {
-        for (long long r = r0 + rl; r < r1; r += 32 * 8) {
+        for (long long r = r0 + rl; r < r1; r += RL * 8) {
             uint4 u[8];
             #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 u[q] = make_uint4(0u, 0u, 0u, 0u);
-                if (r + 32 * q < r1) u[q] = __ldg((const uint4*)(dy + (r + 32 * q) * C + c0));
+                if (r + RL * q < r1) u[q] = __ldg((const uint4*)(dy + (r + RL * q) * C + c0));
             }
             #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -909,7 +915,7 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
     if (tid < 64 && c < C) {
         float s = 0.f;
         #pragma unroll
-        for (int w = 0; w < 8; ++w) s += red[w][tid];
+        for (int w = 0; w < WARPS; ++w) s += red[w][tid];
         if (splits == 1) db[c] = s;
         else partial[(size_t)blockIdx.y * C + c] = s;
     }
@@ -925,19 +931,15 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
     __threadfence();
     const int q4 = tid & 15, zl = tid >> 4, cq = blockIdx.x * 64 + 4 * q4;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (cq < C) {
-        #pragma unroll 4
-        for (int z = zl; z < splits; z += 16) {
-            const float4 t = __ldcg((const float4*)(partial + (size_t)z * C + cq));
-            a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
-        }
-    }
-    *(float4*)&red[zl][4 * q4] = a;
+    if (cq < C && zl < splits) a = sum_splits<THREADS == 1024 ? 3 : 8>(partial + (size_t)zl * C + cq, (long long)ZL * C, (splits - zl + ZL - 1) / ZL);
+    a.x += __shfl_xor_sync(~0u, a.x, 16); a.y += __shfl_xor_sync(~0u, a.y, 16);
+    a.z += __shfl_xor_sync(~0u, a.z, 16); a.w += __shfl_xor_sync(~0u, a.w, 16);
+    if ((tid & 31) < 16) *(float4*)&red[tid >> 5][4 * q4] = a;
     __syncthreads();
     if (tid < 64 && c < C) {
         float s = 0.f;
         #pragma unroll
-        for (int w = 0; w < 16; ++w) s += red[w][tid];
+        for (int w = 0; w < WARPS; ++w) s += red[w][tid];
         db[c] = s;
     }
 }

@@ -121,3 +121,17 @@ def test_bias_grad_noalloc_after_calls_that_overlapped():
             torch.cuda.synchronize()
             # multiples of 1/64: the fp32 sums are exact
             assert np.array_equal(out.cpu().numpy().astype(np.float64), host_colsum(t))
+
+
+# around the line between the two block sizes (300 thousand elements), with one split, the most splits, and remainders of the row lanes
+@pytest.mark.parametrize("rows,C", [(1, 8), (65, 4096), (74, 4096), (781, 384), (782, 384), (4687, 64), (4688, 64), (9473, 64), (20011, 72)])
+def test_bias_grad_noalloc_block_sizes(rows, C):
+    from paper_1412_2302_b200 import alexnet as A
+    rng = np.random.default_rng(rows + C)
+    x = torch.from_numpy((rng.integers(-64, 65, size=(rows, C)) / 64.0).astype(np.float32)).to(torch.bfloat16).cuda()
+    db = torch.full((C,), float("nan"), device="cuda")
+    for _ in range(2):
+        A.bias_grad_noalloc(x, db)
+        torch.cuda.synchronize()
+        # multiples of 1/64 below 2^18 in all: 32-bit sums are exact in any order
+        assert np.array_equal(db.cpu().numpy().astype(np.float64), host_colsum(x)), (rows, C)
