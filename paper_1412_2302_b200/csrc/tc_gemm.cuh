@@ -725,7 +725,7 @@ struct ConvParams {
     void* out;
     int* status;
     // FC forward with the split-K reduction inside the kernel: the `zcluster` CTAs of a thread-block cluster are the k splits
-    // of one 128-row x BN tile (one tile per CTA, m_tiles == 1).  Each leaves its fp32 partial tile in its own shared
+    // of one 128-row x BN tile (one tile per CTA; 1: no splits, the CTA finishes its own tile).  Each leaves its fp32 partial tile in its own shared
     // memory; after a cluster barrier every CTA adds its share of the batch's rows over all partials in split order through
     // distributed shared memory and applies bias, ReLU and dropout (the arithmetic of fc_reduce_fwd_kernel, so the result
     // is bit-identical to the two-launch form), writing the layer's bf16 output and its keep mask.  0: off.
@@ -802,7 +802,8 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
     const int zc = CG == 1 ? p.zcluster : 0;
     const int zrank = zc ? (int)cluster_ctarank() : 0;
     const int zdiv = zc ? zc : 1;
-    if (zc) { vb = zrank * p.n_tiles + (int)blockIdx.x / zdiv; vgrid = p.tiles_total; }    // split zrank of n tile blockIdx / zc; one tile
+    // split zrank of row tile blockIdx.y, n tile blockIdx.x / zc; one tile
+    if (zc) { vb = (zrank * p.n_tiles + (int)blockIdx.x / zdiv) * p.m_tiles + (int)blockIdx.y; vgrid = p.tiles_total; }
     const int tile_rows = 128 * MH * CG, row0 = rank * 128 * MH;
     const int cpg = p.cpg, gw = cpg > 1 ? cpg : p.kw;            // weight tiles per A stage
     const uint32_t a_box_bytes = (uint32_t)p.a_box_rows * 128u, a_bytes = a_box_bytes * MH * cpg, b_bytes = (uint32_t)(BN / CG) * 128u;
@@ -1064,7 +1065,7 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
                 const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * acc_cols + h * BN);
                 if (zc) {
                     // the partial tile stays on chip: row r of the tile to the (idle) operand ring, 32 columns per unit
-                    for (int c = 0; c < BN && quad * 32 < p.M_total; c += 32, ++unit) {       // (quadrants past the batch are not read)
+                    for (int c = 0; c < BN && m0 + quad * 32 < p.M_total; c += 32, ++unit) {       // (quadrants past the batch are not read)
                         if (E == 2 && (unit & 1) != eset) continue;
                         uint32_t v[32];
                         tmem_ld32(t0 + (uint32_t)c, v);
@@ -1102,10 +1103,11 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             // The batch's rows of the tile are dealt out evenly, in quarters of rows, and all remote loads of a thread are in flight
             // together.  With a fixed 32 rows per CTA at any batch and one load at a time: fc6 22.7 -> 21.2 us at batch 1 and 8,
             // 23.7 -> 21.6 at 32, 24.4 -> 24.2 at 128 (bound by distributed shared memory: about 8 B/clk per SM); fc7 alike.
-            const int n0 = ((int)blockIdx.x / zdiv) * BN, total = p.M_total * 32, each = (total + zdiv - 1) / zdiv;
+            const int row_0 = (int)blockIdx.y * 128, n0 = ((int)blockIdx.x / zdiv) * BN;
+            const int total = min(128, p.M_total - row_0) * 32, each = (total + zdiv - 1) / zdiv;
             for (int idx = zrank * each + t; idx < min(total, (zrank + 1) * each); idx += T) {
-                const int row = idx >> 5, c4 = idx & 31;
-                const uint32_t local = ring_a + (uint32_t)(row * kZcPitch + 4 * c4) * 4u;
+                const int row = row_0 + (idx >> 5), c4 = idx & 31;
+                const uint32_t local = ring_a + (uint32_t)((idx >> 5) * kZcPitch + 4 * c4) * 4u;
                 float4 v[8];
                 #pragma unroll
                 for (int q = 0; q < 8; ++q)
