@@ -153,9 +153,10 @@ struct Plan { tc::GemmParams p; tc::ConvParams c; tc::WgradParams w; tc::FcUpdPa
 // CTAs (one per SM) of the FC weight-gradient + update kernels; the SMs left over are those of the data gradients of conv5..conv3
 // that run beside them: fc_update_kernel reaches most of the HBM rate on this many SMs (see there), and a chain
 // kernel whose grid fits beside it neither waits for it nor leaves CTAs of a second wave behind.
-// Measured at batch 128 only (fc6 161 us on 64 SMs, 134 on 80); at smaller batches, where the chain beside the
-// updates is short, more SMs may pay.
-constexpr int kFcUpdCtas = 64;
+// Up to batch 16 the chain is short, the updates are what a step waits for, and they get 72.  One handle alone, 64 / 72 / 80 SMs: batch 1 425 /
+// 410 / 402 us, 4 449 / 426 / 437, 8 459 / 446 / 442, 16 489 / 477 / 481, 32 539 / 533 / 537; three handles taking turns, which fill one another's
+// gaps: 4 340 / 346 / 352, 8 374 / 376 / 377, 16 404 / 407 / 413.  At batch 128 (64 / 80): 976 / 1011.
+inline int fc_upd_ctas(int B) { return B <= 16 ? 72 : 64; }
 // Conv weight gradients of at most this many 128-row steps run with one CTA per tile, which takes all row splits in turn
 // (WgradParams::solo).  Below about batch 64 these kernels are not the longest branch, and a wave of CTAs of a few steps each costs
 // more than it saves: each takes a whole SM from the data gradients and the FC updates beside it for its set-up and epilogue,
@@ -726,7 +727,7 @@ int plan_fc_upd(alexnet* h, Plan& P, const FcL& f, const bf16* dy, const bf16* x
     if ((rc = make_tm_rows(h, &u.tmS, shadow, false, (uint64_t)f.K, (uint64_t)f.N, tc::kUpdRows))) return rc;
     P.upd = true; P.upd_K = f.K;
     P.smem = tc::fc_upd_smem_bytes(u.stages);
-    P.grid = std::min(u.tiles_total, std::min(kFcUpdCtas, h->sm_count));
+    P.grid = std::min(u.tiles_total, std::min(fc_upd_ctas(h->B), h->sm_count));
     P.valid = true;
     return ALEXNET_OK;
 }
@@ -790,7 +791,8 @@ int build_plans(alexnet* h, int r) {
         if ((rc = plan_conv_bwd(h, R.conv_bwd[l], c, dyv[l], R.wt + c.wt_off, maskv[l], dxv[l]))) return rc;
         Plan& P = R.conv_bwd_beside[l];
         P = R.conv_bwd[l];          // same tiles, fewer CTAs
-        if (l >= 2 && h->sm_count > kFcUpdCtas + 1) P.grid = std::min(P.grid, (h->sm_count - kFcUpdCtas) / P.c.cg * P.c.cg);
+        const int upd = fc_upd_ctas(h->B);
+        if (l >= 2 && h->sm_count > upd + 1) P.grid = std::min(P.grid, (h->sm_count - upd) / P.c.cg * P.c.cg);
     }
     const bf16* fx[3] = {R.p5, R.f6, R.f7};
     const bf16* fdy[3] = {R.df6, R.df7, R.dz};
