@@ -293,8 +293,10 @@ int alexnet_set_tensor(alexnet_t* h, int replica, int tensor_id, const float* ho
 /* Run one operation of the step `iters` times on the replica's current
  * tensors (compute stream, asynchronous), for per-layer parity and timing.
  * Operation ids: ALEXNET_OP_*.  Operations that read a batch slot (conv1,
- * softmax labels, preprocess) and get/set_tensor of X0 and CROPFLIP use the slot
- * touched by the most recent load_batch_async or train_step of that replica. */
+ * softmax labels) and get/set_tensor of X0 and CROPFLIP use the slot touched by
+ * the most recent load_batch_async, train_step or eval_batch of that replica;
+ * preprocess takes the images of the most recent load_batch_async or train_step
+ * (an evaluation does not keep all rows of its images) and its slot from then on. */
 enum {
     ALEXNET_OP_CONV1_FWD = 0, ALEXNET_OP_CONV2_FWD, ALEXNET_OP_CONV3_FWD, ALEXNET_OP_CONV4_FWD, ALEXNET_OP_CONV5_FWD,
     ALEXNET_OP_CONV2_BWD_DATA, ALEXNET_OP_CONV3_BWD_DATA, ALEXNET_OP_CONV4_BWD_DATA, ALEXNET_OP_CONV5_BWD_DATA,

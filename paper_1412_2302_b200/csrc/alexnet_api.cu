@@ -183,7 +183,9 @@ struct Replica {
     cudaEvent_t ready[2], consumed[2];
     bool consumed_valid[2];
     uint64_t slot_step[2];
-    int next_load, next_train, loaded, last_slot;
+    int next_load, next_train, loaded;
+    int last_slot;          // the slot of the last load, training pass or evaluation: whose X0, crops and labels the operations read
+    int image_slot;         // the slot of the last load or training pass: whose staging buffer holds a whole batch
     // the step fuses LRN with pooling and never writes n1/n2 or dn1/dn2; get_tensor fills them in on demand
     bool n_stale[2], dn_stale[2];
     // plans
@@ -1556,6 +1558,7 @@ int alexnet_create(const alexnet_config_t* cfg, void* dev_arena, size_t arena_by
     for (int r = 0; r < cfg->replicas; ++r) {
         Replica& R = h->rep[r];
         R.next_load = R.next_train = R.loaded = R.last_slot = 0;
+        R.image_slot = 1;       // (nothing loaded: the slot that an evaluation does not use, zeros)
         R.n_stale[0] = R.n_stale[1] = R.dn_stale[0] = R.dn_stale[1] = false;
         R.grad_pending = false;
         for (int s = 0; s < 2; ++s) {
@@ -1599,7 +1602,7 @@ int alexnet_load_batch_async(alexnet_t* h, int replica, const uint8_t* images, c
     CK(cudaEventRecord(R.ready[s], h->ls));
     if (int rc = launches_ok(h)) return rc;
     R.slot_step[s] = step;
-    R.last_slot = s; R.next_load ^= 1; R.loaded++;
+    R.last_slot = R.image_slot = s; R.next_load ^= 1; R.loaded++;
     return ALEXNET_OK;
 }
 
@@ -1622,7 +1625,7 @@ static int step_impl(alexnet_t* h, int replica, float* host_loss, bool with_upda
     R.consumed_valid[s] = true;
     if (with_update) op_update(h, replica, h->cs, false, 1.f, defer ? s : -1);
     R.grad_pending = !with_update;
-    R.last_slot = s; R.next_train ^= 1; R.loaded--;
+    R.last_slot = R.image_slot = s; R.next_train ^= 1; R.loaded--;
     if (int rc = launches_ok(h)) return rc;
     if (host_loss) {
         launch_k(kn::store_result_kernel, 1, 1, 0, h->cs, (const float*)R.loss, (const int*)h->status, h->host_result, ++h->result_seq);
@@ -1778,7 +1781,7 @@ int alexnet_eval_batch(alexnet_t* h, int replica, const uint8_t* images, const i
     if (int rc = check_status(h)) return rc;
     Replica& R = h->rep[replica];
     if (R.loaded != 0) return fail(h, ALEXNET_ERR_STATE, "eval_batch: a loaded training batch is waiting for its train_step");
-    const int s = R.next_load;      // the free slot the next training load would use; it stays free afterwards
+    const int s = R.next_load;      // the free slot the next training load would use; it stays free afterwards, and is never R.image_slot
     if (R.consumed_valid[s]) CK(cudaStreamWaitEvent(h->ls, R.consumed[s], 0));
     const int32_t* lsrc = label_source(labels);
     if (!lsrc) CK(cudaMemcpyAsync(R.labels[s], labels, (size_t)h->B * sizeof(int32_t), cudaMemcpyDefault, h->ls));
@@ -1980,7 +1983,11 @@ int alexnet_run_op(alexnet_t* h, int replica, int op, int iters) {
         else if (op == ALEXNET_OP_SOFTMAX) op_softmax(h, replica, slot, st);
         else if (op == ALEXNET_OP_UPDATE) op_update(h, replica, st, true);
         else if (op == ALEXNET_OP_AVERAGE) op_average(h, st);
-        else if (op == ALEXNET_OP_PREPROCESS) op_preprocess(h, replica, slot, R.slot_step[slot], st);
+        else if (op == ALEXNET_OP_PREPROCESS) {
+            // (an evaluation leaves at most the rows of its centre crop in its staging buffer)
+            R.last_slot = R.image_slot;
+            op_preprocess(h, replica, R.image_slot, R.slot_step[R.image_slot], st);
+        }
         else if (op == ALEXNET_OP_CONV1_BWD_DATA) op_conv_bwd(h, replica, 0, st);
         else if (op == ALEXNET_OP_LRN1_POOL1_FWD || op == ALEXNET_OP_LRN2_POOL2_FWD) op_lrn_pool_fwd(h, replica, op - ALEXNET_OP_LRN1_POOL1_FWD, st);
         else if (op == ALEXNET_OP_POOL1_LRN1_BWD || op == ALEXNET_OP_POOL2_LRN2_BWD) op_pool_lrn_bwd(h, replica, op - ALEXNET_OP_POOL1_LRN1_BWD, st);

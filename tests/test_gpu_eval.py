@@ -126,3 +126,28 @@ def test_eval_images_where_they_are():
     for g in got[1:]:
         assert g[0] == got[0][0] and np.array_equal(g[1], got[0][1]) and np.array_equal(g[2], got[0][2])
     net.close()
+
+
+@pytest.mark.parametrize("where", ["pinned", "device", "pageable"])
+def test_preprocessing_after_an_evaluation(where):
+    """run_op("PREPROCESS") takes the images of the batch loaded last; an evaluation in between, which keeps the rows of its crop at
+    most, leaves them alone wherever its own images are."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed, B = synth.BASE_SEED + 35, 5
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    gen = torch.Generator().manual_seed(B)
+    lab = torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen).pin_memory()
+    for step in range(3):                              # (both batch slots)
+        net.load_batch_async(0, torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen).pin_memory(), lab, step)
+        net.train_step(0)
+        net.sync()
+        want = net.get_tensor("CROPFLIP"), net.get_tensor("X0")
+        img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen)
+        img = img.pin_memory() if where == "pinned" else img.cuda() if where == "device" else img
+        torch.cuda.synchronize()
+        net.eval_batch(0, img, lab)
+        assert not np.array_equal(net.get_tensor("X0"), want[1])
+        net.run_op("PREPROCESS")
+        net.sync()
+        assert np.array_equal(net.get_tensor("CROPFLIP"), want[0]) and np.array_equal(net.get_tensor("X0"), want[1])
+    net.close()
