@@ -440,7 +440,7 @@ void finish_plan(const alexnet* h, Plan& P) {
     p.splits = (p.steps_total + per - 1) / per;
     p.steps_per_split = per;
     p.tiles_total = p.m_tiles * p.n_tiles * p.groups * p.taps_grid * p.splits;
-    P.smem = tc::smem_bytes(stage_bytes, stages);
+    P.smem = tc::own_sm(tc::smem_bytes(stage_bytes, stages));
     P.grid = std::min(p.tiles_total, h->sm_count);   // persistent: one CTA per SM walks the tile list
     P.valid = true;
 }
@@ -528,7 +528,7 @@ void finish_conv_plan(const alexnet* h, Plan& P) {
         c.b_stages = (int)std::min<size_t>(8, (budget - c.a_stages * a_bytes) / g_bytes);
     }
     P.conv = true;
-    P.smem = tc::conv_smem_bytes(c);
+    P.smem = tc::own_sm(tc::conv_smem_bytes(c));
     c.rot_mod = std::min(c.tiles_total, h->sm_count / c.cg);
     P.grid = c.cg * c.rot_mod;     // persistent: CTAs (or CTA pairs) walk the tile list
     P.valid = true;
@@ -632,7 +632,7 @@ int plan_conv_wg(alexnet* h, Plan& P, int l, const ConvL& c, const bf16* dy, con
     if ((rc = make_tm(h, &p.tmA, dy, c.cout, M, (uint64_t)c.cout * 2, tc::kWgRows))) return rc;
     if ((rc = make_tm(h, &p.tmB, xin, c.cin, M, (uint64_t)c.cin * 2, tc::kWgRows + 8))) return rc;
     P.wgrad = true;
-    P.smem = tc::wgrad_smem_bytes(p);
+    P.smem = tc::own_sm(tc::wgrad_smem_bytes(p));
     P.grid = p.tiles_total;
     P.valid = true;
     return ALEXNET_OK;
@@ -728,7 +728,7 @@ int plan_fc_upd(alexnet* h, Plan& P, const FcL& f, const bf16* dy, const bf16* x
     if ((rc = make_tm_rows(h, &u.tmV, v, true, (uint64_t)f.K, (uint64_t)f.N, tc::kUpdRows))) return rc;
     if ((rc = make_tm_rows(h, &u.tmS, shadow, false, (uint64_t)f.K, (uint64_t)f.N, tc::kUpdRows))) return rc;
     P.upd = true; P.upd_K = f.K;
-    P.smem = tc::fc_upd_smem_bytes(u.stages);
+    P.smem = tc::own_sm(tc::fc_upd_smem_bytes(u.stages));
     P.grid = std::min(u.tiles_total, std::min(fc_upd_ctas(h->B), h->sm_count));
     P.valid = true;
     return ALEXNET_OK;

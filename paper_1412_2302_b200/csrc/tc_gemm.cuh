@@ -465,6 +465,15 @@ __global__ void __launch_bounds__(32) wait_probe_kernel(int* status, long long b
 
 constexpr int kABytes = 128 * 128;  // 128 rows x 64 bf16, or 2 boxes of 64 x 64
 
+// Every CTA that allocates tensor memory asks for at least this much shared memory, more than half of an SM's 228 KB with the 1 KB that the
+// system takes per CTA, so that no two of them share an SM.  tcgen05.alloc waits, without a bound, while another CTA
+// holds the columns; a CTA has let the next launch of its stream start by then, and that launch's CTAs hold columns while they wait for this
+// one to end: two streams whose CTAs met on two SMs could wait for one another for good.  (The convolution rings of
+// batch 1 to 5 are smaller, 84 to 101 KB; there the registers happened to keep two CTAs apart.)
+constexpr size_t kOwnSmSmem = 114 * 1024;
+static_assert(2 * (kOwnSmSmem + 1024) > 228 * 1024, "two CTAs would fit on an SM");
+inline size_t own_sm(size_t smem) { return smem < kOwnSmSmem ? kOwnSmSmem : smem; }
+
 __host__ __device__ inline int b_stage_bytes(int BN) { return ((BN + 63) / 64) * 8192; }
 inline size_t smem_bytes(int stage_bytes, int stages) { return 1024 + (size_t)stages * stage_bytes + 4 * kEpiStageBytes + 512; }
 
