@@ -202,6 +202,8 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
@@ -212,8 +214,15 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(cluster_bar) : "memory");
 }
+// Tensor memory of a CTA pair: allocation, deallocation and the permit to allocate are operations of the PAIR, of which one warp of
+// each CTA issues its half.  Both CTAs must be there for each of them: a cluster barrier before the allocation (the peer runs), one
+// between the allocation and giving up the permit (the peer has allocated too) and one behind the deallocation (neither leaves
+// before both have issued it).  Without these, a pair whose CTAs were far apart in time was left waiting inside tcgen05.alloc
+// for good: with three handles on one device, whose blocks delay one CTA of a pair and not the other, once in some thousand passes.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t smem_dst, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
@@ -801,6 +810,7 @@ template <int CG>
 __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_constant__ ConvParams p) {
     TL(long long* tl = g_timeline + (blockIdx.x % 160) * 16; if (threadIdx.x == 0) { tl[0] = gtime_ns(); tl[8] = 0; tl[10] = 0; tl[11] = 0; tl[7] = 0; })
     kn::pdl_trigger();
+    if (CG == 2) cluster_arrive();            // (this CTA runs)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -842,6 +852,8 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
         tma_prefetch_desc(&p.tmA);
         tma_prefetch_desc(&p.tmB);
     }
+    __syncwarp();
+    if (CG == 2) cluster_wait();              // the peer runs
     if (warp == 2) {
         if (CG == 2) tmem_alloc_pair(smem_u32((const void*)tmem_slot), ncols);
         else tmem_alloc(smem_u32((const void*)tmem_slot), ncols);
@@ -849,12 +861,16 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     __syncwarp();
-    if (CG == 2) cluster_sync_all();          // the peer's barriers exist before anything arrives on them
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    if (CG == 2) cluster_arrive();
     TL(if (threadIdx.x == 0) tl[12] = gtime_ns();)
     // barriers, TMEM and descriptors are set up; global memory is touched from here on (the weights possibly earlier)
     if (!(p.early_b && warp == 1)) kn::pdl_wait();
+    if (CG == 2) {
+        cluster_wait();                       // the peer has its tensor memory too, and its barriers exist before anything arrives on them
+        if (warp == 2) tmem_relinquish_pair();
+    }
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
     TL(if (threadIdx.x == 0) tl[1] = gtime_ns();)
     const int per = p.asteps_per_split, kw = p.kw;
 
@@ -1099,8 +1115,6 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
             else mbar_arrive(acce0 + 8u * ab);
             if (++ab == acc_stages) { ab = 0; aph ^= 1u; }
         }
-        if (p.tma_store && !zc && lane == 0) bulk_wait_all();
-        TL(if (ew == 0 && lane == 0) tl[15] = gtime_ns();)
     }
     if (zc) {
         // every CTA of the cluster has its partial tile in shared memory (all threads arrive: the barrier also orders the
@@ -1160,12 +1174,17 @@ __global__ void __launch_bounds__(kConvMaxThreads, 1) conv_kernel(const __grid_c
     }
     __syncwarp();
     if (CG == 2) cluster_sync_all();          // no CTA leaves while its peer may still arrive on its barriers
-    TL(if (threadIdx.x == 0) tl[2] = gtime_ns();)
     if (warp == 2) {
         tc_fence_after();
         if (CG == 2) tmem_dealloc_pair(tmem, ncols);
         else tmem_dealloc(tmem, ncols);
     }
+    if (CG == 2) { __syncwarp(); cluster_arrive(); }
+    // the last TMA stores land; the hand-over of the tensor memory and both cluster barriers above and below pass meanwhile
+    if (warp > MH + 1 && p.tma_store && !zc && lane == 0) bulk_wait_all();
+    TL(if (warp == MH + 2 && lane == 0) tl[15] = gtime_ns();)
+    if (CG == 2) { __syncwarp(); cluster_wait(); }      // no CTA leaves before its peer has deallocated as well
+    TL(if (threadIdx.x == 0) tl[2] = gtime_ns();)
 }
 
 // ===========================================================================

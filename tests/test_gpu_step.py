@@ -946,3 +946,63 @@ def test_profile_kinds_tell_the_fc_updates_from_the_gemms():
             ms, n = read()
             assert n == want and all((t > 0) == (k > 0) for t, k in zip(ms, n)), (ms, n)
     net.close()
+
+
+@pytest.mark.parametrize("threads", [False, True])
+def test_handles_side_by_side_give_each_ones_results(threads):
+    """Three handles on one device, their passes overlapping (one thread that takes them in turn and waits for none, or a thread
+    for each): parameters, momentum and losses are, bit for bit, those of each handle working alone.  One handle also
+    evaluates in between, one uses the two-call form of the step."""
+    from concurrent.futures import ThreadPoolExecutor
+    from paper_1412_2302_b200 import alexnet as A
+    B, steps = 8, 150
+
+    def batch(k, step):
+        gen = torch.Generator().manual_seed(1000 * k + step)
+        return torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen).pin_memory(), torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen).pin_memory()
+
+    data = [[batch(k, s) for s in range(3)] for k in range(3)]
+
+    def new(k):
+        return A.AlexNet(batch=B, seed=BASE + 40 + k, init_std=0.01, flags=A.FLAG_FUSED_FC_UPDATE, mean_image=synth.mean_image(BASE)), torch.zeros(steps).pin_memory(), []
+
+    def one(k, state, step):
+        net, loss, seen = state
+        net.load_batch_async(0, *data[k][step % 3], step)
+        if k == 1:
+            net.forward_backward(0)
+            net.apply_update(0, 1.0)
+        else:
+            net.train_step(0)
+        net.loss_async(0, loss[step:step + 1])
+        if k == 2 and step % 5 == 4:
+            seen.append(net.eval_batch(0, *data[k][0]))
+
+    def result(state):
+        net, loss, seen = state
+        net.sync()
+        return [t.cpu().numpy() for t in net.param_views(0)[:2]] + [loss.numpy().copy(), np.array(seen)]
+
+    want = []
+    for k in range(3):
+        s = new(k)
+        for step in range(steps):
+            one(k, s, step)
+        want.append(result(s))
+        s[0].close()
+    states = [new(k) for k in range(3)]
+    if threads:
+        def work(k):
+            torch.cuda.set_device(0)
+            for step in range(steps):
+                one(k, states[k], step)
+        with ThreadPoolExecutor(3) as pool:
+            list(pool.map(work, range(3)))
+    else:
+        for step in range(steps):
+            for k in range(3):
+                one(k, states[k], step)
+    for k in range(3):
+        for a, b in zip(result(states[k]), want[k]):
+            assert np.array_equal(a, b), k
+        states[k][0].close()
