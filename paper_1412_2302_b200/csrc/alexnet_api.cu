@@ -1437,7 +1437,7 @@ const void* const kKernels[] = {
     (const void*)LRN_POOL_FWD_1(false), (const void*)LRN_POOL_FWD_1(true), (const void*)LRN_POOL_FWD_2(false), (const void*)LRN_POOL_FWD_2(true),
     (const void*)POOL_LRN_BWD_1(false), (const void*)POOL_LRN_BWD_1(true), (const void*)POOL_LRN_BWD_2(false), (const void*)POOL_LRN_BWD_2(true),
     (const void*)kn::fc_reduce_fwd_kernel, (const void*)kn::fc_reduce_bwd_kernel, (const void*)kn::wgrad_reduce_kernel,
-    (const void*)kn::colsum_kernel, (const void*)kn::colsum_final_kernel, (const void*)kn::colsum_scalar_kernel, (const void*)kn::bias_grad_kernel<256>, (const void*)kn::bias_grad_kernel<1024>,
+    (const void*)kn::colsum_kernel, (const void*)kn::colsum_final_kernel, (const void*)kn::colsum_scalar_kernel, (const void*)kn::bias_grad_kernel,
     (const void*)kn::softmax_xent_kernel, (const void*)kn::mean_kernel, (const void*)kn::fc8_softmax_xent_kernel<false>,
     (const void*)kn::fc8_softmax_xent_kernel<true>, (const void*)kn::store_result_kernel, (const void*)kn::store_value_kernel,
     (const void*)kn::sgd_update_kernel, (const void*)kn::sgd_update_conv_kernel, (const void*)kn::replica_average_kernel,
@@ -2142,17 +2142,19 @@ extern "C" int alexnet_bias_grad_noalloc(const void* dev_dy, int64_t rows, int32
         g_noalloc_cnt[dev] = q;
         g_noalloc_ptr[dev] = p;
     }
-    // row splits: one block of 1024 threads per SM in total, or four of 256 for a small call, at least 64 rows each
-    const int groups = (channels + 63) / 64;
-    const bool small = rows * channels < kn::kBgSmall;
-    int64_t splits = std::min<int64_t>((small ? 4 : 1) * std::min(g_noalloc_sms[dev], kSms) / groups, rows / 64);
+    // row splits: four blocks per SM in total, of at least 64 rows each; one or two groups of columns take blocks of 512 rows before
+    // a group has more splits than the device SMs, whose last block would need a second round of loads (25088 x 96 6.2 -> 5.25 us,
+    // 50000 x 96 6.4 -> 6.1; with never more than 148 splits 200000 x 96 takes 13.0 us instead of 11.6, and 100000 x 192 8.6 instead of 7.8)
+    const int groups = (channels + 63) / 64, sms = std::min(g_noalloc_sms[dev], kSms);
+    int64_t splits = std::min<int64_t>(4 * sms / groups, rows / 64);
+    if (groups <= 2) splits = std::min(splits, std::max<int64_t>(sms, rows / 512));
     splits = std::max<int64_t>(splits, 1);
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     e = cudaStreamIsCapturing((cudaStream_t)stream, &capture);
     if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone)
         e = cudaMemsetAsync(g_noalloc_cnt[dev], 0, groups * sizeof(unsigned long long), (cudaStream_t)stream);
     if (e != cudaSuccess) { cudaGetLastError(); put_err(err, err_len, cudaGetErrorString(e)); return ALEXNET_ERR_CUDA; }
-    launch_k(small ? kn::bias_grad_kernel<256> : kn::bias_grad_kernel<1024>, dim3(groups, (unsigned)splits), small ? 256 : 1024, 0, (cudaStream_t)stream, (const bf16*)dev_dy, (long long)rows, channels,
+    launch_k(kn::bias_grad_kernel, dim3(groups, (unsigned)splits), 256, 0, (cudaStream_t)stream, (const bf16*)dev_dy, (long long)rows, channels,
              g_noalloc_ptr[dev], g_noalloc_cnt[dev], ++g_noalloc_calls, dev_db);
     const std::string refused = take_launch_error();
     e = cudaGetLastError();

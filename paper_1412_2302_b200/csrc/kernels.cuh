@@ -865,18 +865,16 @@ __global__ void colsum_scalar_kernel(const __nv_bfloat16* __restrict__ dy, int r
 // blocks in the low 16 bits of a word whose upper bits are the number of the launch: the first block of a launch sets the
 // word to its number and a count of zero (a maximum: every later block of the launch leaves the count alone), so a launch
 // owes nothing to what an earlier one left there, be it one that overlapped another or one that died.  HBM-bound (L2-bound
-// where dy fits); what it spends beside that is the launch and the tail of the last block.  Hence one block of 1024 threads per SM
-// and not four of 256: a quarter of the partials and of the atomics on a group's word, and one round of loads in the tail.
-// Per call, four blocks of 256 / one of 1024: 25088 x 384 7.33 / 6.26 us, 60000 x 2048 47.4 / 41.1, 8000 x 104 7.0 / 5.5, 3000 x 384 6.3 /
-// 5.6, 3000 x 104 5.05 / 4.95.  Below that the larger block only takes longer to start (1500 x 104 4.3 / 4.9, 700 x 384 4.1 to 4.4 / 4.9),
-// so calls of fewer than 300 thousand elements keep blocks of 256.
-constexpr long long kBgSmall = 300000;
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
-                                                               unsigned long long* __restrict__ counters, unsigned long long launch,
-                                                               float* __restrict__ db) {
+// where dy fits); what it spends beside that is the launch and the tail of the last block, whose loads of up to 160 partials go in one
+// round.  Blocks of 256 threads and 64 registers, four to an SM, fit beside the tensor kernels of a training step, where this
+// call belongs; one block of 1024 per SM waits for an SM to be empty.  Per call alone, 256 / 1024: 25088 x 384 5.97 / 6.27 us (several dy in turn 7.5 /
+// 8.4), 60000 x 2048 40.5 / 40.9, 8000 x 104 5.5 / 5.5; beside a training handle of batch 32: 8000 x 104 23.5 / 38.2, 3000 x 384 24.1 / 37.1,
+// 25088 x 384 34.2 / 38.1, 60000 x 2048 81 / 93, and the step beside them 0.5 to 1% shorter.
+__global__ void __launch_bounds__(256, 4) bias_grad_kernel(const __nv_bfloat16* __restrict__ dy, long long rows, int C, float* __restrict__ partial,
+                                                           unsigned long long* __restrict__ counters, unsigned long long launch,
+                                                           float* __restrict__ db) {
     pdl_sync();
-    constexpr int RL = THREADS / 8, WARPS = THREADS / 32, ZL = THREADS / 16;       // lanes over the rows; over the splits in the tail
+    constexpr int RL = 32, WARPS = 8, ZL = 16;       // lanes over the rows; over the splits in the tail
     __shared__ __align__(16) float red[WARPS][68];
     __shared__ bool last;
     const int tid = threadIdx.x, cc = tid & 7, rl = tid >> 3;
@@ -931,7 +929,7 @@ __global__ void __launch_bounds__(THREADS, 1) bias_grad_kernel(const __nv_bfloat
     __threadfence();
     const int q4 = tid & 15, zl = tid >> 4, cq = blockIdx.x * 64 + 4 * q4;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (cq < C && zl < splits) a = sum_splits<THREADS == 1024 ? 3 : 8>(partial + (size_t)zl * C + cq, (long long)ZL * C, (splits - zl + ZL - 1) / ZL);
+    if (cq < C && zl < splits) a = sum_splits<10>(partial + (size_t)zl * C + cq, (long long)ZL * C, (splits - zl + ZL - 1) / ZL);
     a.x += __shfl_xor_sync(~0u, a.x, 16); a.y += __shfl_xor_sync(~0u, a.y, 16);
     a.z += __shfl_xor_sync(~0u, a.z, 16); a.w += __shfl_xor_sync(~0u, a.w, 16);
     if ((tid & 31) < 16) *(float4*)&red[tid >> 5][4 * q4] = a;

@@ -123,8 +123,10 @@ def test_bias_grad_noalloc_after_calls_that_overlapped():
             assert np.array_equal(out.cpu().numpy().astype(np.float64), host_colsum(t))
 
 
-# around the line between the two block sizes (300 thousand elements), with one split, the most splits, and remainders of the row lanes
-@pytest.mark.parametrize("rows,C", [(1, 8), (65, 4096), (74, 4096), (781, 384), (782, 384), (4687, 64), (4688, 64), (9473, 64), (20011, 72)])
+# one split, the most splits (592 of one column group, 296 of two), two groups around the line from which blocks of 512 rows take more than
+# one split per SM (75776 rows), wide layers of several splits, and remainders of the row lanes
+@pytest.mark.parametrize("rows,C", [(1, 8), (65, 4096), (74, 4096), (781, 384), (782, 384), (4687, 64), (4688, 64), (9473, 64), (20011, 72),
+                                    (75776, 104), (76288, 104), (152001, 128), (303200, 8), (1201, 2432), (1201, 3200), (1201, 4096)])
 def test_bias_grad_noalloc_block_sizes(rows, C):
     from paper_1412_2302_b200 import alexnet as A
     rng = np.random.default_rng(rows + C)
