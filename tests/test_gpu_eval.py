@@ -110,7 +110,8 @@ def test_eval_in_chunks_is_bit_for_bit_the_one_pass(B):
 
 
 def test_eval_images_where_they_are():
-    """Aligned images on the device are read in place, others are copied first, and of pinned images only the crop's rows travel: one result."""
+    """Aligned images on the device are read in place, others are copied first, and of pinned images only the crop's rows travel: one
+    result.  Before each of them another batch, on the device and misaligned, fills the staging buffer, so that rows which did not travel show."""
     from paper_1412_2302_b200 import alexnet as A
     seed, B = synth.BASE_SEED + 34, 3
     net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
@@ -118,13 +119,78 @@ def test_eval_images_where_they_are():
     gen = torch.Generator().manual_seed(B)
     lab = torch.randint(0, 1000, (B,), dtype=torch.int32, generator=gen)
     img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, generator=gen)
-    shifted = torch.zeros(img.numel() + 16, dtype=torch.uint8, device="cuda")
-    odd = shifted[5:5 + img.numel()].view(img.shape)
-    odd.copy_(img)
-    torch.cuda.synchronize()
-    got = [(net.eval_batch(0, im, lab.pin_memory()), net.get_tensor("X0"), net.get_tensor("Z")) for im in (img.cuda(), odd, img.pin_memory(), img)]
+
+    def misaligned(t):
+        odd = torch.zeros(t.numel() + 16, dtype=torch.uint8, device="cuda")[5:5 + t.numel()].view(t.shape)
+        odd.copy_(t)
+        return odd
+
+    got = []
+    for im in (img.cuda(), misaligned(img), img.pin_memory(), img):
+        other = misaligned(torch.randint(0, 256, img.shape, dtype=torch.uint8, generator=gen))
+        torch.cuda.synchronize()
+        net.eval_batch(0, other, lab.pin_memory())
+        got.append((net.eval_batch(0, im, lab.pin_memory()), net.get_tensor("X0"), net.get_tensor("Z")))
     for g in got[1:]:
         assert g[0] == got[0][0] and np.array_equal(g[1], got[0][1]) and np.array_equal(g[2], got[0][2])
+    net.close()
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 5])
+def test_eval_of_few_images_with_new_labels_every_call(B):
+    """Labels at ranks 0, 4 and 5 of the GPU's own logits, other ones every call and in every kind of memory: the counts are those of the labels of
+    the call, the loss is the mean cross-entropy of its logits (one image takes a way of its own out of the softmax kernel)."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed = synth.BASE_SEED + 36
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    net.set_params(synth.init_params(seed, variance_preserving=True, bias=0.1))
+    img = torch.from_numpy(synth.images(seed, 0, 0, B)).pin_memory()
+    net.eval_batch(0, img, torch.zeros(B, dtype=torch.int32).pin_memory())
+    z = net.get_tensor("Z").reshape(B, 1000)
+    order = np.argsort(-z, axis=1, kind="stable")
+    z64 = z.astype(np.float64)
+    lse = np.log(np.exp(z64 - z64.max(1, keepdims=True)).sum(1)) + z64.max(1)
+    for call, ranks in enumerate(([0], [4], [5], [0, 4], [5, 0], [4, 5], [999, 0], [0])):
+        rank = np.array([ranks[i % len(ranks)] for i in range(B)])
+        lab = torch.from_numpy(order[np.arange(B), rank].astype(np.int32))
+        lab = lab.pin_memory() if call % 3 == 0 else lab.cuda() if call % 3 == 1 else lab
+        torch.cuda.synchronize()
+        t1, t5, loss = net.eval_batch(0, img, lab)
+        assert (t1, t5) == (int((rank < 1).sum()), int((rank < 5).sum())), (ranks, t1, t5)
+        want = (lse - z64[np.arange(B), order[np.arange(B), rank]]).mean()
+        # 32-bit exponentials and sums of 1000 terms: some 1e-6 of the logits' size
+        assert abs(loss - want) < 1e-5 * max(1.0, np.abs(z64).max()), (ranks, loss, want)
+        assert np.array_equal(net.get_tensor("Z").reshape(B, 1000), z)
+    net.close()
+
+
+@pytest.mark.parametrize("B", [3, 128, 129, 256, 300, 512, 520])
+def test_eval_fc_layers_against_their_inputs(B):
+    """fc6 and fc7 of an evaluation against the inputs that the GPU gave them: ReLU, and the expectation of the dropout mask, whether the reduction
+    over the k splits runs inside the GEMM (one or several row tiles, 4, 2 or no splits) or, beyond 512 images, as a launch of its own."""
+    from paper_1412_2302_b200 import alexnet as A
+    seed = synth.BASE_SEED + 37
+    net = A.AlexNet(batch=B, seed=seed, mean_image=synth.mean_image(seed))
+    w = synth.init_params(seed, variance_preserving=True, bias=0.1)
+    off, _ = O.param_offsets()
+    rng = np.random.default_rng(B)
+    for k in ("fc6.W", "fc7.W"):
+        o, n, _ = off[k]
+        w[o:o + n] = rng.integers(-16, 17, size=n) / 1024.0      # exact in bf16
+    net.set_params(w)
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    img = torch.randint(0, 256, (B, 256, 256, 3), dtype=torch.uint8, device="cuda", generator=gen)
+    lab = torch.zeros(B, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    net.eval_batch(0, img, lab)
+    P = O.unpack(w)
+    for name, src, dst in (("fc6", "P5", "F6"), ("fc7", "F6", "F7")):
+        K, N = O.FC[name]
+        W, b = (torch.from_numpy(np.ascontiguousarray(P[name + k])).cuda().double() for k in (".W", ".b"))
+        x = torch.from_numpy(net.get_tensor(src)).cuda().double().reshape(B, K)
+        ref = 0.5 * torch.relu(x @ W.reshape(N, K).T + b)
+        # one rounding to bf16: at most 2^-9 of each value, and 32-bit sums of 9216 terms far below that
+        assert rel(net.get_tensor(dst), ref.cpu().numpy()) < 2.0 ** -9 + 1e-5, name
     net.close()
 
 

@@ -167,8 +167,9 @@ def test_fc_forward_with_dropout(net, params, name, tin, tout, tm, stream):
 
 # several row tiles, each finished by the CTAs of its k splits: 2 splits up to batch 256, none up to 512 (a ragged last tile, rows
 # of one, a full one), and beyond that the reduction as a launch of its own
+@pytest.mark.parametrize("name,tin,tout,tm,stream", [("fc6", "P5", "F6", "M6", 2), ("fc7", "F6", "F7", "M7", 3)])
 @pytest.mark.parametrize("batch", [129, 200, 256, 257, 512, 520])
-def test_fc_forward_over_batches(batch):
+def test_fc_forward_over_batches(batch, name, tin, tout, tm, stream):
     import torch
     from paper_1412_2302_b200.alexnet import AlexNet
     n = AlexNet(batch=batch, seed=SEED, mean_image=synth.mean_image(SEED))
@@ -176,17 +177,18 @@ def test_fc_forward_over_batches(batch):
     w = (rng.integers(-64, 65, size=n.param_count) / 256.0).astype(np.float32)
     n.set_params(w, 0, 0)
     P = O.unpack(w)
-    K, N = O.FC["fc7"]
+    K, N = O.FC[name]
     x = synth.bf16_grid(SEED, 33, (batch, K), -1, 1)
-    n.set_tensor("F6", x)
-    n.run_op("FC7_FWD")
+    n.set_tensor(tin, x)
+    n.run_op(name.upper() + "_FWD")
     n.sync()
-    W, b = (torch.from_numpy(np.ascontiguousarray(P[k])).cuda().double() for k in ("fc7.W", "fc7.b"))
+    W, b = (torch.from_numpy(np.ascontiguousarray(P[name + k])).cuda().double() for k in (".W", ".b"))
     ref = (torch.from_numpy(np.ascontiguousarray(x)).cuda().double() @ W.reshape(N, K).T + b).cpu().numpy()
-    keep = O.dropout_mask(SEED, 3, 0, 0, batch, N, 0.5)
-    assert np.array_equal(n.get_tensor("M7").reshape(batch, N).astype(np.uint8), keep)
+    keep = O.dropout_mask(SEED, stream, 0, 0, batch, N, 0.5)
+    assert np.array_equal(n.get_tensor(tm).reshape(batch, N).astype(np.uint8), keep)
     # one rounding to bf16: at most 2^-9 of each value
-    assert rel(n.get_tensor("F7"), np.maximum(ref, 0) * keep) < 2.0 ** -9
+    assert rel(n.get_tensor(tout), np.maximum(ref, 0) * keep) < 2.0 ** -9
+    n.close()
 
 
 FCB = [("fc6", "DF6", "DP5", None), ("fc7", "DF7", "DF6", "F6"), ("fc8", "DZ", "DF7", "F7")]
