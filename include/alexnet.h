@@ -161,9 +161,10 @@ int alexnet_loss_async(alexnet_t* h, int replica, float* loss_out);
  * validation errors ("Experiments": top-1 and top-5 error): forward pass only,
  * on the centre 227 x 227 crop without flip, with the dropout masks replaced by
  * their expectation (outputs of fc6 / fc7 times 1 - p, unless training uses
- * inverted dropout).  Copies images [B][256][256][3] uint8 and labels [B] int32
- * (pinned host or device memory) like load_batch_async, runs on both streams
- * and waits for the result.  A sample counts for top-k when fewer than k classes
+ * inverted dropout).  Takes images [B][256][256][3] uint8 and labels [B] int32
+ * (pinned host or device memory; what lies in this GPU's memory at a 16-byte
+ * boundary is read where it is, of pinned images only the rows of the crop are
+ * copied), runs on both streams and waits for the result.  A sample counts for top-k when fewer than k classes
  * rank before its label (greater logit, or equal logit and smaller index).
  *   host_top1, host_top5  number of samples of the batch in the top 1 / top 5 (may be NULL)
  *   host_loss             mean cross-entropy of the batch (may be NULL)

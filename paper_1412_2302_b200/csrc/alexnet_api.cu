@@ -29,8 +29,9 @@ void note_launch(cudaError_t e, const void* kernel) {
 }  // namespace
 
 // Every kernel is launched with programmatic stream serialization: its blocks may become resident while the kernel
-// before it in the stream drains, and run their set-up; each kernel waits (griddepcontrol.wait) before it touches
-// global memory, so the data dependencies of the stream order are kept.
+// before it in the stream drains, and run their set-up; each kernel waits (griddepcontrol.wait) before it touches global memory
+// that a kernel before it in its pass may still be writing, so the data dependencies of the stream order are kept.  (What is read
+// before the wait - weights by conv_kernel, labels and a bias by fc8_softmax_xent_kernel - stands behind lrn_pool_fwd_kernel.)
 template <typename... KArgs, typename... Args>
 void launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t lc{};
@@ -154,16 +155,16 @@ struct Plan { tc::GemmParams p; tc::ConvParams c; tc::WgradParams w; tc::FcUpdPa
 // that run beside them: fc_update_kernel reaches most of the HBM rate on this many SMs (see there), and a chain
 // kernel whose grid fits beside it neither waits for it nor leaves CTAs of a second wave behind.
 // Up to batch 16 the chain is short, the updates are what a step waits for, and they get 72.  One handle alone, 64 / 72 / 80 SMs: batch 1 425 /
-// 410 / 402 us, 4 449 / 426 / 437, 8 459 / 446 / 442, 16 489 / 477 / 481, 32 539 / 533 / 537; three handles taking turns, which fill one another's
-// gaps: 4 340 / 346 / 352, 8 374 / 376 / 377, 16 404 / 407 / 413.  At batch 128 (64 / 80): 976 / 1011.
+// 410 / 402 us, 4 449 / 426 / 437, 8 459 / 446 / 442, 16 489 / 477 / 481, 32 539 / 533 / 537.  (Three handles taking turns fill one another's
+// gaps: 4 340 / 346 / 352, 8 374 / 376 / 377, 16 404 / 407 / 413; the line is drawn for one.)  At batch 128 (64 / 80): 976 / 1011.
 inline int fc_upd_ctas(int B) { return B <= 16 ? 72 : 64; }
 // Conv weight gradients of at most this many 128-row steps run with one CTA per tile, which takes all row splits in turn
 // (WgradParams::solo).  Below about batch 64 these kernels are not the longest branch, and a wave of CTAs of a few steps each costs
 // more than it saves: each takes a whole SM from the data gradients and the FC updates beside it for its set-up and epilogue,
-// and the update adds its partials (64 MB of them at batch 8).  Steps with three handles taking turns, no solo / 30 / 64 / 110 / 220
-// steps: batch 4 390 / 353 / 353 / 351 / 351 us, 8 414 / 386 / 381 / 381 / 375, 16 441 / 416 / 417 / 416 / 415, 32 512 / 512 / 490 / 489 /
-// 487, 64 687 / 693 / 692 / 677 / 677; one handle alone 457 / 476 / 477 / 472 / 473, 466 / 467 / 467 / 468 / 521, 495 / 494 / 495 / 496 /
-// 496, 552 / 553 / 545 / 545 / 564, 720 / 719 / 719 / 715 / 715: at 220 steps conv1, the last kernel of the pass, takes too long.
+// and the update adds its partials (64 MB of them at batch 8).  Steps of one handle, without / with 110 steps: batch 1 422.7 / 410.7 us, 2
+// 422.5 / 417.5, 4 433.9 / 429.7, 8 447.3 / 449.2, 12 467 / 459, 16 486 / 478.5, 32 545.5 / 538.8, 48 639 / 615.5, 64 714 / 707.5; three handles taking turns 4 390 /
+// 351, 8 414 / 381, 16 441 / 416, 32 512 / 489, 64 687 / 677.  With 220 steps one handle of batch 8 takes 521 instead of 468: conv1,
+// the last kernel of the pass, then has three CTAs for 204 steps.
 constexpr int kWgSoloSteps = 110;
 
 struct Tensor {  // description of one exportable device tensor
@@ -814,7 +815,8 @@ int build_plans(alexnet* h, int r) {
 // copied (3.2 us per image: the 227 rows of the crop).  What is left behind the last copy is one chunk's time and the FC layers.  A
 // chunk's dependent launches cost a fixed time and small grids fill the machine badly, so chunks below about 70 images take
 // longer than the copy they should hide behind and the delay adds up from chunk to chunk, while two chunks can be smaller:
-// only the first has to keep up, and it is the smaller one, so that it ends when the second has arrived.
+// only the first has to keep up, and it is the smaller one, so that it ends when the second has arrived (chunk_begin: a line fitted to
+// the best cut at 68, 100 and 191 images, at this rate of copying).
 // Measured, 1 / 2 chunks: 64 images 464 / 484 us, 72 512 / 490, 100 656 / 593 (two equal ones: 616); 2 / 3: 192 961 / 949, 240 1150 / 1089;
 // 3 / 4: 256 1141 / 1186, 300 1344 / 1337, 320 - / 1376; 5 / 6 / 7: 512 2061 / 2015 / 2100.
 constexpr int kEvalTwoChunks = 68, kEvalThreeChunks = 192, kEvalChunk = 75;

@@ -407,8 +407,9 @@ __global__ void __launch_bounds__((WI + 1) / 2 * CV, MINB) lrn_pool_fwd_kernel(c
                                                                                uint8_t* __restrict__ arg, int opr, int Hpi, int Wpi, int Hpo,
                                                                                int Wpo, float alpha, float beta, float k) {
     // Waits first and lets the next launch start afterwards, unlike every other kernel: when a block of the next kernel runs, conv1
-    // (the kernel before this one) has completed, and with it whatever wrote the weights before the pass.  The
-    // convolution and FC kernels behind this one rely on that when they load weights before their own wait.
+    // (the kernel before this one) has completed, and with it whatever wrote weights and biases before the pass, and in an
+    // evaluation the preprocessing kernel, which brings the labels.  The convolution and FC kernels behind this one rely on that when
+    // they load weights before their own wait, and fc8_softmax_xent_kernel when it loads labels and its bias.
     // (Nothing is lost: batch 8 and 128 and an evaluation of one image take what they took with the trigger first.)
     pdl_wait();
     pdl_trigger();
@@ -1002,7 +1003,9 @@ __global__ void __launch_bounds__(256) fc8_softmax_xent_kernel(const float* __re
                                                                int32_t* __restrict__ counts, const int* __restrict__ status,
                                                                HostResult* host_out, uint32_t seq) {
     pdl_trigger();
-    // the bias and the labels were written before the pass began: fetched while the predecessor runs
+    // the bias and the labels are fetched while the predecessor runs: whatever wrote them (the update of the step before; the loader,
+    // or in an evaluation the preprocessing kernel of this very stream and pass) has completed, because lrn_pool_fwd_kernel, between it
+    // and this kernel, lets no later launch start before it has itself waited
     const int lab = labels[blockIdx.x];
     float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if ((N & 3) == 0 && 4 * (int)threadIdx.x < N) b4 = __ldg((const float4*)bias + threadIdx.x);

@@ -23,7 +23,8 @@
 // rows of each CTA); fc_update_kernel forms the FC weight gradients and applies the momentum update to the weights in place.
 // All kernels are launched with programmatic stream serialization: they let the next launch of the stream start early
 // (griddepcontrol.launch_dependents first thing) and wait for their predecessors (griddepcontrol.wait) after their
-// barriers, tensor memory and descriptors are set up and before they touch global memory.
+// barriers, tensor memory and descriptors are set up and before they touch global memory (conv_kernel's weights excepted, where
+// the launch says so: ConvParams::early_b).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
